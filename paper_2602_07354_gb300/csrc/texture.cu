@@ -23,7 +23,10 @@ namespace elas {
 
 namespace {
 
-constexpr int kTexThreads = 256;
+// one warp per block: a grain costs about 100 FP64 operations (trigonometric functions), so the grains
+// of one microstructure (thousands) are spread over all SMs' FP64 pipes (2,048 grains: 8 blocks of 256
+// 10.9 us, 64 of 32: 7.6 us)
+constexpr int kTexThreads = 32;
 
 // lognormal parameters (log-space mean m, spread s) of a variate with mean mu and deviation sd
 void lognormal_params(double mu, double sd, double* m, double* s) {
