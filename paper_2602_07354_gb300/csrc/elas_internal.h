@@ -390,8 +390,9 @@ inline void hot_weights(double s, int r, double* w) {
   }
   for (int x = -r; x <= r; ++x) w[x + r] /= sum;
 }
-// smooth (device N) written; best2[0]: bits of the largest hotspot value, best2[1]: its lowest
-// voxel id (~0 if there is no hotspot); solid_only: pore neighbours do not compete.  Synchronises s.
+// smooth (device N) written; best2 (device, 6 kMaxParts values, the rest scratch) [0]: bits of the
+// largest hotspot value, [1]: its lowest voxel id (~0 if there is no hotspot); solid_only: pore
+// neighbours do not compete.
 cudaError_t launch_hotspot(const Geo& g, const int32_t* phase, const double* vm, double s_kernel, bool solid_only,
                            double* smooth, unsigned long long* best2, int sm_count, cudaStream_t s);
 

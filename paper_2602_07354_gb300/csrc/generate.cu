@@ -407,7 +407,8 @@ __global__ void __launch_bounds__(kGenThreads)
 // than 1e-4 and the sum by less than 4e-4 of max(1, sum): only voxels within 1e-3 of the surface
 // evaluate the FP64 sum.  A component near half the cell, where the minimum image may go either
 // way, is longer than amax, so its sum is in that band or above it for both images.
-// Bound: FP64 arithmetic, one SM per pore, before (183 pores of r <= 6: 71 us with the scaled frame still divided in FP64, 12.7 us now).
+// Bound: FP64 arithmetic before (183 pores of r <= 6: 71 us with R / a still divided in FP64 by every
+// thread); 12.7 us now, issue-bound.
 __global__ void k_stamp(int nx, int ny, int nz, const double* __restrict__ pores, int32_t* __restrict__ phase) {
   const double* P = pores + (size_t)kPoreDoubles * blockIdx.x;
   __shared__ float sP[kPoreDoubles], s_first[3];

@@ -5,8 +5,12 @@
 // uses the largest of them.  The sums run over dz, dy, dx
 // with the weight (w[dz] * w[dy]) * w[dx], every operation explicitly rounded, so the field is
 // bitwise the same as a plain loop in that order; the maximum (and the lowest voxel id holding it)
-// are formed with order-independent atomics.
+// does not depend on the order in which blocks finish.
 #include <cuda_runtime.h>
+
+#include <algorithm>
+#include <climits>
+#include <cstdlib>
 
 #include "elas_internal.h"
 
@@ -14,65 +18,367 @@ namespace elas {
 
 namespace {
 
-constexpr int kHotThreads = 256;
+constexpr int kHotThreads = 512;
 
+// Weights by class (|dz|, |dy|, |dx|), rounded as (w[dz] * w[dy]) * w[dx]; the sum of all weights in
+// the order of the taps and its reciprocal.
 struct Weights {
-  double w[2 * kHotMaxRadius + 1];
+  double w[(kHotMaxRadius + 1) * (kHotMaxRadius + 1) * (kHotMaxRadius + 1)];
+  double full, inv_full;
 };
 
-__device__ __forceinline__ int wrap1(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
+__device__ __forceinline__ int wrapn(int i, int n) {
+  i %= n;
+  return i < 0 ? i + n : i;
+}
 
-__global__ void k_smooth(int nx, int ny, int nz, const int32_t* __restrict__ phase, const double* __restrict__ vm,
-                         Weights W, int r, double* __restrict__ smooth) {
-  const long long N = (long long)nx * ny * nz;
-  for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < N; v += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(v % nx), j = (int)((v / nx) % ny), k = (int)(v / ((long long)nx * ny));
-    double num = 0.0, den = 0.0;
-    for (int dz = -r; dz <= r; ++dz) {
-      const long long kz = wrap1(k + dz, nz);
-      for (int dy = -r; dy <= r; ++dy) {
-        const long long jy = wrap1(j + dy, ny);
-        const double wzy = __dmul_rn(W.w[dz + r], W.w[dy + r]);
-        for (int dx = -r; dx <= r; ++dx) {
-          const long long u = wrap1(i + dx, nx) + nx * (jy + ny * kz);
-          const double wt = __dmul_rn(wzy, W.w[dx + r]);
-          if (phase[u] >= 0) {
-            num = __dadd_rn(num, __dmul_rn(wt, vm[u]));
-            den = __dadd_rn(den, wt);
+// One item = a tile of tx x ty voxel columns and zc layers; thread t owns column (t % tx, t / tx) and
+// marches z.  Plane p adds its taps to the 2R + 1 outputs it reaches (dz = p - z rises with p, so
+// every output meets its taps in the order dz, dy, dx); a pore's tap adds +0, which changes nothing.
+//
+// Bound: the FP64 pipe (1.66 operations per SM and clock).  The operations that the rounding order
+// leaves are 27 sums a voxel (R = 1); a plain loop spent 4 per tap (two for the weight and its sum).
+// Here a voxel's products with the 8 weight classes are formed once and shared through shared memory
+// (9.6 a voxel with the tile's halo, instead of 27), the weight sum is the constant full sum unless
+// the window holds a pore, and the division by that constant is a multiplication by its correctly
+// rounded reciprocal and one residual correction (Markstein 1990: correctly rounded).  200^3, s = 0.4:
+// 2.05 -> 0.84 ms,
+// FP64 pipe 82% busy.  For R >= 2 the classes outgrow shared memory: one product per tap and |dz|.
+template <int R>
+__global__ void __launch_bounds__(kHotThreads, R == 1 ? 2 : 1)
+    k_smooth(int nx, int ny, int nz, int tx, int ty, int zc, const int32_t* __restrict__ phase,
+             const double* __restrict__ vm, const __grid_constant__ Weights W, double* __restrict__ smooth) {
+  constexpr int D = 2 * R + 1, C = R + 1, NQ = R == 1 ? 8 : 1;
+  constexpr int kPos = 3;  // staged positions per thread
+  extern __shared__ __align__(16) unsigned char hot_smem[];
+  const int t = threadIdx.x, wx = tx + 2 * R, wy = ty + 2 * R, np = wx * wy;
+  double* const val = reinterpret_cast<double*>(hot_smem);            // [2][NQ][np]
+  unsigned char* const sol = reinterpret_cast<unsigned char*>(val + 2 * NQ * np);  // [2][np]
+  const int bx = (nx + tx - 1) / tx, by = (ny + ty - 1) / ty, bz = (nz + zc - 1) / zc;
+  const long long plane = (long long)nx * ny;
+  const int i = t % tx, j = t / tx;
+  const bool own = j < ty;
+  for (long long item = blockIdx.x; item < (long long)bx * by * bz; item += gridDim.x) {
+    const int i0 = (int)(item % bx) * tx, j0 = (int)((item / bx) % by) * ty, z0 = (int)(item / ((long long)bx * by)) * zc;
+    const int z1 = min(z0 + zc, nz);
+    int off[kPos];
+#pragma unroll
+    for (int q = 0; q < kPos; ++q) {
+      const int s = t + q * kHotThreads;
+      off[q] = s < np ? wrapn(j0 - R + s / wx, ny) * nx + wrapn(i0 - R + s % wx, nx) : -1;
+    }
+    double pv[kPos];
+    int pp[kPos];
+    auto fetch = [&](int p) {
+      const long long base = wrapn(p, nz) * plane;
+#pragma unroll
+      for (int q = 0; q < kPos; ++q)
+        if (off[q] >= 0) {
+          pv[q] = vm[base + off[q]];
+          pp[q] = phase[base + off[q]];
+        }
+    };
+    double acc[D];
+    unsigned mask[D];  // solid taps of the planes met so far, oldest first (R = 1: 9 bits a plane)
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      acc[d] = 0.0;
+      mask[d] = 0;
+    }
+    bool whole[D] = {};  // plane without a pore in the window
+    const bool valid = own && i0 + i < nx && j0 + j < ny;
+    fetch(z0 - R);
+    for (int p = z0 - R; p < z1 + R; ++p) {
+      const int b = (p - z0 + R) & 1;
+      double* const v = val + b * NQ * np;
+      unsigned char* const so = sol + b * np;
+#pragma unroll
+      for (int q = 0; q < kPos; ++q)
+        if (off[q] >= 0) {
+          const int s = t + q * kHotThreads;
+          const bool solid = pp[q] >= 0;
+          so[s] = solid;
+          if constexpr (R == 1) {
+#pragma unroll
+            for (int c = 0; c < NQ; ++c) v[c * np + s] = solid ? __dmul_rn(W.w[c], pv[q]) : 0.0;
+          } else {
+            v[s] = solid ? pv[q] : 0.0;
           }
         }
+      if (p + 1 < z1 + R) fetch(p + 1);
+      __syncthreads();  // (the other buffer's readers have passed the last one)
+      if (valid) {
+        bool all = true;
+        unsigned m = 0;
+        if constexpr (R == 1) {
+          // (the planes beside the item's layers reach only one of the three outputs)
+          const bool up = p + 1 < z1, here = p >= z0 && p < z1, down = p > z0;
+#pragma unroll
+          for (int dy = 0; dy < 3; ++dy) {
+            double far[3], near[3];
+#pragma unroll
+            for (int dx = 0; dx < 3; ++dx) {
+              const int s = (j + dy) * wx + i + dx, c = (dy == 1 ? 0 : 2) + (dx == 1 ? 0 : 1);
+              m |= (unsigned)so[s] << (3 * dy + dx);
+              far[dx] = v[(4 + c) * np + s];
+              near[dx] = v[c * np + s];
+            }
+            if (up) {  // output p + 1
+#pragma unroll
+              for (int dx = 0; dx < 3; ++dx) acc[0] = __dadd_rn(acc[0], far[dx]);
+            }
+            if (here) {  // output p
+#pragma unroll
+              for (int dx = 0; dx < 3; ++dx) acc[1] = __dadd_rn(acc[1], near[dx]);
+            }
+            if (down) {  // output p - 1: complete
+#pragma unroll
+              for (int dx = 0; dx < 3; ++dx) acc[2] = __dadd_rn(acc[2], far[dx]);
+            }
+          }
+          all = m == 0x1ff;
+        } else {
+          for (int dy = 0; dy < D; ++dy)
+#pragma unroll
+            for (int dx = 0; dx < D; ++dx) {
+              const int s = (j + dy) * wx + i + dx;
+              const int cy = dy < R ? R - dy : dy - R, cx = dx < R ? R - dx : dx - R;
+              const double x = v[s];
+              all = all && so[s];
+#pragma unroll
+              for (int cz = 0; cz <= R; ++cz) {
+                const double q = __dmul_rn(W.w[(cz * C + cy) * C + cx], x);
+                acc[R - cz] = __dadd_rn(acc[R - cz], q);
+                if (cz) acc[R + cz] = __dadd_rn(acc[R + cz], q);
+              }
+            }
+        }
+#pragma unroll
+        for (int d = 0; d < D - 1; ++d) {
+          whole[d] = whole[d + 1];
+          mask[d] = mask[d + 1];
+        }
+        whole[D - 1] = all;
+        mask[D - 1] = m;
+        const int z = p - R;
+        if (z >= z0) {
+          bool full = true;
+#pragma unroll
+          for (int d = 0; d < D; ++d) full = full && whole[d];
+          const double num = acc[D - 1];
+          const long long n = z * plane + (long long)(j0 + j) * nx + i0 + i;
+          const int e = (__double2hiint(num) >> 20) & 0x7ff;  // exponent field: 2^-930 .. 2^930 passes
+          if (full && e > 93 && e < 1953) {
+            const double q = __dmul_rn(num, W.inv_full);
+            smooth[n] = __fma_rn(__fma_rn(-q, W.full, num), W.inv_full, q);
+          } else {
+            double den = full ? W.full : 0.0;
+            if (!full) {
+              if constexpr (R == 1) {
+#pragma unroll
+                for (int d = 0; d < 27; ++d) {
+                  const int dz = d / 9, dy = (d / 3) % 3, dx = d % 3;
+                  if ((mask[dz] >> (d % 9)) & 1)
+                    den = __dadd_rn(den, W.w[(dz == 1 ? 0 : 4) + (dy == 1 ? 0 : 2) + (dx == 1 ? 0 : 1)]);
+                }
+              } else {
+                for (int dz = -R; dz <= R; ++dz)
+                  for (int dy = -R; dy <= R; ++dy)
+                    for (int dx = -R; dx <= R; ++dx)
+                      if (phase[wrapn(z + dz, nz) * plane + (long long)wrapn(j0 + j + dy, ny) * nx + wrapn(i0 + i + dx, nx)] >= 0)
+                        den = __dadd_rn(den, W.w[(abs(dz) * C + abs(dy)) * C + abs(dx)]);
+              }
+            }
+            smooth[n] = den > 0.0 ? __ddiv_rn(num, den) : 0.0;
+          }
+        }
+#pragma unroll
+        for (int d = D - 1; d > 0; --d) acc[d] = acc[d - 1];
+        acc[0] = 0.0;
       }
     }
-    smooth[v] = den > 0.0 ? __ddiv_rn(num, den) : 0.0;
+    __syncthreads();  // the next item stages into the buffers read last
   }
 }
 
-// pass 0: the largest hotspot value (bits of a non-negative double order like the values);
-// pass 1: the lowest voxel id holding it
-__global__ void k_hotspot(int nx, int ny, int nz, const int32_t* __restrict__ phase, const double* __restrict__ smooth,
-                          bool solid_only, int pass, unsigned long long* __restrict__ best) {
-  const long long N = (long long)nx * ny * nz;
-  for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < N; v += (long long)gridDim.x * blockDim.x) {
-    if (phase[v] < 0) continue;
-    const int i = (int)(v % nx), j = (int)((v / nx) % ny), k = (int)(v / ((long long)nx * ny));
-    const double s = smooth[v];
-    bool is_max = true;
-    for (int dz = -1; dz <= 1 && is_max; ++dz)
-      for (int dy = -1; dy <= 1 && is_max; ++dy)
-        for (int dx = -1; dx <= 1; ++dx) {
-          const long long u = wrap1(i + dx, nx) + nx * (wrap1(j + dy, ny) + (long long)ny * wrap1(k + dz, nz));
-          if (smooth[u] > s && !(solid_only && phase[u] < 0)) {
-            is_max = false;
-            break;
+// Order-preserving integer of a double (equal zeros); NaN, which exceeds nothing, below all others.
+__device__ __forceinline__ long long order_key(double x) {
+  const long long b = __double_as_longlong(x);
+  if ((b & LLONG_MAX) > 0x7ff0000000000000ll) return LLONG_MIN;
+  return b >= 0 ? b : (b == LLONG_MIN ? 0 : b ^ LLONG_MAX);
+}
+
+__device__ __forceinline__ void better(unsigned long long& bits, unsigned long long& vox, unsigned long long b,
+                                       unsigned long long v) {
+  if (b > bits || (b == bits && v < vox)) {
+    bits = b;
+    vox = v;
+  }
+}
+
+// The largest hotspot value (as its bits, compared unsigned) and the lowest voxel holding it, in one
+// pass: thread t marches z through its column with the 3 x 3 maxima of three planes, compared as
+// order-preserving integers (26 FP64 comparisons a voxel and pass would be bound by the FP64 pipe:
+// 200^3: two passes 0.84 ms, this one 0.10).  Each block leaves its best in a slot; the last one to finish reduces them.
+__global__ void __launch_bounds__(kHotThreads)
+    k_hotspot(int nx, int ny, int nz, int tx, int ty, int zc, const int32_t* __restrict__ phase,
+              const double* __restrict__ smooth, bool solid_only, unsigned long long* __restrict__ best,
+              unsigned int* __restrict__ ctr, unsigned long long* __restrict__ slots) {
+  constexpr int kPos = 2;
+  extern __shared__ __align__(16) unsigned char hot_smem[];
+  __shared__ unsigned long long rb[kHotThreads / 32], rv[kHotThreads / 32];
+  __shared__ int last;
+  const int t = threadIdx.x, wx = tx + 2, np = wx * (ty + 2);
+  long long* const key = reinterpret_cast<long long*>(hot_smem);                      // [2][np]
+  unsigned char* const sol = reinterpret_cast<unsigned char*>(key + 2 * np);           // [2][np]
+  const int bx = (nx + tx - 1) / tx, by = (ny + ty - 1) / ty, bz = (nz + zc - 1) / zc;
+  const long long plane = (long long)nx * ny;
+  const int i = t % tx, j = t / tx;
+  unsigned long long bits = 0ull, vox = ~0ull;
+  for (long long item = blockIdx.x; item < (long long)bx * by * bz; item += gridDim.x) {
+    const int i0 = (int)(item % bx) * tx, j0 = (int)((item / bx) % by) * ty, z0 = (int)(item / ((long long)bx * by)) * zc;
+    const int z1 = min(z0 + zc, nz);
+    int off[kPos];
+#pragma unroll
+    for (int q = 0; q < kPos; ++q) {
+      const int s = t + q * kHotThreads;
+      off[q] = s < np ? wrapn(j0 - 1 + s / wx, ny) * nx + wrapn(i0 - 1 + s % wx, nx) : -1;
+    }
+    double pv[kPos];
+    int pp[kPos];
+    auto fetch = [&](int p) {
+      const long long base = wrapn(p, nz) * plane;
+#pragma unroll
+      for (int q = 0; q < kPos; ++q)
+        if (off[q] >= 0) {
+          pv[q] = smooth[base + off[q]];
+          pp[q] = phase[base + off[q]];
+        }
+    };
+    const bool valid = j < ty && i0 + i < nx && j0 + j < ny;
+    long long m0 = LLONG_MIN, m1 = LLONG_MIN, self1 = 0;  // plane maxima of p - 2, p - 1; own key of p - 1
+    bool solid1 = false;
+    fetch(z0 - 1);
+    for (int p = z0 - 1; p <= z1; ++p) {
+      const int b = (p - z0 + 1) & 1;
+      long long* const k = key + b * np;
+      unsigned char* const so = sol + b * np;
+#pragma unroll
+      for (int q = 0; q < kPos; ++q)
+        if (off[q] >= 0) {
+          const int s = t + q * kHotThreads;
+          so[s] = pp[q] >= 0;
+          k[s] = solid_only && pp[q] < 0 ? LLONG_MIN : order_key(pv[q]);
+        }
+      if (p < z1) fetch(p + 1);
+      __syncthreads();
+      if (valid) {
+        const int s = j * wx + i;
+        long long m = k[s];
+#pragma unroll
+        for (int q = 1; q < 9; ++q) m = max(m, k[s + (q / 3) * wx + q % 3]);
+        if (p > z0 && solid1) {
+          const long long self = self1 == LLONG_MIN ? LLONG_MAX : self1;  // no neighbour exceeds a NaN
+          if (self >= max(m0, max(m1, m))) {
+            const long long n = (p - 1) * plane + (long long)(j0 + j) * nx + i0 + i;
+            better(bits, vox, (unsigned long long)__double_as_longlong(smooth[n]), (unsigned long long)n);
           }
         }
-    if (!is_max) continue;
-    const unsigned long long bits = (unsigned long long)__double_as_longlong(s);
-    if (pass == 0)
-      atomicMax(&best[0], bits);
-    else if (bits == best[0])
-      atomicMin(&best[1], (unsigned long long)v);
+        m0 = m1;
+        m1 = m;
+        self1 = k[s + wx + 1];
+        solid1 = so[s + wx + 1];
+      }
+    }
+    __syncthreads();
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long b = __shfl_down_sync(0xffffffffu, bits, o), v = __shfl_down_sync(0xffffffffu, vox, o);
+    better(bits, vox, b, v);
+  }
+  if ((t & 31) == 0) {
+    rb[t / 32] = bits;
+    rv[t / 32] = vox;
+  }
+  __syncthreads();
+  if (t == 0) {
+    for (int w = 1; w < kHotThreads / 32; ++w) better(bits, vox, rb[w], rv[w]);
+    slots[2 * blockIdx.x] = bits;
+    slots[2 * blockIdx.x + 1] = vox;
+    __threadfence();
+    last = atomicAdd(ctr, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  bits = 0ull;
+  vox = ~0ull;
+  for (int q = t; q < (int)gridDim.x; q += kHotThreads) better(bits, vox, __ldcg(slots + 2 * q), __ldcg(slots + 2 * q + 1));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long b = __shfl_down_sync(0xffffffffu, bits, o), v = __shfl_down_sync(0xffffffffu, vox, o);
+    better(bits, vox, b, v);
+  }
+  __syncthreads();
+  if ((t & 31) == 0) {
+    rb[t / 32] = bits;
+    rv[t / 32] = vox;
+  }
+  __syncthreads();
+  if (t == 0) {
+    for (int w = 1; w < kHotThreads / 32; ++w) better(bits, vox, rb[w], rv[w]);
+    best[0] = bits;
+    best[1] = vox;
+  }
+}
+
+// Tile of at most kHotThreads columns with the fewest idle threads over the grid (an idle lane costs
+// its warp's FP64 instructions as much as a busy one), then the fewest halo columns; layers per item
+// so that the busiest SM (the SM's blocks share its pipes) has the least work, the item's neighbour
+// planes counted as one layer.  One block per item: the hardware hands them out as SMs free up.
+struct HotTile {
+  int tx, ty, zc, blocks, pos;
+};
+HotTile hot_tile(const Geo& g, int r, int sm_count, int max_pos) {
+  HotTile best{};
+  double cost0 = 1e300;
+  for (int tx = 4; tx <= 64; ++tx) {
+    const int ty = kHotThreads / tx;
+    if ((tx + 2 * r) * (ty + 2 * r) > max_pos) continue;
+    const double cols = (double)((g.nx + tx - 1) / tx) * ((g.ny + ty - 1) / ty);
+    const double cost = cols * (kHotThreads + 0.3 * (tx + 2 * r) * (ty + 2 * r));
+    if (cost < cost0) {
+      cost0 = cost;
+      best.tx = tx;
+      best.ty = ty;
+      best.pos = (tx + 2 * r) * (ty + 2 * r);
+    }
+  }
+  const long long tiles = (long long)((g.nx + best.tx - 1) / best.tx) * ((g.ny + best.ty - 1) / best.ty);
+  double c0 = 1e300;
+  for (int zc = 1; zc <= g.nz && zc <= 256; ++zc) {
+    const long long items = tiles * ((g.nz + zc - 1) / zc);
+    const double c = (double)((items + sm_count - 1) / sm_count) * (zc + 1.0 * r);
+    if (c < c0 && items < (1 << 30)) {
+      c0 = c;
+      best.zc = zc;
+      best.blocks = (int)items;
+    }
+  }
+  return best;
+}
+
+template <int R>
+cudaError_t launch_smooth(const Geo& g, const int32_t* phase, const double* vm, const Weights& W, double* smooth,
+                          int sm_count, cudaStream_t s) {
+  constexpr int NQ = R == 1 ? 8 : 1;
+  const HotTile h = hot_tile(g, R, sm_count, R == 1 ? 704 : 3 * kHotThreads);
+  const size_t smem = (size_t)h.pos * 2 * (NQ * sizeof(double) + 1);
+  constexpr int most = R == 1 ? 2 * 704 * (8 * NQ + 1) : 2 * 3 * kHotThreads * (8 * NQ + 1);
+  cudaError_t e = cudaFuncSetAttribute(k_smooth<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (e != cudaSuccess) return e;
+  k_smooth<R><<<h.blocks, kHotThreads, smem, s>>>(g.nx, g.ny, g.nz, h.tx, h.ty, h.zc, phase, vm, W, smooth);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -80,19 +386,29 @@ __global__ void k_hotspot(int nx, int ny, int nz, const int32_t* __restrict__ ph
 cudaError_t launch_hotspot(const Geo& g, const int32_t* phase, const double* vm, double s_kernel, bool solid_only,
                            double* smooth, unsigned long long* best2, int sm_count, cudaStream_t s) {
   const int r = hot_radius(s_kernel);
+  double w[2 * kHotMaxRadius + 1];
+  hot_weights(s_kernel, r, w);
   Weights W{};
-  hot_weights(s_kernel, r, W.w);
-  const long long blocks = std::min<long long>((g.N + kHotThreads - 1) / kHotThreads, (long long)sm_count * 16);
-  k_smooth<<<(int)blocks, kHotThreads, 0, s>>>(g.nx, g.ny, g.nz, phase, vm, W, r, smooth);
-  cudaError_t e = cudaGetLastError();
-  const unsigned long long init[2] = {0ull, ~0ull};
-  if (e == cudaSuccess) e = cudaMemcpyAsync(best2, init, sizeof init, cudaMemcpyHostToDevice, s);
-  for (int pass = 0; pass < 2 && e == cudaSuccess; ++pass) {
-    k_hotspot<<<(int)blocks, kHotThreads, 0, s>>>(g.nx, g.ny, g.nz, phase, smooth, solid_only, pass, best2);
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // init lives on this stack frame
-  return e;
+  for (int cz = 0; cz <= r; ++cz)
+    for (int cy = 0; cy <= r; ++cy)
+      for (int cx = 0; cx <= r; ++cx) W.w[(cz * (r + 1) + cy) * (r + 1) + cx] = (w[r + cz] * w[r + cy]) * w[r + cx];
+  W.full = 0.0;
+  for (int dz = -r; dz <= r; ++dz)
+    for (int dy = -r; dy <= r; ++dy)
+      for (int dx = -r; dx <= r; ++dx) W.full += W.w[(std::abs(dz) * (r + 1) + std::abs(dy)) * (r + 1) + std::abs(dx)];
+  W.inv_full = 1.0 / W.full;
+  cudaError_t e = r == 1   ? launch_smooth<1>(g, phase, vm, W, smooth, sm_count, s)
+                  : r == 2 ? launch_smooth<2>(g, phase, vm, W, smooth, sm_count, s)
+                  : r == 3 ? launch_smooth<3>(g, phase, vm, W, smooth, sm_count, s)
+                           : launch_smooth<4>(g, phase, vm, W, smooth, sm_count, s);
+  // best2: the result (2 values), the arrival counter, and the blocks' slots
+  unsigned int* ctr = reinterpret_cast<unsigned int*>(best2 + 2);
+  if (e == cudaSuccess) e = cudaMemsetAsync(ctr, 0, sizeof(unsigned int), s);
+  if (e != cudaSuccess) return e;
+  const HotTile h = hot_tile(g, 1, sm_count, 2 * kHotThreads);
+  k_hotspot<<<std::min(h.blocks, kMaxParts), kHotThreads, (size_t)h.pos * 2 * (sizeof(long long) + 1), s>>>(
+      g.nx, g.ny, g.nz, h.tx, h.ty, h.zc, phase, smooth, solid_only, best2, ctr, best2 + 8);
+  return cudaGetLastError();
 }
 
 }  // namespace elas
