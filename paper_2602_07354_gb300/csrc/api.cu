@@ -719,7 +719,7 @@ int elas_stress(elas_ctx* c, const double* strain, const double* w, double* stre
   }
   DevState* st = c->aux64.d_states;
   ELAS_CUDA(c, launch_stress(c->geo, c->phase, c->cfull, strain, w, stress, von_mises, c->parts_stress, &st->ctr[3],
-                             st->macro, c->sm_count, c->stream));
+                             macro_stress ? st->macro : nullptr, c->sm_count, c->stream));
   if (macro_stress) {
     ELAS_CUDA(c, cudaMemcpyAsync(c->aux64.h_states, st, sizeof(DevState), cudaMemcpyDeviceToHost, c->stream));
     ELAS_CUDA(c, cudaStreamSynchronize(c->stream));

@@ -1,4 +1,4 @@
-// Operator, preconditioner-build, right-hand-side and stress kernels (sm_103a).
+// Operator, preconditioner-build and right-hand-side kernels (sm_103a).
 //
 // Matrix-free product y = A u of ELAS3D-Xtal (arXiv 2602.07354), Sec. 2.1.2 / Algorithm 2
 // step A.  The paper evaluates it node by node as a 27-point stencil with 3x3 blocks gathered
@@ -52,19 +52,6 @@ __device__ double block_sum(double v, double* red) {
     for (int i = 0; i < nw; ++i) r += red[i];
   }
   return r;
-}
-
-// Thread 0 publishes this block's partials, then the last block to arrive sees them all.
-__device__ bool publish_and_arrive(double* parts, const double* vals, int nvals, unsigned int* ctr) {
-  __shared__ int s_last;
-  if (threadIdx.x == 0) {
-    for (int q = 0; q < nvals; ++q) parts[q * kMaxParts + blockIdx.x] = vals[q];
-    __threadfence();
-    const unsigned int t = atomicAdd(ctr, 1u);
-    s_last = (t == gridDim.x - 1);
-  }
-  __syncthreads();
-  return s_last != 0;
 }
 
 // Fixed-order total of one partial slot (called by every thread of the last block).
@@ -1254,79 +1241,6 @@ cudaError_t launch_rhs(const Geo& g, const int32_t* phase, const double* sig, do
   long long blocks = (g.N + threads - 1) / threads;
   if (blocks > (long long)sm_count * 16) blocks = (long long)sm_count * 16;
   k_rhs<<<(int)blocks, threads, 0, s>>>(g.nx, g.ny, g.nz, g.N, phase, sig, b);
-  return cudaGetLastError();
-}
-
-// ---- stress (stress_OpenMP / stress_fullfield_OpenMP) ---------------------------------------
-// Centroid gradient: d w_c / d x_d = (sum_a s_d(a) w_a,c) / 4.
-__global__ void k_stress(int nx, int ny, int nz, long long N, const int32_t* __restrict__ phase,
-                         const double* __restrict__ cfull, StressE E6, const double* __restrict__ w,
-                         double* __restrict__ stress, double* __restrict__ vm, double* parts, unsigned int* ctr,
-                         double* macro_out) {
-  __shared__ double red[32];
-  double acc[6] = {0, 0, 0, 0, 0, 0};
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < N; e += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(e % nx), j = (int)((e / nx) % ny), k = (int)(e / ((long long)nx * ny));
-    const int ph = phase[e];
-    double s6[6] = {0, 0, 0, 0, 0, 0};
-    if (ph >= 0) {
-      double G[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};  // G[c][d]
-#pragma unroll
-      for (int a = 0; a < 8; ++a) {
-        const int ax = a & 1, ay = (a >> 1) & 1, az = (a >> 2) & 1;
-        const long long n = (long long)wrapi(i + ax, nx) + (long long)nx * (wrapi(j + ay, ny) + (long long)ny * wrapi(k + az, nz));
-        const double sd[3] = {0.25 * (2 * ax - 1), 0.25 * (2 * ay - 1), 0.25 * (2 * az - 1)};
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const double wc = w[c * N + n];
-#pragma unroll
-          for (int d = 0; d < 3; ++d) G[c][d] += sd[d] * wc;
-        }
-      }
-      const double ev[6] = {E6.v[0] + G[0][0], E6.v[1] + G[1][1], E6.v[2] + G[2][2],
-                            2.0 * E6.v[3] + G[1][2] + G[2][1], 2.0 * E6.v[4] + G[0][2] + G[2][0],
-                            2.0 * E6.v[5] + G[0][1] + G[1][0]};
-      const double* C = cfull + (long long)ph * kSymStride;
-#pragma unroll
-      for (int r = 0; r < 6; ++r) {
-        double t = 0.0;
-#pragma unroll
-        for (int c = 0; c < 6; ++c) t += C[pk(r, c)] * ev[c];
-        s6[r] = t;
-      }
-    }
-    if (stress) {
-#pragma unroll
-      for (int r = 0; r < 6; ++r) stress[r * N + e] = s6[r];
-    }
-    if (vm) {
-      const double d1 = s6[0] - s6[1], d2 = s6[1] - s6[2], d3 = s6[2] - s6[0];
-      vm[e] = sqrt(0.5 * (d1 * d1 + d2 * d2 + d3 * d3) + 3.0 * (s6[3] * s6[3] + s6[4] * s6[4] + s6[5] * s6[5]));
-    }
-#pragma unroll
-    for (int r = 0; r < 6; ++r) acc[r] += s6[r];
-  }
-  double b[6];
-#pragma unroll
-  for (int r = 0; r < 6; ++r) b[r] = block_sum(acc[r], red);
-  if (!publish_and_arrive(parts, b, 6, ctr)) return;
-  for (int r = 0; r < 6; ++r) {
-    const double tot = total_of(parts + r * kMaxParts, gridDim.x, red);
-    if (threadIdx.x == 0) macro_out[r] = tot / (double)N;
-  }
-  if (threadIdx.x == 0) *ctr = 0u;
-}
-
-cudaError_t launch_stress(const Geo& g, const int32_t* phase, const double* cfull, const double* E6,
-                          const double* w, double* stress, double* vm, double* parts, unsigned int* ctr,
-                          double* macro_out, int sm_count, cudaStream_t s) {
-  const int threads = 256;
-  long long blocks = (g.N + threads - 1) / threads;
-  if (blocks > (long long)sm_count * 8) blocks = (long long)sm_count * 8;
-  if (blocks > kMaxParts) blocks = kMaxParts;  // one partial-sum slot per block
-  StressE e;
-  for (int i = 0; i < 6; ++i) e.v[i] = E6[i];
-  k_stress<<<(int)blocks, threads, 0, s>>>(g.nx, g.ny, g.nz, g.N, phase, cfull, e, w, stress, vm, parts, ctr, macro_out);
   return cudaGetLastError();
 }
 

@@ -408,7 +408,7 @@ int elas_batch_stress(elas_batch* b, int rve, int rhs, const double* strain, dou
   const RveDev& R = b->rves[rve];
   DevState* st = b->stress_state;
   cudaError_t e = launch_stress(R.geo, R.phase, R.cfull, strain, pd.w, stress, von_mises, b->parts_stress, &st->ctr[3],
-                                st->macro, b->sm_count, b->stream);
+                                macro_stress ? st->macro : nullptr, b->sm_count, b->stream);
   if (e != cudaSuccess) return bfail(b, ELAS_ERR_CUDA, "elas_batch_stress: launch");
   if (macro_stress) {
     if (cudaMemcpyAsync(b->aux.h_states, st, sizeof(DevState), cudaMemcpyDeviceToHost, b->stream) != cudaSuccess ||

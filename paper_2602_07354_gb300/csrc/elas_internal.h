@@ -83,10 +83,6 @@ __device__ __forceinline__ bool replacement_due(const DevState* st) {
 }
 #endif
 
-struct StressE {
-  double v[6];
-};
-
 #ifdef __CUDACC__
 // ---- double-float arithmetic ------------------------------------------------------------------
 // An FP64 value carried as an unevaluated pair of floats v = hi + lo (about 48 significant bits),
@@ -354,6 +350,7 @@ cudaError_t launch_jacobi(const Geo& g, const int32_t* phase, const double* coef
                           int mode = ELAS_PRECOND_BLOCK);
 cudaError_t launch_rhs(const Geo& g, const int32_t* phase, const double* sig, double* b, int sm_count,
                        cudaStream_t s);
+// stress.cu: macro_out (device, 6 values) may be null: no macroscopic stress is formed
 cudaError_t launch_stress(const Geo& g, const int32_t* phase, const double* cfull, const double* E6,
                           const double* w, double* stress, double* vm, double* parts, unsigned int* ctr,
                           double* macro_out, int sm_count, cudaStream_t s);

@@ -12,7 +12,7 @@
 #include <climits>
 #include <cstdlib>
 
-#include "elas_internal.h"
+#include "column_tile.h"
 
 namespace elas {
 
@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(kHotThreads, R == 1 ? 2 : 1)
   const int t = threadIdx.x, wx = tx + 2 * R, wy = ty + 2 * R, np = wx * wy;
   double* const val = reinterpret_cast<double*>(hot_smem);            // [2][NQ][np]
   unsigned char* const sol = reinterpret_cast<unsigned char*>(val + 2 * NQ * np);  // [2][np]
-  const int bx = (nx + tx - 1) / tx, by = (ny + ty - 1) / ty, bz = (nz + zc - 1) / zc;
+  const int bx = (nx - 1) / tx + 1, by = (ny - 1) / ty + 1, bz = (nz - 1) / zc + 1;
   const long long plane = (long long)nx * ny;
   const int i = t % tx, j = t / tx;
   const bool own = j < ty;
@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(kHotThreads)
   const int t = threadIdx.x, wx = tx + 2, np = wx * (ty + 2);
   long long* const key = reinterpret_cast<long long*>(hot_smem);                      // [2][np]
   unsigned char* const sol = reinterpret_cast<unsigned char*>(key + 2 * np);           // [2][np]
-  const int bx = (nx + tx - 1) / tx, by = (ny + ty - 1) / ty, bz = (nz + zc - 1) / zc;
+  const int bx = (nx - 1) / tx + 1, by = (ny - 1) / ty + 1, bz = (nz - 1) / zc + 1;
   const long long plane = (long long)nx * ny;
   const int i = t % tx, j = t / tx;
   unsigned long long bits = 0ull, vox = ~0ull;
@@ -332,52 +332,16 @@ __global__ void __launch_bounds__(kHotThreads)
   }
 }
 
-// Tile of at most kHotThreads columns with the fewest idle threads over the grid (an idle lane costs
-// its warp's FP64 instructions as much as a busy one), then the fewest halo columns; layers per item
-// so that the busiest SM (the SM's blocks share its pipes) has the least work, the item's neighbour
-// planes counted as one layer.  One block per item: the hardware hands them out as SMs free up.
-struct HotTile {
-  int tx, ty, zc, blocks, pos;
-};
-HotTile hot_tile(const Geo& g, int r, int sm_count, int max_pos) {
-  HotTile best{};
-  double cost0 = 1e300;
-  for (int tx = 4; tx <= 64; ++tx) {
-    const int ty = kHotThreads / tx;
-    if ((tx + 2 * r) * (ty + 2 * r) > max_pos) continue;
-    const double cols = (double)((g.nx + tx - 1) / tx) * ((g.ny + ty - 1) / ty);
-    const double cost = cols * (kHotThreads + 0.3 * (tx + 2 * r) * (ty + 2 * r));
-    if (cost < cost0) {
-      cost0 = cost;
-      best.tx = tx;
-      best.ty = ty;
-      best.pos = (tx + 2 * r) * (ty + 2 * r);
-    }
-  }
-  const long long tiles = (long long)((g.nx + best.tx - 1) / best.tx) * ((g.ny + best.ty - 1) / best.ty);
-  double c0 = 1e300;
-  for (int zc = 1; zc <= g.nz && zc <= 256; ++zc) {
-    const long long items = tiles * ((g.nz + zc - 1) / zc);
-    const double c = (double)((items + sm_count - 1) / sm_count) * (zc + 1.0 * r);
-    if (c < c0 && items < (1 << 30)) {
-      c0 = c;
-      best.zc = zc;
-      best.blocks = (int)items;
-    }
-  }
-  return best;
-}
-
 template <int R>
 cudaError_t launch_smooth(const Geo& g, const int32_t* phase, const double* vm, const Weights& W, double* smooth,
                           int sm_count, cudaStream_t s) {
   constexpr int NQ = R == 1 ? 8 : 1;
-  const HotTile h = hot_tile(g, R, sm_count, R == 1 ? 704 : 3 * kHotThreads);
-  const size_t smem = (size_t)h.pos * 2 * (NQ * sizeof(double) + 1);
+  const ColumnTile h = column_tile(g, kHotThreads, 2 * R, 2 * R, R, sm_count, R == 1 ? 704 : 3 * kHotThreads);
+  const size_t smem = (size_t)(h.tx + 2 * R) * (h.ty + 2 * R) * 2 * (NQ * sizeof(double) + 1);
   constexpr int most = R == 1 ? 2 * 704 * (8 * NQ + 1) : 2 * 3 * kHotThreads * (8 * NQ + 1);
   cudaError_t e = cudaFuncSetAttribute(k_smooth<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
   if (e != cudaSuccess) return e;
-  k_smooth<R><<<h.blocks, kHotThreads, smem, s>>>(g.nx, g.ny, g.nz, h.tx, h.ty, h.zc, phase, vm, W, smooth);
+  k_smooth<R><<<h.items, kHotThreads, smem, s>>>(g.nx, g.ny, g.nz, h.tx, h.ty, h.zc, phase, vm, W, smooth);
   return cudaGetLastError();
 }
 
@@ -405,8 +369,9 @@ cudaError_t launch_hotspot(const Geo& g, const int32_t* phase, const double* vm,
   unsigned int* ctr = reinterpret_cast<unsigned int*>(best2 + 2);
   if (e == cudaSuccess) e = cudaMemsetAsync(ctr, 0, sizeof(unsigned int), s);
   if (e != cudaSuccess) return e;
-  const HotTile h = hot_tile(g, 1, sm_count, 2 * kHotThreads);
-  k_hotspot<<<std::min(h.blocks, kMaxParts), kHotThreads, (size_t)h.pos * 2 * (sizeof(long long) + 1), s>>>(
+  const ColumnTile h = column_tile(g, kHotThreads, 2, 2, 1, sm_count, 2 * kHotThreads);
+  const size_t smem = (size_t)(h.tx + 2) * (h.ty + 2) * 2 * (sizeof(long long) + 1);
+  k_hotspot<<<std::min(h.items, kMaxParts), kHotThreads, smem, s>>>(
       g.nx, g.ny, g.nz, h.tx, h.ty, h.zc, phase, smooth, solid_only, best2, ctr, best2 + 8);
   return cudaGetLastError();
 }

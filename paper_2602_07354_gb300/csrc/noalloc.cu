@@ -149,7 +149,8 @@ extern "C" int elas_stress_noalloc(int nx, int ny, int nz, const int32_t* phase_
   Geo g{nx, ny, nz, N};
   double* macro_dev = reinterpret_cast<double*>(base + kOffMacro);
   if (launch_stress(g, phase_id, reinterpret_cast<const double*>(base + kOffC), strain, w, stress, von_mises,
-                    reinterpret_cast<double*>(base + kOffParts), ctr, macro_dev, sms, s) != cudaSuccess)
+                    reinterpret_cast<double*>(base + kOffParts), ctr, macro_stress ? macro_dev : nullptr, sms,
+                    s) != cudaSuccess)
     return ELAS_ERR_CUDA;
   if (macro_stress) {
     if (cudaMemcpyAsync(macro_stress, macro_dev, sizeof(double) * 6, cudaMemcpyDeviceToHost, s) != cudaSuccess)
