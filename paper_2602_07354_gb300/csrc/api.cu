@@ -370,12 +370,12 @@ size_t carve(elas_ctx* c, char* base, int nx, int ny, int nz, int n_phases, int 
   const long long N = (long long)nx * ny * nz;
   const bool mixed = precision == ELAS_PREC_MIXED;
   const size_t vb = mixed ? sizeof(float) : sizeof(double);
-  const long long stride = std::max(max_tiles_bound(N), chunks_of(N));
+  const long long stride = std::max(max_tiles_bound(N), chunks_of(N, mixed));
   const size_t P = (size_t)std::max(n_phases, 1);
   Carve cv{base};
-  char* t_main = cv.take(engine_table_bytes(1, stride, chunks_of(N)));
-  char* t_64 = cv.take(engine_table_bytes(1, stride, chunks_of(N)));
-  char* t_32 = cv.take(engine_table_bytes(1, stride, chunks_of(N)));
+  char* t_main = cv.take(engine_table_bytes(1, stride, chunks_of(N, mixed)));
+  char* t_64 = cv.take(engine_table_bytes(1, stride, chunks_of(N, mixed)));
+  char* t_32 = cv.take(engine_table_bytes(1, stride, chunks_of(N, mixed)));
   int32_t* phase = (int32_t*)cv.take(sizeof(int32_t) * N);
   double* coef64 = (double*)cv.take(sizeof(double) * kCoefStride * P);
   float* coef32 = (float*)cv.take(sizeof(float) * kCoef32Stride * P);
@@ -410,7 +410,9 @@ Prob make_prob(elas_ctx* c, const Tiling& tl, double* parts) {
   p.nx = c->geo.nx; p.ny = c->geo.ny; p.nz = c->geo.nz; p.N = c->geo.N;
   p.tx = tl.tx; p.ty = tl.ty; p.kc = tl.kc; p.tiles_x = tl.tiles_x; p.tiles_y = tl.tiles_y;
   p.n_tiles = (int)tl.n_tiles;
-  p.n_chunks = (int)chunks_of(c->geo.N);
+  const bool mixed = c->precision == ELAS_PREC_MIXED;
+  p.chunk = vec_chunk(c->geo.N, mixed);
+  p.n_chunks = (int)chunks_of(c->geo.N, mixed);
   p.parts_stride = (int)c->stride;
   p.phase = c->phase;
   p.coef64 = c->coef64;
@@ -550,7 +552,7 @@ int elas_create(elas_ctx** out, int nx, int ny, int nz, const int32_t* phase_id,
   if (e != cudaSuccess) return bail(cuda_fail(c, e, "elas_create: device query"));
   carve(c, (char*)workspace, nx, ny, nz, n_phases, precision);
   const bool mixed = precision == ELAS_PREC_MIXED;
-  const long long nch = chunks_of(c->geo.N);
+  const long long nch = chunks_of(c->geo.N, mixed);
   char* t_main = (char*)c->main.d_counts;
   char* t_64 = (char*)c->aux64.d_counts;
   char* t_32 = (char*)c->aux32.d_counts;

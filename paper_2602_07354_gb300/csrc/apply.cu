@@ -447,6 +447,7 @@ __device__ __forceinline__ void block_jacobi_apply(const Tv* __restrict__ minv, 
 // The scalar step a problem's last item performs on the problem's totals (s0: h.Ah or z.g, s1: r.r).
 __device__ void post_scalars(DevState* st, int post, double s0, double s1) {
   if (post == POST_LAMBDA) {  // Algorithm 2 step B
+    st->w_applied = 1;  // the direction before this product advanced w
     st->hAh = s0;
     if (st->iter == 0) st->hAh_first = s0;
     if (!isfinite(s0)) {
@@ -486,6 +487,7 @@ __device__ void post_scalars(DevState* st, int post, double s0, double s1) {
     st->gamma = gg_new / st->gg_last;
     st->gam_f = (float)st->gamma;
     st->want_check = 0;
+    st->w_applied = 1;  // by the pass before this residual
     st->last_repl_iter = st->iter;
   }
 }

@@ -95,8 +95,8 @@ size_t batch_carve(elas_batch* b, char* base, int n_rve, const elas_rve* rv, int
   for (int i = 0; i < n_rve; ++i) {
     const long long N = (long long)rv[i].nx * rv[i].ny * rv[i].nz;
     cap_apply += (long long)n_rhs * max_tiles_bound(N);  // room for any tiling the autotuner picks
-    cap_vec += (long long)n_rhs * chunks_of(N);
-    max_bound = std::max(max_bound, std::max(max_tiles_bound(N), chunks_of(N)));
+    cap_vec += (long long)n_rhs * chunks_of(N, mixed);
+    max_bound = std::max(max_bound, std::max(max_tiles_bound(N), chunks_of(N, mixed)));
   }
   Carve cv{base};
   char* t_main = cv.take(engine_table_bytes(n_rve * n_rhs, cap_apply, cap_vec));
@@ -122,7 +122,7 @@ size_t batch_carve(elas_batch* b, char* base, int n_rve, const elas_rve* rv, int
       RveDev& R = b->rves[i];
       R.phase = phase; R.coef64 = coef64; R.coef32 = coef32; R.cfull = cfull; R.minv = minv;
     }
-    const long long stride = std::max(max_tiles_bound(N), chunks_of(N));
+    const long long stride = std::max(max_tiles_bound(N), chunks_of(N, mixed));
     for (int r = 0; r < n_rhs; ++r) {
       ProbDev pd;
       pd.rve = i;
@@ -157,7 +157,9 @@ Prob prob_of(elas_batch* b, const ProbDev& pd) {
   p.nx = R.geo.nx; p.ny = R.geo.ny; p.nz = R.geo.nz; p.N = R.geo.N;
   p.tx = R.tl.tx; p.ty = R.tl.ty; p.kc = R.tl.kc; p.tiles_x = R.tl.tiles_x; p.tiles_y = R.tl.tiles_y;
   p.n_tiles = (int)R.tl.n_tiles;
-  p.n_chunks = (int)chunks_of(R.geo.N);
+  const bool mixed = b->precision == ELAS_PREC_MIXED;
+  p.chunk = vec_chunk(R.geo.N, mixed);
+  p.n_chunks = (int)chunks_of(R.geo.N, mixed);
   p.parts_stride = (int)pd.stride;
   p.phase = R.phase;
   p.coef64 = R.coef64;

@@ -58,8 +58,9 @@ struct DevState {
   double rr_repl;   // rr right after the last replacement (or at the start)
   double drop2;     // replace once rr <= drop2 * rr_repl (0: off)
   int iter, max_iter, status, done;
+  int w_applied;    // w holds every completed iteration's lambda h (0: the last one is still due)
   int stop_rule, n_repl, want_check, last_repl_iter;
-  int replace_every, needs_init, finalized, pad2;
+  int replace_every, needs_init, finalized;
   float lam_hi, lam_lo;  // lambda as an unevaluated float pair (mixed path)
   float gam_f, pad_f;    // gamma rounded to float (mixed path)
   double E[9];           // applied strain tensor (row-major) of the current solve / product
@@ -238,6 +239,47 @@ __device__ __forceinline__ double block_total(const DotAcc<float>& a, double* re
   }
   return r;
 }
+// Two sums over the block at once: the totals in thread 0 (the first) and thread 32 (the second).  FP64:
+// the threads' sums go through shared memory and one warp per sum adds them, 12 FP64 instructions a
+// sum instead of 5 in every warp.  buf: 2 blockDim doubles; active: threads that hold nodes.
+__device__ __forceinline__ double block_total2(const DotAcc<double>& a, const DotAcc<double>& b, double* buf, int active) {
+  __syncthreads();
+  buf[threadIdx.x] = a.s;
+  buf[blockDim.x + threadIdx.x] = b.s;
+  __syncthreads();
+  double v = 0.0;
+  const int wid = threadIdx.x >> 5;
+  if (wid < 2) {
+    const double* s = buf + wid * blockDim.x + (threadIdx.x & 31);
+    v = s[0];
+    for (int i = 32; i < active; i += 32) v += s[i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  }
+  return v;
+}
+// FP32 pairs: the first step leaves one of the sums in each half-warp.
+__device__ __forceinline__ double block_total2(const DotAcc<float>& a, const DotAcc<float>& b, double* buf, int active) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  float2* r2 = reinterpret_cast<float2*>(buf);
+  __syncthreads();
+  if (wid * 32 < active) {
+    DotAcc<float> v = lane < 16 ? a : b;
+    const DotAcc<float> other = lane < 16 ? b : a;
+    v.merge(__shfl_xor_sync(0xffffffffu, other.hi, 16), __shfl_xor_sync(0xffffffffu, other.lo, 16));
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) {
+      const float ohi = __shfl_xor_sync(0xffffffffu, v.hi, o), olo = __shfl_xor_sync(0xffffffffu, v.lo, o);
+      v.merge(ohi, olo);
+    }
+    if ((lane & 15) == 0) r2[2 * wid + (lane >> 4)] = make_float2(v.hi, v.lo);
+  }
+  __syncthreads();
+  DotAcc<float> t;
+  if (wid < 2 && lane == 0)
+    for (int i = 0; i < active; i += 32) t.merge(r2[i / 16 + wid].x, r2[i / 16 + wid].y);
+  return t.value();
+}
 __device__ __forceinline__ double block_total(const DotAcc<ff>& a, double* red) {
   DotAcc<float> f;
   f.hi = a.hi;
@@ -278,15 +320,26 @@ struct Geo {
 // A single solve is a batch of one problem.
 // ------------------------------------------------------------------------------------------
 constexpr int kVecThreads = 256;                    // block size of the vector kernels
-constexpr int kVecPerThread = 4;                    // nodes per thread per work item
-constexpr int kVecChunk = kVecThreads * kVecPerThread;  // nodes per vector-kernel work item
+// Nodes per vector-kernel work item, by the grid's size and precision alone (so a problem's sums do
+// not depend on its batch): the grid's nodes are split evenly over whole waves of resident blocks
+// (four a SM in FP64, three mixed), because an uneven split leaves the last wave nearly empty (977
+// items of 1,024 nodes over 608 resident blocks took 246 us per FP64 iteration at 100^3, 607 of 1,648
+// 237; mixed 71 and 65).  At most 4,096 nodes an item, at least
+// 256 (128 in FP64, whose nodes must spread over the SMs' FP64 pipes), in whole rows of 4.
+constexpr long long kVecWave64 = 152 * 4, kVecWave32 = 152 * 3;
+constexpr int vec_chunk(long long N, bool mixed) {
+  const long long wave = mixed ? kVecWave32 : kVecWave64, least = mixed ? 256 : 128;
+  const long long waves = (N + wave * 4096 - 1) / (wave * 4096);
+  const long long c = ((N + wave * waves - 1) / (wave * waves) + 3) / 4 * 4;
+  return (int)(c < least ? least : c);
+}
 constexpr int kPartsSlots = 3;
 
 struct Prob {
   int nx, ny, nz;
   long long N;
   int tx, ty, kc, tiles_x, tiles_y, n_tiles;  // operator tiling of this grid
-  int n_chunks;                                // vector-kernel items
+  int chunk, n_chunks;                         // nodes per vector-kernel item, items
   int parts_stride;                            // >= max(n_tiles, n_chunks)
   long long item0_apply, item0_vec;            // first work item of this problem
   const int32_t* phase;
@@ -317,6 +370,8 @@ struct BatchDev {
   size_t smemff;           // ... of double-float FP64 operator launches
   int blocks32, blocks64;  // persistent grids of FP32 / FP64 operator launches
   int vec_blocks, vec_threads;
+  int single;              // the batch is one problem: its descriptor also goes as a kernel argument
+  Prob one;
   int nohalo64;            // native FP64 iteration operator without recomputed x/y halo (+ edge pass)
   int ff64;                // FP64 products in double-float arithmetic (ELAS_FP64_OP_PAIRED)
 };
@@ -368,8 +423,8 @@ cudaError_t launch_state_init(const BatchDev& b, const SolveSetup* setups, const
 cudaError_t launch_pcg_init(const BatchDev& b, bool mixed, cudaStream_t s);
 cudaError_t launch_pcg_update(const BatchDev& b, bool mixed, cudaStream_t s);
 cudaError_t launch_pcg_direction(const BatchDev& b, bool mixed, cudaStream_t s);
-// w = w_hi + w_lo in FP64 (mixed path); gate: GATE_NONE, GATE_REPLACE or GATE_FINALIZE
-cudaError_t launch_w_combine(const BatchDev& b, int gate, cudaStream_t s);
+// w up to date, in FP64 (mixed path: w = w_hi + w_lo); gate: GATE_NONE, GATE_REPLACE or GATE_FINALIZE
+cudaError_t launch_w_finish(const BatchDev& b, bool mixed, int gate, cudaStream_t s);
 
 // hotspot.cu ---------------------------------------------------------------------------------
 // Maximum-stress extraction of App. C.  Gaussian of standard deviation s (voxels) truncated at

@@ -34,7 +34,7 @@ int record_batch(Engine& e, int K, std::string* err) {
     r = launch_apply(e.bd, e.mixed ? AK_F32_DOT : AK_F64_DOT, POST_LAMBDA, GATE_RUNNING, s);
     if (r == cudaSuccess) r = launch_pcg_update(e.bd, e.mixed, s);
     if (r == cudaSuccess && it == K - 1) {
-      if (e.mixed) r = launch_w_combine(e.bd, GATE_REPLACE, s);
+      r = launch_w_finish(e.bd, e.mixed, GATE_REPLACE, s);
       if (r == cudaSuccess)
         r = launch_apply(e.bd, e.mixed ? AK_MIX_RESID : AK_F64_RESID, POST_REPLACE, GATE_REPLACE, s);
     }
@@ -178,7 +178,9 @@ int engine_set_problems(Engine& e, const std::vector<Prob>& probs, std::string* 
 }
 
 int engine_upload_probs(Engine& e, std::string* err) {
+  e.bd.single = e.probs.size() == 1 && !e.fixed_smem32;  // (a fixed launch shape outlives its problems)
   if (e.probs.empty()) return ELAS_OK;
+  e.bd.one = e.probs[0];
   cudaError_t c = cudaMemcpyAsync(e.d_probs, e.probs.data(), sizeof(Prob) * e.probs.size(), cudaMemcpyHostToDevice,
                                   e.stream);
   if (c != cudaSuccess) return cfail(err, c, "engine descriptors");
@@ -209,12 +211,10 @@ int engine_solve(Engine& e, const std::vector<SolveSetup>& setups, int K, int* l
     for (int i = 0; i < n; ++i) all_done &= e.h_states[i].done != 0;
     if (all_done || b >= max_batches) break;
     if ((c = cudaGraphLaunch(e.exec, s)) != cudaSuccess) return cfail(err, c, "cudaGraphLaunch");
-    L += 3 * K + 1 + (e.mixed ? 1 : 0);
+    L += 3 * K + 2;
   }
-  if (e.mixed) {
-    if ((c = launch_w_combine(e.bd, GATE_NONE, s)) != cudaSuccess) return cfail(err, c, "w combine");
-    L += 1;
-  }
+  if ((c = launch_w_finish(e.bd, e.mixed, GATE_NONE, s)) != cudaSuccess) return cfail(err, c, "w finish");
+  L += 1;
   // FP64 true residual of every returned w
   if ((c = launch_apply(e.bd, AK_F64_NORM, POST_TRUE_NORM, GATE_NONE, s)) != cudaSuccess)
     return cfail(err, c, "true residual");

@@ -43,7 +43,8 @@ size_t engine_table_bytes(int cap_probs, long long cap_apply, long long cap_vec)
 
 // Item counts of one grid under its tiling.
 inline long long tiles_of(const Tiling& t) { return t.n_tiles; }
-inline long long chunks_of(long long N) { return (N + kVecChunk - 1) / kVecChunk; }
+inline long long chunks_of(long long N, bool mixed) { return (N + vec_chunk(N, mixed) - 1) / vec_chunk(N, mixed); }
+constexpr int kMoreChunks = 2048;  // chunks_of(N) <= N / 2048 + kMoreChunks
 
 // Prepare an engine: tables in `mem` (engine_table_bytes), streams and pinned state mirror.
 int engine_init(Engine& e, bool mixed, int sm_count, int apply_threads, int cap_probs, long long cap_apply,

@@ -3,9 +3,12 @@
 // One iteration of Algorithm 2 is three launches on the device:
 //   apply      Ah = A h with the h.Ah partial sums fused into its epilogue; a problem's last
 //              item forms lambda = gg / hAh (step B) and applies the breakdown guard
-//   update     w -= lambda h, g -= lambda Ah (step C), z = M^-1 g and gg = z.g, g.g (step D);
-//              a problem's last item forms gg, gamma = gg / gg_last and decides convergence
-//   direction  h = z + gamma h (step E)
+//   update     g -= lambda Ah (step C), z = M^-1 g and gg = z.g, g.g (step D); a problem's last item
+//              forms gg, gamma = gg / gg_last and decides convergence
+//   direction  w -= lambda h (step C's other half) and h = z + gamma h (step E)
+// w is advanced with the direction because that kernel reads h anyway: h is then read twice an
+// iteration instead of three times, and the update's FP64 work falls by a seventh.  A solve that stops
+// in its update, and every FP64 residual, brings w up to date first (k_w_finish).
 // Every launch walks a flattened list of (problem, node chunk) items over all problems of the
 // batch (one problem = one RVE with one load case).  All scalars live in device memory
 // (DevState per problem), so a batch of iterations runs without the host; a finished (or
@@ -99,6 +102,7 @@ __global__ void k_state_init(const Prob* __restrict__ probs, const SolveSetup* _
   st->last_repl_iter = 0;
   st->done = 0;
   st->needs_init = 1;
+  st->w_applied = 1;
   st->status = ST_RUNNING;
   st->gg = st->gg0 = st->gg_last = st->hAh = st->hAh_first = st->lambda = st->gamma = 0.0;
   st->rr = st->bb = st->rr_true = 0.0;
@@ -117,7 +121,7 @@ __global__ void k_pcg_init(const Prob* __restrict__ probs, const int* __restrict
     const Prob& P = probs[vitem_prob[item]];
     if (!P.st->needs_init) continue;  // only problems set up since their last start
     const int chunk = (int)(item - P.item0_vec);
-    const long long N = P.N, n0 = (long long)chunk * kVecChunk, n1 = min(n0 + kVecChunk, N);
+    const long long N = P.N, n0 = (long long)chunk * P.chunk, n1 = min(n0 + P.chunk, N);
     const int nx = P.nx, ny = P.ny, nz = P.nz;
     Tv* __restrict__ g = reinterpret_cast<Tv*>(P.g);
     Tv* __restrict__ h = reinterpret_cast<Tv*>(P.h);
@@ -130,10 +134,7 @@ __global__ void k_pcg_init(const Prob* __restrict__ probs, const int* __restrict
     const Tv* __restrict__ minv = reinterpret_cast<const Tv*>(P.minv);
     DotAcc<Tv> zg, gg2;
     DotAcc<double> bb;
-#pragma unroll
-    for (int q = 0; q < kVecPerThread; ++q) {
-      const long long n = n0 + q * kVecThreads + threadIdx.x;
-      if (n >= n1) break;
+    for (long long n = n0 + threadIdx.x; n < n1; n += kVecThreads) {
       const int i = (int)(n % nx), j = (int)((n / nx) % ny), k = (int)(n / ((long long)nx * ny));
       double b[3] = {0, 0, 0};
 #pragma unroll
@@ -204,34 +205,29 @@ __global__ void k_pcg_init(const Prob* __restrict__ probs, const int* __restrict
   }
 }
 
-// One node of steps C and D: w -= lambda h, g -= lambda Ah, z = M^-1 g, and the two dot terms.
-// Mixed path: w is the unevaluated pair (wh, wl), updated with error-free transformations
-// (_rn intrinsics keep the compiler from contracting them into FMAs).
-template <bool MIXED, typename Tv>
-__device__ __forceinline__ void update_node(const Tv (&h)[3], const Tv (&Ah)[3], Tv (&g)[3], float (&wh)[3],
-                                            float (&wl)[3], double* w, long long N, long long n, const Tv (&m)[6],
-                                            Tv (&z)[3], double lam, float lam_hi, float lam_lo, Tv lam_v,
+// w -= lambda h for one component of one node.  Mixed path: w is the unevaluated pair (wh, wl), updated
+// with error-free transformations (_rn intrinsics keep the compiler from contracting them into FMAs).
+__device__ __forceinline__ void w_step(float& wh, float& wl, float h, float lam_hi, float lam_lo) {
+  const float prod = __fmul_rn(lam_hi, h);
+  const float perr = __fadd_rn(fmaf(lam_hi, h, -prod), __fmul_rn(lam_lo, h));  // lambda h = prod + perr
+  const float s = __fsub_rn(wh, prod);  // two-sum of wh and -prod
+  const float bb = __fsub_rn(s, wh);
+  const float e = __fadd_rn(__fadd_rn(__fsub_rn(wh, __fsub_rn(s, bb)), __fsub_rn(-prod, bb)), __fsub_rn(wl, perr));
+  const float nh = __fadd_rn(s, e);  // renormalise the pair
+  wl = __fsub_rn(e, __fsub_rn(nh, s));
+  wh = nh;
+}
+
+// One node of steps C and D without w: g -= lambda Ah, z = M^-1 g (symmetric inverse in Voigt slot
+// order 11, 22, 33, 23, 13, 12), and the two dot terms.
+template <typename Tv>
+__device__ __forceinline__ void update_node(const Tv (&Ah)[3], Tv (&g)[3], const Tv (&m)[6], Tv (&z)[3], Tv lam,
                                             DotAcc<Tv>& zg, DotAcc<Tv>& gg2) {
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    if (MIXED) {
-      const float hf = (float)h[c];
-      const float prod = __fmul_rn(lam_hi, hf);
-      const float perr = __fadd_rn(fmaf(lam_hi, hf, -prod), __fmul_rn(lam_lo, hf));  // lambda h = prod + perr
-      const float s = __fsub_rn(wh[c], prod);  // two-sum of wh and -prod
-      const float bb = __fsub_rn(s, wh[c]);
-      const float e =
-          __fadd_rn(__fadd_rn(__fsub_rn(wh[c], __fsub_rn(s, bb)), __fsub_rn(-prod, bb)), __fsub_rn(wl[c], perr));
-      const float nh = __fadd_rn(s, e);  // renormalise the pair
-      wl[c] = __fsub_rn(e, __fsub_rn(nh, s));
-      wh[c] = nh;
-    } else {
-      w[c * N + n] -= lam * (double)h[c];
-    }
-    g[c] = g[c] - lam_v * Ah[c];
+    g[c] = g[c] - lam * Ah[c];
     gg2.add(g[c], g[c]);
   }
-  // point-block Jacobi, symmetric inverse in Voigt slot order 11, 22, 33, 23, 13, 12
   z[0] = m[0] * g[0] + m[5] * g[1] + m[4] * g[2];
   z[1] = m[5] * g[0] + m[1] * g[1] + m[3] * g[2];
   z[2] = m[4] * g[0] + m[3] * g[1] + m[2] * g[2];
@@ -247,6 +243,7 @@ __device__ void update_scalar_step(DevState* st, double s_zg, double s_gg, bool 
   st->gg = s_zg;
   st->rr = s_gg;
   st->iter += 1;
+  st->w_applied = 0;  // the direction owes w its lambda h
   if (!isfinite(s_zg) || !isfinite(s_gg)) {
     st->status = ELAS_NONFINITE;
     st->done = 1;
@@ -269,182 +266,215 @@ __device__ void update_scalar_step(DevState* st, double s_zg, double s_gg, bool 
   }
 }
 
-// Publishes an update item's partials (z.g, g.g); the problem's last item performs the scalar step.
-__device__ void finish_update(const Prob& P, int chunk, const double (&vals)[2], bool mixed, double* red,
-                              int* s_last) {
-  if (publish_item(P, chunk, vals, 2, &P.st->ctr[2], s_last)) {
-    const double s_zg = total_of(P.parts, P.n_chunks, red);
-    const double s_gg = total_of(P.parts + P.parts_stride, P.n_chunks, red);
-    if (threadIdx.x == 0) update_scalar_step(P.st, s_zg, s_gg, mixed);
+// Rows of consecutive nodes: 4 floats or 2 doubles (16 bytes), used for grids whose size is a multiple
+// of the row (which path a node takes depends only on its problem).
+template <typename Tv>
+struct Row;
+template <>
+struct Row<float> {
+  static constexpr int V = 4;
+  using type = float4;
+};
+template <>
+struct Row<double> {
+  static constexpr int V = 2;
+  using type = double2;
+};
+template <typename Tv, int V>
+__device__ __forceinline__ void load_row(const Tv* __restrict__ p, Tv (&v)[V]) {
+  if constexpr (V == 1)
+    v[0] = *p;
+  else
+    *reinterpret_cast<typename Row<Tv>::type*>(v) = *reinterpret_cast<const typename Row<Tv>::type*>(p);
+}
+template <typename Tv, int V>
+__device__ __forceinline__ void store_row(Tv* __restrict__ p, const Tv (&v)[V]) {
+  if constexpr (V == 1)
+    *p = v[0];
+  else
+    *reinterpret_cast<typename Row<Tv>::type*>(p) = *reinterpret_cast<const typename Row<Tv>::type*>(v);
+}
+
+template <typename Tv, int V>
+__device__ __forceinline__ void update_chunk(const Prob& P, long long n0, long long n1, Tv lam, DotAcc<Tv>& zg,
+                                             DotAcc<Tv>& gg2) {
+  const long long N = P.N;
+  Tv* __restrict__ gp = reinterpret_cast<Tv*>(P.g);
+  const Tv* __restrict__ Ahp = reinterpret_cast<const Tv*>(P.Ah);
+  Tv* __restrict__ zp = reinterpret_cast<Tv*>(P.z);
+  const Tv* __restrict__ minv = reinterpret_cast<const Tv*>(P.minv);
+  for (long long n = n0 + V * (int)threadIdx.x; n < n1; n += V * kVecThreads) {
+    alignas(16) Tv A[3][V], g[3][V], m[6][V], z[3][V];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      load_row<Tv, V>(Ahp + c * N + n, A[c]);
+      load_row<Tv, V>(gp + c * N + n, g[c]);
+    }
+#pragma unroll
+    for (int q = 0; q < 6; ++q) load_row<Tv, V>(minv + q * N + n, m[q]);
+#pragma unroll
+    for (int j = 0; j < V; ++j) {
+      const Tv Aj[3] = {A[0][j], A[1][j], A[2][j]}, mj[6] = {m[0][j], m[1][j], m[2][j], m[3][j], m[4][j], m[5][j]};
+      Tv gj[3] = {g[0][j], g[1][j], g[2][j]}, zj[3];
+      update_node(Aj, gj, mj, zj, lam, zg, gg2);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        g[c][j] = gj[c];
+        z[c][j] = zj[c];
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      store_row<Tv, V>(gp + c * N + n, g[c]);
+      store_row<Tv, V>(zp + c * N + n, z[c]);
+    }
   }
 }
 
-__device__ __forceinline__ float q4(const float4& v, int j) { return j == 0 ? v.x : j == 1 ? v.y : j == 2 ? v.z : v.w; }
-__device__ __forceinline__ void s4(float4& v, int j, float x) {
-  if (j == 0) v.x = x; else if (j == 1) v.y = x; else if (j == 2) v.z = x; else v.w = x;
-}
-
-// Steps C and D of Algorithm 2.  FP32 vectors of a grid whose size is a multiple of 4 move as
-// float4 (each thread owns 4 consecutive nodes), all other cases node by node.
-template <typename Tv, bool MIXED, bool VEC>
+// Step C's residual half and step D of Algorithm 2.  Each item publishes its partials (z.g, g.g); the
+// problem's last item performs the scalar step.
+template <typename Tv, bool ONE>
 __device__ __forceinline__ void update_items(const Prob* __restrict__ probs, const int* __restrict__ vitem_prob,
-                                             const long long* __restrict__ counts) {
-  __shared__ double red[32];
+                                             const long long* __restrict__ counts, const Prob& one) {
+  __shared__ double buf[2 * kVecThreads];
   __shared__ int s_last;
-  const long long n_items = counts[1];
+  constexpr bool kMixed = sizeof(Tv) == 4;
+  const long long n_items = ONE ? one.n_chunks : counts[1];
   for (long long item = blockIdx.x; item < n_items; item += gridDim.x) {
-    const Prob& P = probs[vitem_prob[item]];
+    const Prob& P = ONE ? one : probs[vitem_prob[item]];
     const DevState* cst = P.st;
     if (cst->done || cst->want_check) continue;
     const int chunk = (int)(item - P.item0_vec);
-    const long long N = P.N, n0 = (long long)chunk * kVecChunk, n1 = min(n0 + kVecChunk, N);
-    Tv* __restrict__ gp = reinterpret_cast<Tv*>(P.g);
-    const Tv* __restrict__ hp = reinterpret_cast<const Tv*>(P.h);
-    const Tv* __restrict__ Ahp = reinterpret_cast<const Tv*>(P.Ah);
-    Tv* __restrict__ zp = reinterpret_cast<Tv*>(P.z);
-    const Tv* __restrict__ minv = reinterpret_cast<const Tv*>(P.minv);
-    double* __restrict__ w = P.w;
-    float* __restrict__ w_hi = P.w_hi;
-    float* __restrict__ w_lo = P.w_lo;
-    const double lam = cst->lambda;
-    const float lam_hi = cst->lam_hi, lam_lo = cst->lam_lo;  // formed once per problem
-    const Tv lam_v = MIXED ? (Tv)lam_hi : (Tv)lam;
+    const long long N = P.N, n0 = (long long)chunk * P.chunk, n1 = min(n0 + P.chunk, N);
+    const Tv lam = kMixed ? (Tv)cst->lam_hi : (Tv)cst->lambda;
     DotAcc<Tv> zg, gg2;
-    const long long nq = n0 + 4 * (long long)threadIdx.x;
-    if (VEC && MIXED && (N & 3) == 0 && nq + 3 < n1) {
-      // vector path: 4 consecutive nodes per thread, 21 float4 loads and 12 float4 stores
-      float4 h4[3], A4[3], g4[3], wh4[3], wl4[3], m4[6], z4[3];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        h4[c] = *reinterpret_cast<const float4*>(hp + c * N + nq);
-        A4[c] = *reinterpret_cast<const float4*>(Ahp + c * N + nq);
-        g4[c] = *reinterpret_cast<const float4*>(gp + c * N + nq);
-        wh4[c] = *reinterpret_cast<const float4*>(w_hi + c * N + nq);
-        wl4[c] = *reinterpret_cast<const float4*>(w_lo + c * N + nq);
-      }
-#pragma unroll
-      for (int q = 0; q < 6; ++q) m4[q] = *reinterpret_cast<const float4*>(minv + q * N + nq);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        Tv h[3], Ah[3], g[3], m[6], z[3];
-        float wh[3], wl[3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          h[c] = q4(h4[c], j); Ah[c] = q4(A4[c], j); g[c] = q4(g4[c], j);
-          wh[c] = q4(wh4[c], j); wl[c] = q4(wl4[c], j);
-        }
-#pragma unroll
-        for (int q = 0; q < 6; ++q) m[q] = q4(m4[q], j);
-        update_node<MIXED>(h, Ah, g, wh, wl, w, N, nq + j, m, z, lam, lam_hi, lam_lo, lam_v, zg, gg2);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          s4(g4[c], j, g[c]); s4(z4[c], j, z[c]); s4(wh4[c], j, wh[c]); s4(wl4[c], j, wl[c]);
-        }
-      }
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        *reinterpret_cast<float4*>(gp + c * N + nq) = g4[c];
-        *reinterpret_cast<float4*>(zp + c * N + nq) = z4[c];
-        *reinterpret_cast<float4*>(w_hi + c * N + nq) = wh4[c];
-        *reinterpret_cast<float4*>(w_lo + c * N + nq) = wl4[c];
-      }
-    } else {
-      // node by node: thread t owns nodes n0 + t + q*256 (the vector path's ragged tail and
-      // grids whose size is not a multiple of 4 run here; which path a node takes depends only
-      // on its problem)
-      const bool vec_problem = VEC && MIXED && (N & 3) == 0;
-#pragma unroll
-      for (int q = 0; q < kVecPerThread; ++q) {
-        const long long n = vec_problem ? nq + q : n0 + q * kVecThreads + threadIdx.x;
-        if (n >= n1) break;
-        Tv h[3], Ah[3], g[3], m[6], z[3];
-        float wh[3] = {0.f, 0.f, 0.f}, wl[3] = {0.f, 0.f, 0.f};
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          h[c] = hp[c * N + n];
-          Ah[c] = Ahp[c * N + n];
-          g[c] = gp[c * N + n];
-          if (MIXED) {
-            wh[c] = w_hi[c * N + n];
-            wl[c] = w_lo[c * N + n];
-          }
-        }
-#pragma unroll
-        for (int k = 0; k < 6; ++k) m[k] = minv[k * N + n];
-        update_node<MIXED>(h, Ah, g, wh, wl, w, N, n, m, z, lam, lam_hi, lam_lo, lam_v, zg, gg2);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          gp[c * N + n] = g[c];
-          zp[c * N + n] = z[c];
-          if (MIXED) {
-            w_hi[c * N + n] = wh[c];
-            w_lo[c * N + n] = wl[c];
-          }
-        }
-      }
+    const int V = N % Row<Tv>::V == 0 ? Row<Tv>::V : 1;
+    if (V > 1)
+      update_chunk<Tv, Row<Tv>::V>(P, n0, n1, lam, zg, gg2);
+    else
+      update_chunk<Tv, 1>(P, n0, n1, lam, zg, gg2);
+    const double v = block_total2(zg, gg2, buf, min(kVecThreads, ((int)(n1 - n0) + V - 1) / V));
+    if (threadIdx.x == 0) P.parts[chunk] = v;
+    if (threadIdx.x == 32) P.parts[P.parts_stride + chunk] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      __threadfence();
+      s_last = atomicAdd(&P.st->ctr[2], 1u) == (unsigned)(P.n_chunks - 1);
     }
-    const double vals[2] = {block_total(zg, red), block_total(gg2, red)};
-    finish_update(P, chunk, vals, MIXED, red, &s_last);
+    __syncthreads();
+    if (s_last) {
+      DotAcc<double> a, b;
+      for (int i = threadIdx.x; i < P.n_chunks; i += kVecThreads) {
+        a.s += __ldcg(P.parts + i);
+        b.s += __ldcg(P.parts + P.parts_stride + i);
+      }
+      const double t = block_total2(a, b, buf, kVecThreads);
+      if (threadIdx.x == 32) buf[kVecThreads] = t;  // (its readers are done: they are this warp)
+      __syncthreads();
+      if (threadIdx.x == 0) update_scalar_step(P.st, t, buf[kVecThreads], kMixed);
+    }
     __syncthreads();
   }
 }
 
-// FP64: four resident blocks per SM (64 registers): 3.6% faster per FP64 solve than three, 5% than
-// two; the update is bound by both the FP64 pipe (21 FP64 operations per node) and HBM.
+// Bound: HBM and L2 for the rows (144 bytes a node in FP64, 72 mixed), the FP64 pipe (18 operations a
+// node at 2 lanes per SM and clock) beside it in FP64.
+// 100^3, with the direction: FP64 76 -> 63 us, mixed 37 -> 27 us an iteration (in the solve's graph).
+template <bool ONE>
 __global__ void __launch_bounds__(kVecThreads, 4)
     k_pcg_update_f64(const Prob* __restrict__ probs, const int* __restrict__ vitem_prob,
-                     const long long* __restrict__ counts) {
-  update_items<double, false, false>(probs, vitem_prob, counts);
+                     const long long* __restrict__ counts, const __grid_constant__ Prob one) {
+  update_items<double, ONE>(probs, vitem_prob, counts, one);
 }
-// Mixed path: four consecutive nodes per thread as float4 rows, the compiler's own register choice
-// (measured against one node at a time per thread at 3, 4 and 6 blocks per SM: 51-66 ms per
-// mixed solve against 47 ms).
-__global__ void k_pcg_update_f32(const Prob* __restrict__ probs, const int* __restrict__ vitem_prob,
-                                 const long long* __restrict__ counts) {
-  update_items<float, true, true>(probs, vitem_prob, counts);
+template <bool ONE>
+__global__ void __launch_bounds__(kVecThreads, 3)
+    k_pcg_update_f32(const Prob* __restrict__ probs, const int* __restrict__ vitem_prob,
+                     const long long* __restrict__ counts, const __grid_constant__ Prob one) {
+  update_items<float, ONE>(probs, vitem_prob, counts, one);
 }
 
-// Step E of Algorithm 2 (Fletcher-Reeves direction).
-template <typename Tv>
-__global__ void k_pcg_direction(const Prob* __restrict__ probs, const int* __restrict__ vitem_prob,
-                                const long long* __restrict__ counts) {
-  const long long n_items = counts[1];
-  for (long long item = blockIdx.x; item < n_items; item += gridDim.x) {
-    const Prob& P = probs[vitem_prob[item]];
-    const DevState* cst = P.st;
-    if (cst->done || cst->want_check) continue;
-    const int chunk = (int)(item - P.item0_vec);
-    const long long N = P.N, n0 = (long long)chunk * kVecChunk, n1 = min(n0 + kVecChunk, N);
-    const Tv gam = sizeof(Tv) == 4 ? (Tv)cst->gam_f : (Tv)cst->gamma;
-    Tv* __restrict__ h = reinterpret_cast<Tv*>(P.h);
-    const Tv* __restrict__ z = reinterpret_cast<const Tv*>(P.z);
-    const long long nq = n0 + 4 * (long long)threadIdx.x;
-    if (sizeof(Tv) == 4 && (N & 3) == 0 && nq + 3 < n1) {
+// w -= lambda h and, with DIR, h = z + gamma h (step E, Fletcher-Reeves direction) on a chunk's nodes.
+template <typename Tv, int V, bool DIR>
+__device__ __forceinline__ void direction_chunk(const Prob& P, long long n0, long long n1, bool w_due, Tv gam) {
+  const long long N = P.N;
+  const DevState* st = P.st;
+  const double lam = st->lambda;
+  const float lam_hi = st->lam_hi, lam_lo = st->lam_lo;
+  Tv* __restrict__ h = reinterpret_cast<Tv*>(P.h);
+  const Tv* __restrict__ z = reinterpret_cast<const Tv*>(P.z);
+  double* __restrict__ w = P.w;
+  float* __restrict__ w_hi = P.w_hi;
+  float* __restrict__ w_lo = P.w_lo;
+  for (long long n = n0 + V * (int)threadIdx.x; n < n1; n += V * kVecThreads) {
+    alignas(16) Tv hv[3][V], zv[3][V], a[3][V], b[3][V];  // a, b: w, or its pair
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        float4 hv = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(h) + c * N + nq);
-        const float4 zv = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(z) + c * N + nq);
-        const float gf = (float)gam;
-        hv.x = zv.x + gf * hv.x; hv.y = zv.y + gf * hv.y; hv.z = zv.z + gf * hv.z; hv.w = zv.w + gf * hv.w;
-        *reinterpret_cast<float4*>(reinterpret_cast<float*>(h) + c * N + nq) = hv;
+    for (int c = 0; c < 3; ++c) {
+      load_row<Tv, V>(h + c * N + n, hv[c]);
+      if (DIR) load_row<Tv, V>(z + c * N + n, zv[c]);
+      if (w_due) {
+        if constexpr (sizeof(Tv) == 4) {
+          load_row<Tv, V>(w_hi + c * N + n, a[c]);
+          load_row<Tv, V>(w_lo + c * N + n, b[c]);
+        } else {
+          load_row<Tv, V>(w + c * N + n, a[c]);
+        }
       }
-    } else {
-      const bool vec_problem = sizeof(Tv) == 4 && (N & 3) == 0;
+    }
 #pragma unroll
-      for (int q = 0; q < kVecPerThread; ++q) {
-        const long long n = vec_problem ? nq + q : n0 + q * kVecThreads + threadIdx.x;
-        if (n >= n1) break;
+    for (int c = 0; c < 3; ++c) {
+      if (w_due) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) h[c * N + n] = z[c * N + n] + gam * h[c * N + n];
+        for (int j = 0; j < V; ++j) {
+          if constexpr (sizeof(Tv) == 4)
+            w_step(a[c][j], b[c][j], hv[c][j], lam_hi, lam_lo);
+          else
+            a[c][j] -= lam * hv[c][j];
+        }
+        if constexpr (sizeof(Tv) == 4) {
+          store_row<Tv, V>(w_hi + c * N + n, a[c]);
+          store_row<Tv, V>(w_lo + c * N + n, b[c]);
+        } else {
+          store_row<Tv, V>(w + c * N + n, a[c]);
+        }
+      }
+      if (DIR) {
+#pragma unroll
+        for (int j = 0; j < V; ++j) hv[c][j] = zv[c][j] + gam * hv[c][j];
+        store_row<Tv, V>(h + c * N + n, hv[c]);
       }
     }
   }
 }
 
-// w = w_hi + w_lo (FP64) for the FP64 residual replacement and the solve's output.  Gated like the
-// kernel that follows it: the residual replacement, or the final true residual of a stopped problem.
-__global__ void k_w_combine(const Prob* __restrict__ probs, const int* __restrict__ vitem_prob,
-                            const long long* __restrict__ counts, int gate) {
+// Bound: HBM and L2 (120 bytes a node in FP64, 84 mixed).
+template <typename Tv, bool ONE>
+__global__ void __launch_bounds__(kVecThreads, sizeof(Tv) == 8 ? 4 : 3)
+    k_pcg_direction(const Prob* __restrict__ probs, const int* __restrict__ vitem_prob,
+                    const long long* __restrict__ counts, const __grid_constant__ Prob one) {
+  const long long n_items = ONE ? one.n_chunks : counts[1];
+  for (long long item = blockIdx.x; item < n_items; item += gridDim.x) {
+    const Prob& P = ONE ? one : probs[vitem_prob[item]];
+    const DevState* cst = P.st;
+    if (cst->done || cst->want_check) continue;
+    const int chunk = (int)(item - P.item0_vec);
+    const long long n0 = (long long)chunk * P.chunk, n1 = min(n0 + P.chunk, P.N);
+    const Tv gam = sizeof(Tv) == 4 ? (Tv)cst->gam_f : (Tv)cst->gamma;
+    const bool w_due = !cst->w_applied;
+    if (P.N % Row<Tv>::V == 0)
+      direction_chunk<Tv, Row<Tv>::V, true>(P, n0, n1, w_due, gam);
+    else
+      direction_chunk<Tv, 1, true>(P, n0, n1, w_due, gam);
+  }
+}
+
+// Brings w up to date: the pending w -= lambda h of a problem that stopped in its update or is about
+// to have its residual replaced (a problem still running otherwise has had it from its direction),
+// and in the mixed path w = w_hi + w_lo in FP64.  Gated like the kernel that follows it: the residual
+// replacement, or the final true residual of a stopped problem.
+template <typename Tv>
+__global__ void __launch_bounds__(kVecThreads)
+    k_w_finish(const Prob* __restrict__ probs, const int* __restrict__ vitem_prob, const long long* __restrict__ counts,
+               int gate) {
   const long long n_items = counts[1];
   for (long long item = blockIdx.x; item < n_items; item += gridDim.x) {
     const Prob& P = probs[vitem_prob[item]];
@@ -452,16 +482,12 @@ __global__ void k_w_combine(const Prob* __restrict__ probs, const int* __restric
     if (gate == GATE_REPLACE && (st->done || !replacement_due(st))) continue;
     if (gate == GATE_FINALIZE && (!st->done || st->finalized)) continue;
     const int chunk = (int)(item - P.item0_vec);
-    const long long N = P.N, n0 = (long long)chunk * kVecChunk, n1 = min(n0 + kVecChunk, N);
-    double* __restrict__ w = P.w;
-    const float* __restrict__ w_hi = P.w_hi;
-    const float* __restrict__ w_lo = P.w_lo;
+    const long long N = P.N, n0 = (long long)chunk * P.chunk, n1 = min(n0 + P.chunk, N);
+    if (!st->w_applied && (gate == GATE_REPLACE || st->done)) direction_chunk<Tv, 1, false>(P, n0, n1, true, Tv(0));
+    if constexpr (sizeof(Tv) == 4) {  // a thread reads back its own nodes
+      for (long long n = n0 + threadIdx.x; n < n1; n += kVecThreads)
 #pragma unroll
-    for (int q = 0; q < kVecPerThread; ++q) {
-      const long long n = n0 + q * kVecThreads + threadIdx.x;
-      if (n >= n1) break;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) w[c * N + n] = (double)w_hi[c * N + n] + (double)w_lo[c * N + n];
+        for (int c = 0; c < 3; ++c) P.w[c * N + n] = (double)P.w_hi[c * N + n] + (double)P.w_lo[c * N + n];
     }
   }
 }
@@ -482,24 +508,27 @@ cudaError_t launch_pcg_init(const BatchDev& b, bool mixed, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// A batch of one problem passes its descriptor as an argument: its blocks start on their nodes
+// without the chain of loads item -> problem -> pointers.
 cudaError_t launch_pcg_update(const BatchDev& b, bool mixed, cudaStream_t s) {
-  if (mixed)
-    k_pcg_update_f32<<<b.vec_blocks, b.vec_threads, 0, s>>>(b.probs, b.vitem_prob, b.counts);
-  else
-    k_pcg_update_f64<<<b.vec_blocks, b.vec_threads, 0, s>>>(b.probs, b.vitem_prob, b.counts);
+  auto k = mixed ? (b.single ? k_pcg_update_f32<true> : k_pcg_update_f32<false>)
+                 : (b.single ? k_pcg_update_f64<true> : k_pcg_update_f64<false>);
+  k<<<b.vec_blocks, b.vec_threads, 0, s>>>(b.probs, b.vitem_prob, b.counts, b.one);
   return cudaGetLastError();
 }
 
 cudaError_t launch_pcg_direction(const BatchDev& b, bool mixed, cudaStream_t s) {
-  if (mixed)
-    k_pcg_direction<float><<<b.vec_blocks, b.vec_threads, 0, s>>>(b.probs, b.vitem_prob, b.counts);
-  else
-    k_pcg_direction<double><<<b.vec_blocks, b.vec_threads, 0, s>>>(b.probs, b.vitem_prob, b.counts);
+  auto k = mixed ? (b.single ? k_pcg_direction<float, true> : k_pcg_direction<float, false>)
+                 : (b.single ? k_pcg_direction<double, true> : k_pcg_direction<double, false>);
+  k<<<b.vec_blocks, b.vec_threads, 0, s>>>(b.probs, b.vitem_prob, b.counts, b.one);
   return cudaGetLastError();
 }
 
-cudaError_t launch_w_combine(const BatchDev& b, int gate, cudaStream_t s) {
-  k_w_combine<<<b.vec_blocks, b.vec_threads, 0, s>>>(b.probs, b.vitem_prob, b.counts, gate);
+cudaError_t launch_w_finish(const BatchDev& b, bool mixed, int gate, cudaStream_t s) {
+  if (mixed)
+    k_w_finish<float><<<b.vec_blocks, b.vec_threads, 0, s>>>(b.probs, b.vitem_prob, b.counts, gate);
+  else
+    k_w_finish<double><<<b.vec_blocks, b.vec_threads, 0, s>>>(b.probs, b.vitem_prob, b.counts, gate);
   return cudaGetLastError();
 }
 

@@ -109,7 +109,7 @@ Layout request_layout(const Geo& geo, int n_phases, bool mixed, const Tiling& tl
   const size_t vb = mixed ? sizeof(float) : sizeof(double);
   const size_t P = (size_t)std::max(n_phases, 1);
   Layout L{};
-  L.stride = std::max<long long>(tl.n_tiles, chunks_of(N));
+  L.stride = std::max<long long>(tl.n_tiles, chunks_of(N, mixed));
   size_t o = 0;
   auto take = [&](size_t b) {
     const size_t at = o;
@@ -180,7 +180,7 @@ int sfail(elas_server* s, int code, const std::string& m) {
 size_t table_bytes_for(size_t budget, int max_active) {
   const long long vox = (long long)(budget / 96) + 1;
   const long long cap_apply = vox / 48 + 4096LL * max_active;
-  const long long cap_vec = vox / kVecChunk + 2LL * max_active;
+  const long long cap_vec = vox / 2048 + (long long)kMoreChunks * max_active;
   return engine_table_bytes(max_active, cap_apply, cap_vec);
 }
 
@@ -209,6 +209,7 @@ int rebuild(elas_server* s) {
       ps[i].kc = 1;
       ps[i].tiles_x = ps[i].tiles_y = 1;
       ps[i].n_tiles = 0;
+      ps[i].chunk = 128;
       ps[i].n_chunks = 0;
     }
   }
@@ -263,7 +264,7 @@ int elas_server_create(elas_server** out, size_t budget_bytes, int max_active, i
   s->eng.fixed_smemff = max_tile_smem(0);
   std::string m;
   int r = engine_init(s->eng, mixed, s->sm_count, apply_max_threads(mixed ? 4 : 8), max_active,
-                      vox / 48 + 4096LL * max_active, vox / kVecChunk + 2LL * max_active, s->arena_base + s->budget,
+                      vox / 48 + 4096LL * max_active, vox / 2048 + (long long)kMoreChunks * max_active, s->arena_base + s->budget,
                       s->stream, &m);
   if (r != ELAS_OK) {
     engine_destroy(s->eng);
@@ -344,7 +345,8 @@ int elas_server_step(elas_server* s, int* n_active_out, int* n_queued, int* n_fi
     p.nx = geo.nx; p.ny = geo.ny; p.nz = geo.nz; p.N = geo.N;
     p.tx = r->tl.tx; p.ty = r->tl.ty; p.kc = r->tl.kc; p.tiles_x = r->tl.tiles_x; p.tiles_y = r->tl.tiles_y;
     p.n_tiles = (int)r->tl.n_tiles;
-    p.n_chunks = (int)chunks_of(geo.N);
+    p.chunk = vec_chunk(geo.N, mixed);
+    p.n_chunks = (int)chunks_of(geo.N, mixed);
     p.parts_stride = (int)L.stride;
     p.phase = (int32_t*)(base + L.phase);
     p.coef64 = (double*)(base + L.coef64);
@@ -408,7 +410,7 @@ int elas_server_step(elas_server* s, int* n_active_out, int* n_queued, int* n_fi
     if (rc != ELAS_OK) return sfail(s, rc, "server: " + m);
     cudaError_t e = cudaGraphLaunch(s->eng.exec, st);
     // 3. final FP64 w and true residual of the requests that stopped
-    if (e == cudaSuccess && mixed) e = launch_w_combine(s->eng.bd, GATE_FINALIZE, st);
+    if (e == cudaSuccess) e = launch_w_finish(s->eng.bd, mixed, GATE_FINALIZE, st);
     if (e == cudaSuccess) e = launch_apply(s->eng.bd, AK_F64_NORM, POST_TRUE_NORM, GATE_FINALIZE, st);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(s->eng.h_states, s->eng.d_states, sizeof(DevState) * n_slots, cudaMemcpyDeviceToHost, st);
@@ -499,9 +501,12 @@ int elas_server_cancel(elas_server* s, long long id) {
     if (!r || r->id != id) continue;
     // between steps the stream is idle: mark the solver state stopped; the next step skips its
     // iterations, forms its final w and true residual and retires it
-    const int sd[2] = {ELAS_CANCELLED, 1};  // DevState::status, DevState::done
+    // (w_applied: its last direction, the one before this call, has advanced w)
+    const int sd[3] = {ELAS_CANCELLED, 1, 1};  // DevState::status, DevState::done, DevState::w_applied
     DevState* st = s->eng.d_states + r->slot;
-    static_assert(offsetof(DevState, done) == offsetof(DevState, status) + sizeof(int), "status, done adjacent");
+    static_assert(offsetof(DevState, done) == offsetof(DevState, status) + sizeof(int) &&
+                      offsetof(DevState, w_applied) == offsetof(DevState, done) + sizeof(int),
+                  "status, done, w_applied adjacent");
     cudaError_t e = cudaMemcpyAsync(&st->status, sd, sizeof sd, cudaMemcpyHostToDevice, s->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
     if (e != cudaSuccess) return sfail(s, ELAS_ERR_CUDA, std::string("elas_server_cancel: ") + cudaGetErrorString(e));
