@@ -144,8 +144,16 @@ int grid_prepare(GridHost& g, int nx, int ny, int nz, const int32_t* phase_id, i
         g.cfull[kSymStride * p + pk(i, j)] = v;
         g.coef64[kCoefStride * p + kCoefMode0 + pk(i, j)] = v / 16.0;
         g.coef64[kCoefStride * p + kCoefMode1 + pk(i, j)] = v / 48.0;
-        g.coef64[kCoefStride * p + kCoefMode2 + pk(i, j)] = v / 144.0;
       }
+    // the bilinear modes eta zeta, xi zeta, xi eta carry the gradients [a|0|0], [0|a|0], [0|0|a] of the
+    // trilinear coefficients a: their forces on them add up to M a, M_ij = sum_d C_idjd
+    static const int dir[3][3] = {{0, 5, 4}, {5, 1, 3}, {4, 3, 2}};  // Voigt slot of the pair (i, d)
+    static const int mi[6] = {0, 1, 2, 1, 0, 0}, mj[6] = {0, 1, 2, 2, 2, 1};
+    for (int q = 0; q < 6; ++q) {
+      double m = 0.0;
+      for (int d = 0; d < 3; ++d) m += g.cfull[kSymStride * p + pk(dir[mi[q]][d], dir[mj[q]][d])];
+      g.coef64[kCoefStride * p + kCoefMode2 + q] = m / 144.0;
+    }
     g.coef64[kCoefStride * p + kCoefFlag] = solid ? 1.0 : 0.0;
     g.coef64[kCoefStride * p + kCoefMode0 + kCoefSolid0] = solid ? 1.0 : 0.0;
     // diagonal blocks of K_e for the Jacobi preconditioner (Eq. 9):

@@ -13,10 +13,12 @@
 //     eta zeta, xi zeta, xi eta} that are orthogonal on the voxel, so the element energy
 //     int eps:C:eps (Eq. 7) is a sum of 7 independent quadratic forms with weights 1, 1/12 and
 //     1/144.  The corner forces follow by the transposed transform.  This is the same K_e as
-//     the 2x2x2 Gauss integral of B^T C B (exact for trilinear elements), at 432 instead of
-//     1,152 flops per voxel (30 MUL + 108 FMA in the mode products, 186 adds).
-//   * Per-phase coefficients are the sample-frame stiffness scaled by 1/16, 1/48 and 1/144
-//     (the products of the transform scalings and mode weights), built on the host in FP64.
+//     the 2x2x2 Gauss integral of B^T C B (exact for trilinear elements), at 396 instead of
+//     1,152 flops per voxel (24 MUL + 96 FMA in the mode products, 180 adds): the three bilinear
+//     modes share one vector of coefficients, so their three products fold into one 3x3 block.
+//   * Per-phase coefficients are the sample-frame stiffness scaled by 1/16 and 1/48 and the folded
+//     bilinear block scaled by 1/144 (the products of the transform scalings and mode weights),
+//     built on the host in FP64.
 //   * Periodic wrap (Eq. 1) is applied when node layers are staged into shared memory.
 //   * Node sums are gathered in a fixed order and block partial sums are combined in a fixed
 //     order by the last block to finish, so every result is bitwise reproducible.
@@ -168,6 +170,45 @@ __device__ __forceinline__ void symv(const LazyK& k, const ff (&e)[6], ff (&s)[6
   symv_ff<MASK>(k, e, s);
 }
 
+// s = M e for a symmetric 3x3 block M (11, 22, 33, 23, 13, 12); the double-float rows are compensated
+// dot products as above.
+__device__ constexpr int pm(int i, int j) { return i == j ? i : 6 - i - j; }
+template <typename T>
+__device__ __forceinline__ void sym3(const T (&m)[6], const T (&e)[3], T (&s)[3]) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i) s[i] = fma(m[pm(i, 2)], e[2], fma(m[pm(i, 1)], e[1], m[pm(i, 0)] * e[0]));
+}
+__device__ __forceinline__ void sym3(const LazyK& m, const ff (&e)[3], ff (&s)[3]) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    float hi = 0.f, lo = 0.f;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const ff a = m[pm(i, j)], b = e[j];
+      const float p = __fmul_rn(a.hi, b.hi);
+      float pe = fmaf(a.hi, b.hi, -p);
+      pe = fmaf(a.hi, b.lo, pe);
+      pe = fmaf(a.lo, b.hi, pe);
+      if (j == 0) {
+        hi = p;
+        lo = pe;
+      } else {
+        float t;
+        hi = two_sum(hi, p, t);
+        lo = __fadd_rn(lo, __fadd_rn(t, pe));
+      }
+    }
+    s[i] = ff_norm(hi, lo);
+  }
+}
+__device__ __forceinline__ void load_m(const double* __restrict__ K, double (&m)[6]) {
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const double2 v = __ldg(reinterpret_cast<const double2*>(K) + q);
+    m[2 * q] = v.x; m[2 * q + 1] = v.y;
+  }
+}
+
 // 24 consecutive coefficients (16-byte aligned) through the read-only path as vectors.
 __device__ __forceinline__ void load_k(const float* __restrict__ K, float (&k)[24]) {
   const float4* K4 = reinterpret_cast<const float4*>(K);
@@ -257,8 +298,8 @@ __device__ __forceinline__ double lane1(P2<double> a) { return a.y; }
 __device__ __forceinline__ ff lane0(P2<ff> a) { return ff(a.hi.x, a.lo.x); }
 __device__ __forceinline__ ff lane1(P2<ff> a) { return ff(a.hi.y, a.lo.y); }
 
-// (x, y, z, 4th) shared-memory records: float [x y z id], double [x y | z id], double-float
-// [x.hi y.hi x.lo y.lo | z.hi z.lo id -]; the 4th element holds a phase id in the node ring
+// (x, y, z, 4th) shared-memory records: float [x y z id], double [x y | z id]; the 4th element holds a
+// phase id in the node ring.  Double-float nodes: planes of [x.hi y.hi x.lo y.lo] and [z.hi z.lo].
 __device__ __forceinline__ void ld_xyz(const float* p, P2<float>& xy, float& z) {
   const float4 v = *reinterpret_cast<const float4*>(p);
   xy.v = make_float2(v.x, v.y);
@@ -269,12 +310,15 @@ __device__ __forceinline__ void ld_xyz(const double* p, P2<double>& xy, double& 
   xy = {a.x, a.y};
   z = p[2];
 }
-__device__ __forceinline__ void ld_xyz(const ff* p, P2<ff>& xy, ff& z) {
-  const float4 a = *reinterpret_cast<const float4*>(p);
-  const float2 b = *reinterpret_cast<const float2*>(p + 2);
+__device__ __forceinline__ void ld_node_ff(const float4* pxy, const float2* pz, P2<ff>& xy, ff& z) {
+  const float4 a = *pxy;
+  const float2 b = *pz;
   xy = {make_float2(a.x, a.y), make_float2(a.z, a.w)};
   z = ff(b.x, b.y);
 }
+// (never called for the other arithmetics)
+template <typename P, typename T>
+__device__ __forceinline__ void ld_node_ff(const float4*, const float2*, P&, T&) {}
 __device__ __forceinline__ void st_xyz(float* p, P2<float> xy, float z) {
   *reinterpret_cast<float4*>(p) = make_float4(xy.v.x, xy.v.y, z, 0.f);
 }
@@ -282,11 +326,6 @@ __device__ __forceinline__ void st_xyz(double* p, P2<double> xy, double z) {
   *reinterpret_cast<double2*>(p) = make_double2(xy.x, xy.y);
   p[2] = z;
 }
-__device__ __forceinline__ void st_xyz(ff* p, P2<ff> xy, ff z) {
-  *reinterpret_cast<float4*>(p) = make_float4(xy.hi.x, xy.hi.y, xy.lo.x, xy.lo.y);
-  *reinterpret_cast<float2*>(p + 2) = make_float2(z.hi, z.lo);
-}
-
 // the butterflies of one face: corners b = ax + 2 ay -> face modes q = mx + 2 my (any lane type)
 template <typename L>
 __device__ __forceinline__ void face_bf(const L& c0, const L& c1, const L& c2, const L& c3, L (&V)[4]) {
@@ -320,12 +359,22 @@ __device__ __forceinline__ void face_forward(const T* face, int row, P2<T> (&Vxy
   face_bf(cz[0], cz[1], cz[2], cz[3], Vz);
 }
 
+// the double-float form: pxy, pz point at corner 0 in the planes, row: records per row
+template <typename T>
+__device__ __forceinline__ void face_forward_ff(const float4* pxy, const float2* pz, int row, P2<T> (&Vxy)[4], T (&Vz)[4]) {
+  P2<T> cxy[4];
+  T cz[4];
+#pragma unroll
+  for (int b = 0; b < 4; ++b) ld_node_ff(pxy + (b >> 1) * row + (b & 1), pz + (b >> 1) * row + (b & 1), cxy[b], cz[b]);
+  face_bf(cxy[0], cxy[1], cxy[2], cxy[3], Vxy);
+  face_bf(cz[0], cz[1], cz[2], cz[3], Vz);
+}
+
 // Modal element forces F[c][m] (m = 1..7; F[c][0] = 0) from the mode coefficients W[c][m]:
 // seven orthogonal gradient monomials, each a symmetric-stiffness product (see file header).
-// k0 holds the C/16 block (already loaded).  FP64 reads the C/48 and C/144 blocks as well; FP32
-// instead scales the linear-mode coefficients by 1/3 and the trilinear one by 1/9 and uses C/16
-// for all seven products (C/48 e = C/16 (e/3)), which trades 12 multiplies for 12 of the 18
-// vector loads of the coefficient blocks.
+// k0 holds the C/16 block (already loaded).  FP64 reads the C/48 block as well; FP32 instead scales
+// the linear-mode coefficients by 1/3 and uses C/16 for them too (C/48 e = C/16 (e/3)), which trades
+// 9 multiplies for 6 vector loads of the coefficient blocks.  The bilinear block is read by all.
 template <typename T, typename K0>
 __device__ __forceinline__ void modal_forces(T (&W)[3][8], const K0& k0, const T* __restrict__ K,
                                              T (&F)[3][8]) {
@@ -360,23 +409,13 @@ __device__ __forceinline__ void modal_forces(T (&W)[3][8], const K0& k0, const T
       F[0][6] += s[5]; F[1][6] += s[1]; F[2][6] += s[3];
     }
   };
-  // bilinear modes: eta zeta -> [A_xyz|0|0], xi zeta -> [0|A_xyz|0], xi eta -> [0|0|A_xyz]
-  auto bilinear_modes = [&](const auto& k2) {
-    {
-      const T e[6] = {W[0][7], T(0), T(0), T(0), W[2][7], W[1][7]};
-      symv<0x31>(k2, e, s);
-      F[0][7] = s[0]; F[1][7] = s[5]; F[2][7] = s[4];
-    }
-    {
-      const T e[6] = {T(0), W[1][7], T(0), W[2][7], T(0), W[0][7]};
-      symv<0x2a>(k2, e, s);
-      F[0][7] += s[5]; F[1][7] += s[1]; F[2][7] += s[3];
-    }
-    {
-      const T e[6] = {T(0), T(0), W[2][7], W[1][7], W[0][7], T(0)};
-      symv<0x1c>(k2, e, s);
-      F[0][7] += s[4]; F[1][7] += s[3]; F[2][7] += s[2];
-    }
+  // bilinear modes: eta zeta -> [A_xyz|0|0], xi zeta -> [0|A_xyz|0], xi eta -> [0|0|A_xyz], all
+  // three by the combined block
+  auto bilinear_modes = [&](const auto& m) {
+    const T e[3] = {W[0][7], W[1][7], W[2][7]};
+    T r[3];
+    sym3(m, e, r);
+    F[0][7] = r[0]; F[1][7] = r[1]; F[2][7] = r[2];
   };
   if constexpr (f32) {
     const T third = T(1.0 / 3.0), ninth = T(1.0 / 9.0);
@@ -388,7 +427,11 @@ __device__ __forceinline__ void modal_forces(T (&W)[3][8], const K0& k0, const T
       W[c][7] *= ninth;
     }
     linear_modes(k0);
-    bilinear_modes(k0);
+    // the combined block from the C/16 entries at hand: 12 additions instead of two more loads
+    const T m[6] = {k0[pk(0, 0)] + (k0[pk(5, 5)] + k0[pk(4, 4)]), k0[pk(1, 1)] + (k0[pk(5, 5)] + k0[pk(3, 3)]),
+                    k0[pk(2, 2)] + (k0[pk(4, 4)] + k0[pk(3, 3)]), k0[pk(4, 5)] + (k0[pk(1, 3)] + k0[pk(2, 3)]),
+                    k0[pk(0, 4)] + (k0[pk(3, 5)] + k0[pk(2, 4)]), k0[pk(0, 5)] + (k0[pk(1, 5)] + k0[pk(3, 4)])};
+    bilinear_modes(m);
   } else if constexpr (lazy) {
     linear_modes(LazyK{K + CoefOf<T>::m1});
     bilinear_modes(LazyK{K + CoefOf<T>::m2});
@@ -396,8 +439,9 @@ __device__ __forceinline__ void modal_forces(T (&W)[3][8], const K0& k0, const T
     T kb[24];
     load_k(K + CoefOf<T>::m1, kb);
     linear_modes(kb);
-    load_k(K + CoefOf<T>::m2, kb);
-    bilinear_modes(kb);
+    T km[6];
+    load_m(K + CoefOf<T>::m2, km);
+    bilinear_modes(km);
   }
 #pragma unroll
   for (int c = 0; c < 3; ++c) F[c][0] = T(0);
@@ -419,6 +463,16 @@ __device__ __forceinline__ void ld_face_ff(const ff* Fc, int NV, int r, P2<ff>& 
   xy = {make_float2(a.x, a.y), make_float2(a.z, a.w)};
   z = ff(b.x, b.y);
 }
+// Exact split of a double into its leading float and the float nearest the remainder, as ff(double),
+// but with the leading part rounded in integer arithmetic (the bits below a float's 24 are rounded to
+// nearest and cleared): 3 instead of 4 operations on the FP64 pipe, which all warps' splits share
+// (100^3 product 140 -> 137 us).  Leading parts beyond the float range become infinite, as there.
+__device__ __forceinline__ ff split_double(double v) {
+  const double h = __longlong_as_double((__double_as_longlong(v) + (1LL << 28)) & ~((1LL << 29) - 1));
+  return ff(__double2float_rn(h), __double2float_rn(v - h));
+}
+// bytes of the double-float node ring of NP-record layers (a multiple of 16)
+__host__ __device__ constexpr size_t ff_ring_bytes(int NP) { return ((size_t)kRing * NP * 28 + 15) / 16 * 16; }
 // the same helpers for the other forms are never called (their records stay 4-wide)
 template <typename T, typename P>
 __device__ __forceinline__ void st_face_ff(T*, int, int, const P&, T) {}
@@ -526,8 +580,15 @@ __global__ void __launch_bounds__(MAXT, MINB)
     const int NXv = tx + 1, NV = (tx + 1) * (ty + 1);
     const int NXp = tx + 2, NP = (tx + 2) * (ty + 2);
     constexpr int RS = 4;                       // elements per node record
-    T* ring = reinterpret_cast<T*>(smem_raw);  // [kRing][NP][RS]
-    T* Fc = ring + kRing * NP * RS;             // [2][4 corners][NV][4] (double-float: compact, below)
+    // node ring [kRing][NP][RS]; double-float: planes of (x, y) records of 16 bytes, z records of 8 and
+    // ids of 4, so that neighbouring threads touch neighbouring addresses (records of 32 bytes cost
+    // 4-way bank conflicts: 128 of 288 shared-memory wavefronts per warp and layer)
+    T* ring = reinterpret_cast<T*>(smem_raw);
+    float4* const rxy = reinterpret_cast<float4*>(smem_raw);
+    float2* const rz = reinterpret_cast<float2*>(rxy + kRing * NP);
+    int* const rid = reinterpret_cast<int*>(rz + kRing * NP);
+    // face forces [2][4 corners][NV][4] (double-float: compact, below)
+    T* Fc = kFF ? reinterpret_cast<T*>(smem_raw + ff_ring_bytes(NP)) : ring + kRing * NP * RS;
     const long long plane = (long long)nx * ny;
     const int32_t* __restrict__ phase = P.phase;
     const T* __restrict__ coef = CoefOf<T>::table(P) + CoefOf<T>::base;
@@ -585,9 +646,11 @@ __global__ void __launch_bounds__(MAXT, MINB)
     for (int r = 0; r < 3; ++r) {
       const int sl = t + r * (int)blockDim.x;
       soff[r] = sl < NP ? wrapi(j0 - 1 + sl / NXp, ny) * nx + wrapi(i0 - 1 + sl % NXp, nx) : -1;
-      srec[r] = (unsigned)__cvta_generic_to_shared(ring + RS * (sl < NP ? sl : 0));
+      srec[r] = kFF ? (unsigned)(sl < NP ? sl : 0) : (unsigned)__cvta_generic_to_shared(ring + RS * (sl < NP ? sl : 0));
     }
     const unsigned slot_bytes = (unsigned)(NP * RS * sizeof(T));
+    const unsigned sxy = (unsigned)__cvta_generic_to_shared(rxy), sz = (unsigned)__cvta_generic_to_shared(rz);
+    const unsigned sid = (unsigned)__cvta_generic_to_shared(rid);
     const Tin* __restrict__ u1 = u + N;
     const Tin* __restrict__ u2 = u + 2 * N;
     // the layers are staged in order from k0 - 1: the offset of the next one, wrapped periodically
@@ -601,11 +664,19 @@ __global__ void __launch_bounds__(MAXT, MINB)
       for (int r = 0; r < 3; ++r) {
         if (soff[r] < 0) break;
         const int e = kofs + soff[r];
-        const unsigned d = srec[r] + sb;
-        cp_async_to(d, u + e);
-        cp_async_to(d + sizeof(T), u1 + e);
-        cp_async_to(d + 2 * sizeof(T), u2 + e);
-        cp_async_to(d + 3 * sizeof(T), phase + e);
+        if constexpr (kFF) {
+          const unsigned d = srec[r] + (unsigned)(b * NP);
+          cp_async_to(sxy + 16 * d, u + e);
+          cp_async_to(sxy + 16 * d + 8, u1 + e);
+          cp_async_to(sz + 8 * d, u2 + e);
+          cp_async_to(sid + 4 * d, phase + e);
+        } else {
+          const unsigned d = srec[r] + sb;
+          cp_async_to(d, u + e);
+          cp_async_to(d + sizeof(T), u1 + e);
+          cp_async_to(d + 2 * sizeof(T), u2 + e);
+          cp_async_to(d + 3 * sizeof(T), phase + e);
+        }
       }
       cp_async_commit();
       kofs_next = kofs + (int)plane < (int)N ? kofs + (int)plane : kofs + (int)plane - (int)N;
@@ -616,6 +687,7 @@ __global__ void __launch_bounds__(MAXT, MINB)
     const T* const face0 = ring + RS * (vj * NXp + vi);
     const int row = RS * NXp, slot_elems = NP * RS, fbuf = 4 * NV * 4;
     const T* const hrec0 = ring + RS * ((nj + 1) * NXp + ni + 1);
+    const int face_rec = vj * NXp + vi, own_rec = (nj + 1) * NXp + ni + 1;  // (double-float planes)
     T* const fcol = Fc + 4 * vcol;
     int goff[4];
 #pragma unroll
@@ -627,15 +699,17 @@ __global__ void __launch_bounds__(MAXT, MINB)
     // records' doubles into float pairs in place (before the barrier that publishes the slot)
     auto split_slot = [&](int b) {
       if constexpr (kFF) {
-        T* dst = ring + b * NP * RS;
 #pragma unroll
         for (int r = 0; r < 3; ++r) {
           if (soff[r] < 0) break;
-          T* rec = dst + RS * (t + r * (int)blockDim.x);
-          const double* d = reinterpret_cast<const double*>(rec);
-          const double v0 = d[0], v1 = d[1], v2 = d[2];
+          float4* xy = rxy + b * NP + t + r * (int)blockDim.x;
+          float2* z = rz + b * NP + t + r * (int)blockDim.x;
+          const double2 vxy = *reinterpret_cast<const double2*>(xy);
+          const double vz = *reinterpret_cast<const double*>(z);
           asm volatile("" ::: "memory");  // the pairs overwrite the doubles they are made from
-          st_xyz(rec, pk2(T(v0), T(v1)), T(v2));
+          const ff px = split_double(vxy.x), py = split_double(vxy.y), pz = split_double(vz);
+          *xy = make_float4(px.hi, py.hi, px.lo, py.lo);
+          *z = make_float2(pz.hi, pz.lo);
         }
       }
     };
@@ -692,6 +766,12 @@ __global__ void __launch_bounds__(MAXT, MINB)
             st_xyz(fcol + buf * fbuf + b * 4 * NV, zxy, T(0));
         }
     }
+    // Double-float: the second half of the busy warps takes a layer's two halves in the other order, so
+    // that one half's splits, gathers and stores (20 FP64-pipe operations a node) run beside the other's
+    // element products on the FP32 pipe.  With all warps in one order they queued for the FP64 pipe
+    // right after every barrier (short-scoreboard stalls 0.83 of 5.9 cycles per instruction, 0.21 now):
+    // 100^3 product 160 -> 139 us.  The native FP64 and FP32 forms have no such pair of pipes to overlap.
+    const bool late = t >= (NV + 63) / 64 * 32;
     T hown[3] = {T(0), T(0), T(0)};  // the owned node's operand on the previous layer (h.Ah)
     for (int kv = k0 - 1; kv <= k1; ++kv) {
       const int L = kv - k0 + 1;
@@ -700,6 +780,9 @@ __global__ void __launch_bounds__(MAXT, MINB)
         stage((L + kAhead) % kRing);  // prefetch layer kv + kAhead: overlaps the next layers' arithmetic
       else
         cp_async_commit();
+      // the layer's two independent halves: (gather) split layer kv+2 and gather layer kv-1 from the face
+      // forces, (compute) the element products of voxel layer kv
+      auto gather_half = [&]() {
       cp_async_wait_ahead();  // this thread's copies of layer kv+2 have landed
       if (kFF && kv + 2 <= k1) split_slot((L + 2) % kRing);
       if (kv > k0 && has_node) {
@@ -749,15 +832,36 @@ __global__ void __launch_bounds__(MAXT, MINB)
           for (int c = 0; c < 3; ++c) dot1.add((double)out[c], (double)out[c]);
         }
       }
+      if (EPI == EPI_STORE_DOT && kv < k1 && has_node) {
+        P2<T> hxy;
+        if constexpr (kFF)
+          ld_node_ff(rxy + (L % kRing) * NP + own_rec, rz + (L % kRing) * NP + own_rec, hxy, hown[2]);
+        else
+          ld_xyz(hrec0 + (L % kRing) * slot_elems, hxy, hown[2]);
+        hown[0] = lane0(hxy);
+        hown[1] = lane1(hxy);
+      }
+      };
+      auto compute_half = [&]() {
       if (kv < k1 && has_vox && own_col) {
         const bool own = own_col;
-        if (L == 0) face_forward<RS>(face0, row, Vlo_xy, Vlo_z);
         P2<T> Vup_xy[4];
         T Vup_z[4];
-        face_forward<RS>(face0 + ((L + 1) % kRing) * slot_elems, row, Vup_xy, Vup_z);
+        if constexpr (kFF) {
+          if (L == 0) face_forward_ff(rxy + face_rec, rz + face_rec, NXp, Vlo_xy, Vlo_z);
+          const int at = ((L + 1) % kRing) * NP + face_rec;
+          face_forward_ff(rxy + at, rz + at, NXp, Vup_xy, Vup_z);
+        } else {
+          if (L == 0) face_forward<RS>(face0, row, Vlo_xy, Vlo_z);
+          face_forward<RS>(face0 + ((L + 1) % kRing) * slot_elems, row, Vup_xy, Vup_z);
+        }
         P2<T> FL_xy[4], FU_xy[4];
         T FL_z[4], FU_z[4];
-        const int ph = own ? *reinterpret_cast<const int*>(face0 + (L % kRing) * slot_elems + 3) : -1;
+        int ph = -1;
+        if constexpr (kFF)
+          ph = rid[(L % kRing) * NP + face_rec];
+        else if (own)
+          ph = *reinterpret_cast<const int*>(face0 + (L % kRing) * slot_elems + 3);
         const T* K = ph >= 0 ? coef + (long long)ph * CoefOf<T>::stride : nullptr;
         T k0[24];
         bool solid = false;
@@ -885,11 +989,18 @@ __global__ void __launch_bounds__(MAXT, MINB)
           }
         }
       }
-      if (EPI == EPI_STORE_DOT && kv < k1 && has_node) {
-        P2<T> hxy;
-        ld_xyz(hrec0 + (L % kRing) * slot_elems, hxy, hown[2]);
-        hown[0] = lane0(hxy);
-        hown[1] = lane1(hxy);
+      };
+      if constexpr (kFF) {
+#pragma unroll 1
+        for (int half = 0; half < 2; ++half) {
+          if ((half == 0) != late)
+            gather_half();
+          else
+            compute_half();
+        }
+      } else {
+        gather_half();
+        compute_half();
       }
       if (kv > k0) nrow += (int)plane;
     }
@@ -1098,9 +1209,9 @@ size_t apply_smem_bytes(int tx, int ty, int elem_bytes) {
 
 size_t apply_smem_bytes_ff(int tx, int ty) {
   const size_t NP = (size_t)(tx + 2) * (ty + 2), NV = (size_t)(tx + 1) * (ty + 1);
-  // node ring (double records, split in place), 2 compact face-force buffers (24 bytes a record),
+  // node ring (28 bytes a record, the doubles split in place), 2 compact face-force buffers (24 bytes a record),
   // the per-thread slots of the carried face forces
-  return 4 * kRing * NP * sizeof(double) + 2 * 4 * NV * 24 + kFupSlotBytes;
+  return ff_ring_bytes((int)NP) + 2 * 4 * NV * 24 + kFupSlotBytes;
 }
 
 Tiling make_tiling(const Geo& g, int elem_bytes, int sm_count, int tx_hint, int ty_hint, int kc_hint) {
