@@ -14,12 +14,14 @@
 namespace elas {
 
 // ------------------------------------------------------------------------------------------
-// Per-phase coefficient block (device): the three scaled copies of the sample-frame Voigt
-// stiffness used by the modal element product, packed symmetric (21 entries each, each copy
-// starting on a 32-entry boundary so it loads as aligned vectors):
+// Per-phase coefficient block (device): the scaled copies of the sample-frame Voigt stiffness used
+// by the modal element product, packed symmetric (21 entries each, each copy starting on a 32-entry
+// boundary so it loads as aligned vectors):
 //   [0,21)   C/16   constant-strain mode
 //   [32,53)  C/48   the three linear modes
-//   [64,85)  C/144  the three bilinear modes
+//   [64,70)  M/144  the three bilinear modes together: they share the trilinear coefficients, so
+//                   their forces are one symmetric 3x3 matrix M (11, 22, 33, 23, 13, 12) times them,
+//                   9 products instead of 27
 //   [96]     1 if the phase is solid, 0 for a pore
 // plus, in a separate table, the unscaled C (21 entries) for stress and Jacobi.
 // ------------------------------------------------------------------------------------------
@@ -321,17 +323,22 @@ struct Geo {
 // ------------------------------------------------------------------------------------------
 constexpr int kVecThreads = 256;                    // block size of the vector kernels
 // Nodes per vector-kernel work item, by the grid's size and precision alone (so a problem's sums do
-// not depend on its batch): the grid's nodes are split evenly over whole waves of resident blocks
+// not depend on its batch).  The grid's nodes are split evenly over whole waves of resident blocks
 // (four a SM in FP64, three mixed), because an uneven split leaves the last wave nearly empty (977
 // items of 1,024 nodes over 608 resident blocks took 246 us per FP64 iteration at 100^3, 607 of 1,648
-// 237; mixed 71 and 65).  At most 4,096 nodes an item, at least
-// 256 (128 in FP64, whose nodes must spread over the SMs' FP64 pipes), in whole rows of 4.
-constexpr long long kVecWave64 = 152 * 4, kVecWave32 = 152 * 3;
+// 237; mixed 71 and 65).  Smaller grids take fewer blocks a SM rather than blocks with idle threads,
+// whose per-item cost a batch of small problems pays in full (mixed items of 256 nodes made a batch
+// of 32^3 and 48^3 cells 10% slower); the smallest FP64 grids are spread over the SMs' FP64 pipes all
+// the same.  At most 4,096 nodes an item, in whole rows of 4.
+constexpr long long kVecSms = 152;
 constexpr int vec_chunk(long long N, bool mixed) {
-  const long long wave = mixed ? kVecWave32 : kVecWave64, least = mixed ? 256 : 128;
-  const long long waves = (N + wave * 4096 - 1) / (wave * 4096);
-  const long long c = ((N + wave * waves - 1) / (wave * waves) + 3) / 4 * 4;
-  return (int)(c < least ? least : c);
+  const long long full = mixed ? 768 : 512;  // (nearly) every thread holds a row
+  for (int per = mixed ? 3 : 4; per >= 1; --per) {
+    const long long wave = kVecSms * per, waves = (N + wave * 4096 - 1) / (wave * 4096);
+    const long long c = ((N + wave * waves - 1) / (wave * waves) + 3) / 4 * 4;
+    if (c >= full) return (int)c;
+  }
+  return mixed ? (int)full : N >= (1 << 16) ? 512 : N >= (1 << 14) ? 256 : 128;
 }
 constexpr int kPartsSlots = 3;
 
