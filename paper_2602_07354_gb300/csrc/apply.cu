@@ -316,9 +316,12 @@ __device__ __forceinline__ void ld_node_ff(const float4* pxy, const float2* pz, 
   xy = {make_float2(a.x, a.y), make_float2(a.z, a.w)};
   z = ff(b.x, b.y);
 }
-// (never called for the other arithmetics)
-template <typename P, typename T>
-__device__ __forceinline__ void ld_node_ff(const float4*, const float2*, P&, T&) {}
+__device__ __forceinline__ void ld_node_ff(const float2* pxy, const float* pz, P2<float>& xy, float& z) {
+  xy.v = *pxy;
+  z = *pz;
+}
+// (never called for native FP64)
+__device__ __forceinline__ void ld_node_ff(const float2*, const float*, P2<double>&, double&) {}
 __device__ __forceinline__ void st_xyz(float* p, P2<float> xy, float z) {
   *reinterpret_cast<float4*>(p) = make_float4(xy.v.x, xy.v.y, z, 0.f);
 }
@@ -359,9 +362,9 @@ __device__ __forceinline__ void face_forward(const T* face, int row, P2<T> (&Vxy
   face_bf(cz[0], cz[1], cz[2], cz[3], Vz);
 }
 
-// the double-float form: pxy, pz point at corner 0 in the planes, row: records per row
-template <typename T>
-__device__ __forceinline__ void face_forward_ff(const float4* pxy, const float2* pz, int row, P2<T> (&Vxy)[4], T (&Vz)[4]) {
+// the form with planes: pxy, pz point at corner 0, row: records per row
+template <typename T, typename Rxy, typename Rz>
+__device__ __forceinline__ void face_forward_ff(const Rxy* pxy, const Rz* pz, int row, P2<T> (&Vxy)[4], T (&Vz)[4]) {
   P2<T> cxy[4];
   T cz[4];
 #pragma unroll
@@ -450,9 +453,17 @@ __device__ __forceinline__ void modal_forces(T (&W)[3][8], const K0& k0, const T
 // ---- the tile kernel --------------------------------------------------------------------------
 // elements of one face-force buffer: 4 corners x NV columns x 4-wide records
 __host__ __device__ constexpr int fbuf_elems(int NV) { return 4 * NV * 4; }
-// Double-float face-force records, compact: record r (= buffer x 4 NV + corner x NV + column) keeps
-// its x and y pairs (x.hi, y.hi, x.lo, y.lo) at pair offset 2 r and its z pair at 16 NV + r (both
-// buffers' xy parts first), 24 bytes a record instead of a padded 32.
+// Double-float and FP32 face-force records, compact: record r (= buffer x 4 NV + corner x NV + column)
+// keeps its x and y (pairs: x.hi, y.hi, x.lo, y.lo) at element offset 2 r and its z at 16 NV + r (both
+// buffers' xy parts first), 3 elements a record instead of a padded 4.
+__device__ __forceinline__ void st_face_ff(float* Fc, int NV, int r, const P2<float>& xy, float z) {
+  *reinterpret_cast<float2*>(Fc + 2 * r) = xy.v;
+  Fc[16 * NV + r] = z;
+}
+__device__ __forceinline__ void ld_face_ff(const float* Fc, int NV, int r, P2<float>& xy, float& z) {
+  xy.v = *reinterpret_cast<const float2*>(Fc + 2 * r);
+  z = Fc[16 * NV + r];
+}
 __device__ __forceinline__ void st_face_ff(ff* Fc, int NV, int r, const P2<ff>& xy, ff z) {
   *reinterpret_cast<float4*>(Fc + 2 * r) = make_float4(xy.hi.x, xy.hi.y, xy.lo.x, xy.lo.y);
   *reinterpret_cast<float2*>(Fc + 16 * NV + r) = make_float2(z.hi, z.lo);
@@ -471,13 +482,14 @@ __device__ __forceinline__ ff split_double(double v) {
   const double h = __longlong_as_double((__double_as_longlong(v) + (1LL << 28)) & ~((1LL << 29) - 1));
   return ff(__double2float_rn(h), __double2float_rn(v - h));
 }
-// bytes of the double-float node ring of NP-record layers (a multiple of 16)
-__host__ __device__ constexpr size_t ff_ring_bytes(int NP) { return ((size_t)kRing * NP * 28 + 15) / 16 * 16; }
-// the same helpers for the other forms are never called (their records stay 4-wide)
-template <typename T, typename P>
-__device__ __forceinline__ void st_face_ff(T*, int, int, const P&, T) {}
-template <typename T, typename P>
-__device__ __forceinline__ void ld_face_ff(const T*, int, int, P&, T&) {}
+// bytes of the node ring of NP-record layers kept as planes: three components of eb bytes and an id
+// (a multiple of 16)
+__host__ __device__ constexpr size_t plane_ring_bytes(int NP, size_t eb) {
+  return ((size_t)kRing * NP * (3 * eb + 4) + 15) / 16 * 16;
+}
+// the same helpers for native FP64 are never called (its records stay 4-wide)
+__device__ __forceinline__ void st_face_ff(double*, int, int, const P2<double>&, double) {}
+__device__ __forceinline__ void ld_face_ff(const double*, int, int, P2<double>&, double&) {}
 
 __device__ __forceinline__ bool gate_skips(int gate, const DevState* st) {
   if (gate == GATE_RUNNING) return st->done || st->want_check;
@@ -557,10 +569,11 @@ __device__ void post_scalars(DevState* st, int post, double s0, double s1) {
 // for in the layer that uses them, and two buffers of per-column face corner forces
 // ([corner][column] records).  One barrier per layer.  Each item publishes its own partial sums;
 // the problem's last item sums them in tile order.
-template <typename Tin, typename T, typename Tvec, int EPI, bool AFFINE, int MAXT, int MINB, bool NOHALO = false>
+template <typename Tin, typename T, typename Tvec, int EPI, bool AFFINE, int MAXT, int MINB, bool NOHALO = false,
+          bool ONE = false>
 __global__ void __launch_bounds__(MAXT, MINB)
     k_apply(const Prob* __restrict__ probs, const int* __restrict__ item_prob, const long long* __restrict__ counts,
-            int role, int post, int gate) {
+            int role, int post, int gate, const __grid_constant__ Prob one) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double red[32];
   __shared__ int s_last;
@@ -568,11 +581,14 @@ __global__ void __launch_bounds__(MAXT, MINB)
   // double-float arithmetic: node layers arrive as doubles and are split into pairs in place
   constexpr bool kFF = std::is_same<T, ff>::value;
   using Tst = typename std::conditional<kFF, double, T>::type;  // type of the stored products
+  constexpr bool kPlanes = kFF || std::is_same<T, float>::value;  // node ring and face forces as planes
+  using Rxy = typename std::conditional<kFF, float4, float2>::type;
+  using Rz = typename std::conditional<kFF, float2, float>::type;
   const int t = threadIdx.x;
-  const long long n_items = counts[0];
+  const long long n_items = ONE ? one.n_tiles : counts[0];
 
   for (long long item = blockIdx.x; item < n_items; item += gridDim.x) {
-    const Prob& P = probs[item_prob[item]];
+    const Prob& P = ONE ? one : probs[item_prob[item]];
     if (gate != GATE_NONE && gate_skips(gate, P.st)) continue;  // uniform over the block
     const int nx = P.nx, ny = P.ny, nz = P.nz;
     const long long N = P.N;
@@ -580,15 +596,17 @@ __global__ void __launch_bounds__(MAXT, MINB)
     const int NXv = tx + 1, NV = (tx + 1) * (ty + 1);
     const int NXp = tx + 2, NP = (tx + 2) * (ty + 2);
     constexpr int RS = 4;                       // elements per node record
-    // node ring [kRing][NP][RS]; double-float: planes of (x, y) records of 16 bytes, z records of 8 and
-    // ids of 4, so that neighbouring threads touch neighbouring addresses (records of 32 bytes cost
-    // 4-way bank conflicts: 128 of 288 shared-memory wavefronts per warp and layer)
+    // node ring: native FP64 [kRing][NP][RS]; FP32 and double-float: planes of (x, y) records, z records
+    // and ids, so that neighbouring threads touch neighbouring addresses (double-float records of 32
+    // bytes cost 4-way bank conflicts: 128 of 288 shared-memory wavefronts per warp and layer; FP32
+    // records of 16 bytes made the 4-byte staging copies conflict; with the coefficients kept below, 152 ->
+    // 108 wavefronts, 200^3 product 230 -> 208 us)
     T* ring = reinterpret_cast<T*>(smem_raw);
-    float4* const rxy = reinterpret_cast<float4*>(smem_raw);
-    float2* const rz = reinterpret_cast<float2*>(rxy + kRing * NP);
+    Rxy* const rxy = reinterpret_cast<Rxy*>(smem_raw);
+    Rz* const rz = reinterpret_cast<Rz*>(rxy + kRing * NP);
     int* const rid = reinterpret_cast<int*>(rz + kRing * NP);
-    // face forces [2][4 corners][NV][4] (double-float: compact, below)
-    T* Fc = kFF ? reinterpret_cast<T*>(smem_raw + ff_ring_bytes(NP)) : ring + kRing * NP * RS;
+    // face forces [2][4 corners][NV][4] (FP32 and double-float: compact, below)
+    T* Fc = kPlanes ? reinterpret_cast<T*>(smem_raw + plane_ring_bytes(NP, sizeof(T))) : ring + kRing * NP * RS;
     const long long plane = (long long)nx * ny;
     const int32_t* __restrict__ phase = P.phase;
     const T* __restrict__ coef = CoefOf<T>::table(P) + CoefOf<T>::base;
@@ -605,7 +623,6 @@ __global__ void __launch_bounds__(MAXT, MINB)
     DotAcc<T> dot0;       // h.Ah (the product's own precision, compensated in FP32)
     DotAcc<double> dot1;  // r.r of the FP64 residual variants
     DotAcc<double> dot0r; // z.g of the residual replacement
-    const int ni = t % tx, nj = t / tx;
     // voxel column of this thread; NOHALO puts the tile's own columns (1..tx x 1..ty) on the
     // first threads and the halo columns (row 0, then column 0) on the last ones, so that whole
     // warps of halo columns skip the element product
@@ -622,6 +639,10 @@ __global__ void __launch_bounds__(MAXT, MINB)
       vj = hh <= tx ? 0 : hh - tx;
     }
     const int vcol = vi + NXv * vj;  // the column's slot in the face-force buffer
+    // node of this thread: with planes the one at its column's low corner, so that the column's records
+    // and the node's share their addresses (the columns t, t - 1, t - NXv and t - NXv - 1 meet there);
+    // otherwise the first tx x ty threads take the nodes
+    const int ni = kPlanes ? vi - 1 : t % tx, nj = kPlanes ? vj - 1 : t / tx;
 
     const int tile = (int)(item - P.item0_apply);
     const int bx = tile % P.tiles_x;
@@ -634,7 +655,8 @@ __global__ void __launch_bounds__(MAXT, MINB)
     // nodes of this tile inside the grid (NOHALO: its own voxel columns are 1..rx x 1..ry)
     const int rx = min(tx, nx - i0), ry = min(ty, ny - j0);
     const int kbase = k0;  // (the voxel block's coefficient array is also called k0)
-    const bool has_node = (t < tx * ty) && (i0 + ni < nx) && (j0 + nj < ny);
+    const bool has_node =
+        (kPlanes ? t < NV && ni >= 0 && nj >= 0 : t < tx * ty) && (i0 + ni < nx) && (j0 + nj < ny);
     const long long node_xy = has_node ? (long long)(j0 + nj) * nx + (i0 + ni) : 0;
 
     // this thread's staging records of the node layer (at most 3, since blockDim >= (tx+1)(ty+1)):
@@ -646,7 +668,7 @@ __global__ void __launch_bounds__(MAXT, MINB)
     for (int r = 0; r < 3; ++r) {
       const int sl = t + r * (int)blockDim.x;
       soff[r] = sl < NP ? wrapi(j0 - 1 + sl / NXp, ny) * nx + wrapi(i0 - 1 + sl % NXp, nx) : -1;
-      srec[r] = kFF ? (unsigned)(sl < NP ? sl : 0) : (unsigned)__cvta_generic_to_shared(ring + RS * (sl < NP ? sl : 0));
+      srec[r] = kPlanes ? (unsigned)(sl < NP ? sl : 0) : (unsigned)__cvta_generic_to_shared(ring + RS * (sl < NP ? sl : 0));
     }
     const unsigned slot_bytes = (unsigned)(NP * RS * sizeof(T));
     const unsigned sxy = (unsigned)__cvta_generic_to_shared(rxy), sz = (unsigned)__cvta_generic_to_shared(rz);
@@ -664,11 +686,11 @@ __global__ void __launch_bounds__(MAXT, MINB)
       for (int r = 0; r < 3; ++r) {
         if (soff[r] < 0) break;
         const int e = kofs + soff[r];
-        if constexpr (kFF) {
+        if constexpr (kPlanes) {
           const unsigned d = srec[r] + (unsigned)(b * NP);
-          cp_async_to(sxy + 16 * d, u + e);
-          cp_async_to(sxy + 16 * d + 8, u1 + e);
-          cp_async_to(sz + 8 * d, u2 + e);
+          cp_async_to(sxy + 2 * (unsigned)sizeof(Tin) * d, u + e);
+          cp_async_to(sxy + 2 * (unsigned)sizeof(Tin) * d + (unsigned)sizeof(Tin), u1 + e);
+          cp_async_to(sz + (unsigned)sizeof(Tin) * d, u2 + e);
           cp_async_to(sid + 4 * d, phase + e);
         } else {
           const unsigned d = srec[r] + sb;
@@ -687,11 +709,11 @@ __global__ void __launch_bounds__(MAXT, MINB)
     const T* const face0 = ring + RS * (vj * NXp + vi);
     const int row = RS * NXp, slot_elems = NP * RS, fbuf = 4 * NV * 4;
     const T* const hrec0 = ring + RS * ((nj + 1) * NXp + ni + 1);
-    const int face_rec = vj * NXp + vi, own_rec = (nj + 1) * NXp + ni + 1;  // (double-float planes)
+    const int face_rec = vj * NXp + vi;  // (planes: the column's corner 0 and the owned node)
     T* const fcol = Fc + 4 * vcol;
-    int goff[4];
+    int goff[kPlanes ? 1 : 4];
 #pragma unroll
-    for (int b = 0; b < 4; ++b) goff[b] = 4 * (b * NV + (ni + 1 - (b & 1)) + NXv * (nj + 1 - (b >> 1)));
+    for (int b = 0; !kPlanes && b < 4; ++b) goff[b] = 4 * (b * NV + (ni + 1 - (b & 1)) + NXv * (nj + 1 - (b >> 1)));
     // linear index of the owned node on the layer the next gather writes (layer kv - 1; the first
     // gather, at kv = k0 + 1, writes layer k0)
     int nrow = k0 * (int)plane + (int)node_xy;
@@ -714,6 +736,11 @@ __global__ void __launch_bounds__(MAXT, MINB)
       }
     };
 
+    // FP32: a column keeps its voxel's coefficient block in registers and loads another only where the
+    // phase changes along z, right after a voxel's products, a layer before it is needed (the loads were
+    // 45 of 152 LSU wavefronts per warp and layer and its longest stall: 100^3 product 37 -> 35 us)
+    constexpr bool kKeep = std::is_same<T, float>::value;
+    T kept[kKeep ? 24 : 1];
     P2<T> Vlo_xy[4], FUp_xy[4];  // modes of the lower face, forces the previous voxel left on it
     T Vlo_z[4], FUp_z[4];
     // double-float form: the forces the previous voxel left on the lower face wait in a per-thread
@@ -760,7 +787,7 @@ __global__ void __launch_bounds__(MAXT, MINB)
       for (int buf = 0; buf < 2; ++buf)
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
-          if constexpr (kFF)
+          if constexpr (kPlanes)
             st_face_ff(Fc, NV, buf * 4 * NV + b * NV + vcol, zxy, T(0));
           else
             st_xyz(fcol + buf * fbuf + b * 4 * NV, zxy, T(0));
@@ -795,8 +822,8 @@ __global__ void __launch_bounds__(MAXT, MINB)
         for (int b = 3; b >= 0; --b) {
           P2<T> xy;
           T z;
-          if constexpr (kFF) {
-            ld_face_ff(Fc, NV, ((kv - 1) & 1) * 4 * NV + goff[b] / 4, xy, z);
+          if constexpr (kPlanes) {
+            ld_face_ff(Fc, NV, t + (((kv - 1) & 1) * 4 * NV + b * NV - (b & 1) - NXv * (b >> 1)), xy, z);
           } else {
             ld_xyz(fp + goff[b], xy, z);
           }
@@ -827,15 +854,19 @@ __global__ void __launch_bounds__(MAXT, MINB)
             z_v[c * N + n] = zv[c];
             dot0r.add((double)zv[c], (double)gv[c]);
           }
-        } else {  // EPI_NORM
+        } else {  // EPI_NORM, EPI_STORE_NORM
 #pragma unroll
-          for (int c = 0; c < 3; ++c) dot1.add((double)out[c], (double)out[c]);
+          for (int c = 0; c < 3; ++c) {
+            const double r = (double)out[c];
+            if (EPI == EPI_STORE_NORM) y[c * N + n] = (Tst)r;
+            dot1.add(r, r);
+          }
         }
       }
       if (EPI == EPI_STORE_DOT && kv < k1 && has_node) {
         P2<T> hxy;
-        if constexpr (kFF)
-          ld_node_ff(rxy + (L % kRing) * NP + own_rec, rz + (L % kRing) * NP + own_rec, hxy, hown[2]);
+        if constexpr (kPlanes)
+          ld_node_ff(rxy + (L % kRing) * NP + face_rec, rz + (L % kRing) * NP + face_rec, hxy, hown[2]);
         else
           ld_xyz(hrec0 + (L % kRing) * slot_elems, hxy, hown[2]);
         hown[0] = lane0(hxy);
@@ -847,7 +878,7 @@ __global__ void __launch_bounds__(MAXT, MINB)
         const bool own = own_col;
         P2<T> Vup_xy[4];
         T Vup_z[4];
-        if constexpr (kFF) {
+        if constexpr (kPlanes) {
           if (L == 0) face_forward_ff(rxy + face_rec, rz + face_rec, NXp, Vlo_xy, Vlo_z);
           const int at = ((L + 1) % kRing) * NP + face_rec;
           face_forward_ff(rxy + at, rz + at, NXp, Vup_xy, Vup_z);
@@ -858,14 +889,17 @@ __global__ void __launch_bounds__(MAXT, MINB)
         P2<T> FL_xy[4], FU_xy[4];
         T FL_z[4], FU_z[4];
         int ph = -1;
-        if constexpr (kFF)
+        if constexpr (kPlanes)
           ph = rid[(L % kRing) * NP + face_rec];
         else if (own)
           ph = *reinterpret_cast<const int*>(face0 + (L % kRing) * slot_elems + 3);
         const T* K = ph >= 0 ? coef + (long long)ph * CoefOf<T>::stride : nullptr;
         T k0[24];
         bool solid = false;
-        if (K != nullptr) {
+        if constexpr (kKeep) {
+          if (L == 0 && K != nullptr) load_k(K + kCoefMode0, kept);
+          solid = K != nullptr && kept[kCoefSolid0] != T(0);
+        } else if (K != nullptr) {
           if constexpr (kFF) {
             solid = __ldg(reinterpret_cast<const float*>(K + kCoefSolid0)) != 0.f;
           } else {
@@ -901,6 +935,8 @@ __global__ void __launch_bounds__(MAXT, MINB)
           }
           if constexpr (kFF)
             modal_forces(W, LazyK{K + kCoefMode0}, K, F);
+          else if constexpr (kKeep)
+            modal_forces(W, kept, K, F);
           else
             modal_forces(W, k0, K, F);
           // transposed z stage: forces on the lower (this node layer) and upper face
@@ -918,6 +954,10 @@ __global__ void __launch_bounds__(MAXT, MINB)
             FL_xy[q] = FU_xy[q] = pk2(T(0), T(0));
             FL_z[q] = FU_z[q] = T(0);
           }
+        }
+        if constexpr (kKeep) {
+          const int pn = rid[((L + 1) % kRing) * NP + face_rec];
+          if (pn != ph && pn >= 0) load_k(coef + (long long)pn * CoefOf<T>::stride + kCoefMode0, kept);
         }
         // face of node layer kv: lower-face forces of this voxel + upper-face forces of the one below,
         // back-transformed to the 4 corners (transposed x and y stages)
@@ -945,7 +985,7 @@ __global__ void __launch_bounds__(MAXT, MINB)
         face_bf_t(m_z, cor_z);
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
-          if constexpr (kFF)
+          if constexpr (kPlanes)
             st_face_ff(Fc, NV, (kv & 1) * 4 * NV + b * NV + vcol, cor_xy[b], cor_z[b]);
           else
             st_xyz(fcol + (kv & 1) * fbuf + b * 4 * NV, cor_xy[b], cor_z[b]);
@@ -1127,14 +1167,16 @@ __global__ void __launch_bounds__(kEdgeThreads)
   }
 }
 
-template <typename Tin, typename T, typename Tvec, int EPI, bool AFFINE, bool NOHALO = false>
+// ONE: the batch is one problem, whose descriptor goes as a kernel argument (its blocks start on their
+// nodes without the chain of loads item -> problem -> pointers, and its tile's strides are uniform)
+template <typename Tin, typename T, typename Tvec, int EPI, bool AFFINE, bool NOHALO = false, bool ONE = false>
 cudaError_t launch_t(const BatchDev& b, int role, int post, int gate, cudaStream_t s) {
   constexpr bool f64 = sizeof(T) == 8;  // FP64 and double-float share the 8-byte configuration
   constexpr bool kFF = std::is_same<T, ff>::value;
   static_assert(!NOHALO || (f64 && EPI == EPI_STORE_DOT && !AFFINE), "no-halo form: FP64 h -> Ah with h.Ah only");
   // one block of up to 384 threads per SM for every arithmetic (FP32: 168 registers a thread; two
   // blocks of 256 at 128 registers measured 6% slower)
-  auto kern = k_apply<Tin, T, Tvec, EPI, AFFINE, f64 ? kMaxThreadsF64 : kMaxThreadsF32, 1, NOHALO>;
+  auto kern = k_apply<Tin, T, Tvec, EPI, AFFINE, f64 ? kMaxThreadsF64 : kMaxThreadsF32, 1, NOHALO, ONE>;
   // the native FP64 form does without the double-float form's carried-force slots
   const size_t smem = kFF ? b.smemff : f64 ? b.smem64 : b.smem32;
   const int blocks = f64 ? b.blocks64 : b.blocks32;
@@ -1149,7 +1191,7 @@ cudaError_t launch_t(const BatchDev& b, int role, int post, int gate, cudaStream
     set_err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kApplySmemMax);
   });
   if (set_err != cudaSuccess) return set_err;
-  kern<<<blocks, b.apply_threads, smem, s>>>(b.probs, b.item_prob, b.counts, role, post, gate);
+  kern<<<blocks, b.apply_threads, smem, s>>>(b.probs, b.item_prob, b.counts, role, post, gate, b.one);
   cudaError_t e = cudaGetLastError();
   if (NOHALO && e == cudaSuccess) {
     k_edge64<<<4 * blocks, kEdgeThreads, 0, s>>>(b.probs, b.item_prob, b.counts,
@@ -1157,6 +1199,12 @@ cudaError_t launch_t(const BatchDev& b, int role, int post, int gate, cudaStream
     e = cudaGetLastError();
   }
   return e;
+}
+
+template <typename Tvec, int EPI, bool AFFINE>
+cudaError_t launch_ff(const BatchDev& b, int role, int post, int gate, cudaStream_t s) {
+  return b.single ? launch_t<double, ff, Tvec, EPI, AFFINE, false, true>(b, role, post, gate, s)
+                  : launch_t<double, ff, Tvec, EPI, AFFINE>(b, role, post, gate, s);
 }
 
 }  // namespace
@@ -1168,11 +1216,12 @@ cudaError_t launch_apply(const BatchDev& b, int kind, int post, int gate, cudaSt
         // the recomputed-halo form: its halo columns cost the FP32 pipe less than the no-halo
         // form's edge pass and layout cost it (173 against 223 us per product at 100^3); the
         // no-halo form pays for native FP64, whose halo columns would occupy the FP64 pipe
-        return launch_t<double, ff, double, EPI_STORE_DOT, false>(b, ROLE_H, post, gate, s);
-      case AK_F64_RESID: return launch_t<double, ff, double, EPI_RESIDUAL, true>(b, ROLE_W, post, gate, s);
-      case AK_MIX_RESID: return launch_t<double, ff, float, EPI_RESIDUAL, true>(b, ROLE_W, post, gate, s);
-      case AK_F64_NORM: return launch_t<double, ff, double, EPI_NORM, true>(b, ROLE_W, post, gate, s);
-      case AK_F64_AFFINE: return launch_t<double, ff, double, EPI_STORE, true>(b, ROLE_W, post, gate, s);
+        return launch_ff<double, EPI_STORE_DOT, false>(b, ROLE_H, post, gate, s);
+      case AK_F64_RESID: return launch_ff<double, EPI_RESIDUAL, true>(b, ROLE_W, post, gate, s);
+      case AK_MIX_RESID: return launch_ff<float, EPI_RESIDUAL, true>(b, ROLE_W, post, gate, s);
+      case AK_F64_NORM: return launch_ff<double, EPI_NORM, true>(b, ROLE_W, post, gate, s);
+      case AK_F64_AFFINE: return launch_ff<double, EPI_STORE, true>(b, ROLE_W, post, gate, s);
+      case AK_F64_AFFINE_NORM: return launch_ff<double, EPI_STORE_NORM, true>(b, ROLE_W, post, gate, s);
       default: break;
     }
   }
@@ -1180,11 +1229,14 @@ cudaError_t launch_apply(const BatchDev& b, int kind, int post, int gate, cudaSt
     case AK_F64_DOT:
       if (b.nohalo64) return launch_t<double, double, double, EPI_STORE_DOT, false, true>(b, ROLE_H, post, gate, s);
       return launch_t<double, double, double, EPI_STORE_DOT, false>(b, ROLE_H, post, gate, s);
-    case AK_F32_DOT: return launch_t<float, float, float, EPI_STORE_DOT, false>(b, ROLE_H, post, gate, s);
+    case AK_F32_DOT:
+      if (b.single) return launch_t<float, float, float, EPI_STORE_DOT, false, false, true>(b, ROLE_H, post, gate, s);
+      return launch_t<float, float, float, EPI_STORE_DOT, false>(b, ROLE_H, post, gate, s);
     case AK_F64_RESID: return launch_t<double, double, double, EPI_RESIDUAL, true>(b, ROLE_W, post, gate, s);
     case AK_MIX_RESID: return launch_t<double, double, float, EPI_RESIDUAL, true>(b, ROLE_W, post, gate, s);
     case AK_F64_NORM: return launch_t<double, double, double, EPI_NORM, true>(b, ROLE_W, post, gate, s);
     case AK_F64_AFFINE: return launch_t<double, double, double, EPI_STORE, true>(b, ROLE_W, post, gate, s);
+    case AK_F64_AFFINE_NORM: return launch_t<double, double, double, EPI_STORE_NORM, true>(b, ROLE_W, post, gate, s);
   }
   return cudaErrorInvalidValue;
 }
@@ -1204,6 +1256,7 @@ int apply_resident_blocks(int elem_bytes, int threads, size_t smem) {
 
 size_t apply_smem_bytes(int tx, int ty, int elem_bytes) {
   const size_t NP = (size_t)(tx + 2) * (ty + 2), NV = (size_t)(tx + 1) * (ty + 1);
+  if (elem_bytes == 4) return plane_ring_bytes((int)NP, 4) + 2 * 4 * NV * 12;  // ring and face planes
   return 4 * (kRing * NP + 8 * NV) * elem_bytes;  // node ring + 2 face-force buffers, 4-wide records
 }
 
@@ -1211,7 +1264,7 @@ size_t apply_smem_bytes_ff(int tx, int ty) {
   const size_t NP = (size_t)(tx + 2) * (ty + 2), NV = (size_t)(tx + 1) * (ty + 1);
   // node ring (28 bytes a record, the doubles split in place), 2 compact face-force buffers (24 bytes a record),
   // the per-thread slots of the carried face forces
-  return ff_ring_bytes((int)NP) + 2 * 4 * NV * 24 + kFupSlotBytes;
+  return plane_ring_bytes((int)NP, 8) + 2 * 4 * NV * 24 + kFupSlotBytes;
 }
 
 Tiling make_tiling(const Geo& g, int elem_bytes, int sm_count, int tx_hint, int ty_hint, int kc_hint) {
