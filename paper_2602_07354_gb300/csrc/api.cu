@@ -631,9 +631,9 @@ int elas_residual(elas_ctx* c, const double* strain, const double* w, double* g,
   int r = set_aux_strain(c, c->aux64, strain);
   if (r == ELAS_OK) r = point_aux(c, c->aux64, nullptr, nullptr, w, g);
   if (r != ELAS_OK) return r;
-  ELAS_CUDA(c, launch_apply(c->aux64.bd, AK_F64_AFFINE, POST_NONE, GATE_NONE, c->stream));
+  ELAS_CUDA(c, launch_apply(c->aux64.bd, rnorm ? AK_F64_AFFINE_NORM : AK_F64_AFFINE,
+                            rnorm ? POST_TRUE_NORM : POST_NONE, GATE_NONE, c->stream));
   if (rnorm) {
-    ELAS_CUDA(c, launch_apply(c->aux64.bd, AK_F64_NORM, POST_TRUE_NORM, GATE_NONE, c->stream));
     ELAS_CUDA(c, cudaMemcpyAsync(c->aux64.h_states, c->aux64.d_states, sizeof(DevState), cudaMemcpyDeviceToHost,
                                  c->stream));
     ELAS_CUDA(c, cudaStreamSynchronize(c->stream));

@@ -384,7 +384,7 @@ struct BatchDev {
 };
 
 // apply.cu ---------------------------------------------------------------------------------
-enum ApplyEpi { EPI_STORE = 0, EPI_STORE_DOT = 1, EPI_RESIDUAL = 2, EPI_NORM = 3 };
+enum ApplyEpi { EPI_STORE = 0, EPI_STORE_DOT = 1, EPI_RESIDUAL = 2, EPI_NORM = 3, EPI_STORE_NORM = 4 };
 enum ApplyRole { ROLE_H = 0, ROLE_W = 1 };  // input h -> Ah, or input w (FP64) -> g / norms
 // post actions of a problem's last item
 enum { POST_NONE = 0, POST_LAMBDA = 1, POST_TRUE_NORM = 2, POST_REPLACE = 3 };
@@ -395,6 +395,7 @@ enum ApplyKind {
   AK_MIX_RESID = 3,     // FP64 w -> g, z (FP32 vectors): residual replacement of the mixed path
   AK_F64_NORM = 4,      // ||A w + b||^2 only
   AK_F64_AFFINE = 5,    // g = A w + b stored (FP64)
+  AK_F64_AFFINE_NORM = 6,  // both: g stored and its norm squared
 };
 
 size_t apply_smem_bytes(int tx, int ty, int elem_bytes);
