@@ -218,7 +218,8 @@ Tiling choose_tiling(const Geo& geo, int elem_bytes, int sm_count) {
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tuned.find(std::make_tuple(geo.nx, geo.ny, geo.nz, elem_bytes, sm_count));
-    if (it != g_tuned.end()) return it->second;
+    if (it != g_tuned.end() && (elem_bytes == 8 || (it->second.tx + 1) * (it->second.ty + 1) <= kMaxThreadsF32))
+      return it->second;
   }
   return make_tiling(geo, elem_bytes, sm_count);
 }
@@ -271,9 +272,12 @@ int tune_tiling(Engine& e, const Prob& proto, int eb, int sm_count, long long ma
   int rc = ELAS_OK;
   for (auto& cand : cands) {
     Prob p = proto;
-    p.tx = cand.second.tx; p.ty = cand.second.ty; p.kc = cand.second.kc;
-    p.tiles_x = cand.second.tiles_x; p.tiles_y = cand.second.tiles_y;
-    p.n_tiles = (int)cand.second.n_tiles;
+    if (eb == 4) {
+      const Tiling t64{proto.tx, proto.ty, proto.kc, proto.tiles_x, proto.tiles_y, 0, proto.n_tiles};
+      set_tilings(p, t64, &cand.second);
+    } else {
+      set_tilings(p, cand.second, nullptr);
+    }
     rc = engine_set_problems(e, {p}, err);
     if (rc != ELAS_OK) break;
     ce = launch_apply(e.bd, kind, POST_NONE, GATE_NONE, e.stream);  // warm-up
@@ -331,7 +335,7 @@ struct elas_ctx {
   double *parts = nullptr, *parts64 = nullptr, *parts32 = nullptr, *parts_stress = nullptr;
   long long stride = 0;
   Engine main, aux64, aux32;   // the solve, stand-alone FP64 products, stand-alone FP32 products
-  Tiling tl_main{}, tl64{}, tl32{};
+  Tiling tl64{}, tl32{};
   bool has_solution = false;
   std::string err;
 };
@@ -413,11 +417,10 @@ size_t carve(elas_ctx* c, char* base, int nx, int ny, int nz, int n_phases, int 
   return cv.off;
 }
 
-Prob make_prob(elas_ctx* c, const Tiling& tl, double* parts) {
+Prob make_prob(elas_ctx* c, bool f32, double* parts) {
   Prob p{};
   p.nx = c->geo.nx; p.ny = c->geo.ny; p.nz = c->geo.nz; p.N = c->geo.N;
-  p.tx = tl.tx; p.ty = tl.ty; p.kc = tl.kc; p.tiles_x = tl.tiles_x; p.tiles_y = tl.tiles_y;
-  p.n_tiles = (int)tl.n_tiles;
+  set_tilings(p, c->tl64, f32 ? &c->tl32 : nullptr);
   const bool mixed = c->precision == ELAS_PREC_MIXED;
   p.chunk = vec_chunk(c->geo.N, mixed);
   p.n_chunks = (int)chunks_of(c->geo.N, mixed);
@@ -438,10 +441,9 @@ Prob make_prob(elas_ctx* c, const Tiling& tl, double* parts) {
 int install_tilings(elas_ctx* c) {
   std::string m;
   const bool mixed = c->precision == ELAS_PREC_MIXED;
-  c->tl_main = mixed ? c->tl32 : c->tl64;
-  int r = engine_set_problems(c->main, {make_prob(c, c->tl_main, c->parts)}, &m);
-  if (r == ELAS_OK) r = engine_set_problems(c->aux64, {make_prob(c, c->tl64, c->parts64)}, &m);
-  if (r == ELAS_OK) r = engine_set_problems(c->aux32, {make_prob(c, c->tl32, c->parts32)}, &m);
+  int r = engine_set_problems(c->main, {make_prob(c, mixed, c->parts)}, &m);
+  if (r == ELAS_OK) r = engine_set_problems(c->aux64, {make_prob(c, false, c->parts64)}, &m);
+  if (r == ELAS_OK) r = engine_set_problems(c->aux32, {make_prob(c, true, c->parts32)}, &m);
   if (r != ELAS_OK) return fail(c, r, m);
   return ELAS_OK;
 }
@@ -564,9 +566,9 @@ int elas_create(elas_ctx** out, int nx, int ny, int nz, const int32_t* phase_id,
   char* t_main = (char*)c->main.d_counts;
   char* t_64 = (char*)c->aux64.d_counts;
   char* t_32 = (char*)c->aux32.d_counts;
-  r = engine_init(c->main, mixed, c->sm_count, apply_max_threads(mixed ? 4 : 8), 1, c->stride, nch, t_main, c->stream, &m);
+  r = engine_init(c->main, mixed, c->sm_count, apply_max_threads(8), 1, c->stride, nch, t_main, c->stream, &m);
   if (r == ELAS_OK) r = engine_init(c->aux64, false, c->sm_count, apply_max_threads(8), 1, c->stride, nch, t_64, c->stream, &m);
-  if (r == ELAS_OK) r = engine_init(c->aux32, true, c->sm_count, apply_max_threads(4), 1, c->stride, nch, t_32, c->stream, &m);
+  if (r == ELAS_OK) r = engine_init(c->aux32, true, c->sm_count, apply_max_threads(8), 1, c->stride, nch, t_32, c->stream, &m);
   if (r != ELAS_OK) return bail(fail(c, r, "elas_create: " + m));
   c->tl64 = choose_tiling(c->geo, 8, c->sm_count);
   c->tl32 = choose_tiling(c->geo, 4, c->sm_count);
@@ -813,7 +815,9 @@ int elas_tuning_import(const char* text) {
       return fail(nullptr, ELAS_ERR_INVALID_ARG, m);
     }
     const Geo geo{v[0], v[1], v[2], (long long)v[0] * v[1] * v[2]};
-    const Tiling t = make_tiling(geo, v[3], v[4], v[5], v[6], v[7]);
+    Tiling t = make_tiling(geo, v[3], v[4], v[5], v[6], v[7]);
+    if (v[3] == 4 && t.n_tiles <= 0 && (v[5] + 1LL) * (v[6] + 1LL) <= kMaxColumnsF32)
+      t = tiling_of(geo, v[5], v[6], v[7]);  // from a build with wider FP32 blocks: kept, not used
     if (t.n_tiles <= 0 || t.tx != v[5] || t.ty != v[6] || t.kc != v[7]) {
       char m[96];
       std::snprintf(m, sizeof m, "elas_tuning_import: line %d is not a valid tiling for its grid", line_no);
@@ -830,7 +834,7 @@ int elas_autotune(elas_ctx* c, int max_candidates, double* best_ms) {
   if (!c) return ELAS_ERR_INVALID_ARG;
   const bool mixed = c->precision == ELAS_PREC_MIXED;
   const int eb = mixed ? 4 : 8;
-  Prob proto = make_prob(c, mixed ? c->tl32 : c->tl64, mixed ? c->parts32 : c->parts64);
+  Prob proto = make_prob(c, mixed, mixed ? c->parts32 : c->parts64);
   const size_t vb = mixed ? sizeof(float) : sizeof(double);
   ELAS_CUDA(c, cudaMemsetAsync(c->h, 0, vb * 3 * c->geo.N, c->stream));
   Tiling best_t{};

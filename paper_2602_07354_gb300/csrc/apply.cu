@@ -585,14 +585,16 @@ __global__ void __launch_bounds__(MAXT, MINB)
   using Rxy = typename std::conditional<kFF, float4, float2>::type;
   using Rz = typename std::conditional<kFF, float2, float>::type;
   const int t = threadIdx.x;
-  const long long n_items = ONE ? one.n_tiles : counts[0];
+  constexpr bool kF32 = std::is_same<T, float>::value;  // the FP32 product has its own tiling
+  const long long n_items = kF32 ? (ONE ? one.fn_items : counts[2]) : (ONE ? one.n_tiles : counts[0]);
 
   for (long long item = blockIdx.x; item < n_items; item += gridDim.x) {
     const Prob& P = ONE ? one : probs[item_prob[item]];
     if (gate != GATE_NONE && gate_skips(gate, P.st)) continue;  // uniform over the block
     const int nx = P.nx, ny = P.ny, nz = P.nz;
     const long long N = P.N;
-    const int tx = P.tx, ty = P.ty;
+    const int tx = kF32 ? P.fx : P.tx, ty = kF32 ? P.fy : P.ty, kc = kF32 ? P.fkc : P.kc;
+    const int tiles_x = kF32 ? P.ftiles_x : P.tiles_x, tiles_y = kF32 ? P.ftiles_y : P.tiles_y;
     const int NXv = tx + 1, NV = (tx + 1) * (ty + 1);
     const int NXp = tx + 2, NP = (tx + 2) * (ty + 2);
     constexpr int RS = 4;                       // elements per node record
@@ -644,12 +646,13 @@ __global__ void __launch_bounds__(MAXT, MINB)
     // otherwise the first tx x ty threads take the nodes
     const int ni = kPlanes ? vi - 1 : t % tx, nj = kPlanes ? vj - 1 : t / tx;
 
-    const int tile = (int)(item - P.item0_apply);
-    const int bx = tile % P.tiles_x;
-    const int by = (tile / P.tiles_x) % P.tiles_y;
-    const int bz = tile / (P.tiles_x * P.tiles_y);
-    const int i0 = bx * tx, j0 = by * ty, k0 = bz * P.kc;
-    const int k1 = min(k0 + P.kc, nz);
+    const int tile = (int)(item - (kF32 ? P.item0_f32 : P.item0_apply));
+    const int bx = tile % tiles_x;
+    const int by = (tile / tiles_x) % tiles_y;
+    const int bz = tile / (tiles_x * tiles_y);
+    const int height = kF32 ? kc * P.fmerge : kc;  // layers of an item
+    const int i0 = bx * tx, j0 = by * ty, k0 = bz * height;
+    const int k1 = min(k0 + height, nz);
 
     const bool has_vox = t < NV;
     // nodes of this tile inside the grid (NOHALO: its own voxel columns are 1..rx x 1..ry)
@@ -799,6 +802,7 @@ __global__ void __launch_bounds__(MAXT, MINB)
     // right after every barrier (short-scoreboard stalls 0.83 of 5.9 cycles per instruction, 0.21 now):
     // 100^3 product 160 -> 139 us.  The native FP64 and FP32 forms have no such pair of pipes to overlap.
     const bool late = t >= (NV + 63) / 64 * 32;
+    int chunk_end = min(k0 + kc, k1), part = bx + tiles_x * (by + tiles_y * bz * (kF32 ? P.fmerge : 1));  // (FP32)
     T hown[3] = {T(0), T(0), T(0)};  // the owned node's operand on the previous layer (h.Ah)
     for (int kv = k0 - 1; kv <= k1; ++kv) {
       const int L = kv - k0 + 1;
@@ -1040,6 +1044,17 @@ __global__ void __launch_bounds__(MAXT, MINB)
         }
       } else {
         gather_half();
+        if constexpr (kF32) {
+          // the chunk that ends with layer kv - 1 publishes its own partial sum, so that the sums are the
+          // same however many chunks an item takes
+          if (kv == chunk_end) {
+            const double b = block_total(dot0, red);
+            if (t == 0) P.parts[part] = b;
+            dot0 = DotAcc<T>();
+            chunk_end = min(chunk_end + kc, k1);
+            part += tiles_x * tiles_y;
+          }
+        }
         compute_half();
       }
       if (kv > k0) nrow += (int)plane;
@@ -1051,6 +1066,20 @@ __global__ void __launch_bounds__(MAXT, MINB)
       // interior nodes' h.Ah; the edge pass adds the tile-edge nodes and takes the scalar step
       const double b0 = block_total(dot0, red);
       if (t == 0) P.parts[tile] = b0;
+      __syncthreads();
+    } else if (kF32) {
+      if (t == 0) {
+        __threadfence();
+        s_last = atomicAdd(&P.st->ctr[0], 1u) == (unsigned)(P.fn_items - 1);
+      }
+      __syncthreads();
+      if (s_last) {
+        const double s0 = total_of(P.parts, P.fn_tiles, red);
+        if (t == 0) {
+          P.st->ctr[0] = 0u;
+          post_scalars(P.st, post, s0, 0.0);
+        }
+      }
       __syncthreads();
     } else if (EPI != EPI_STORE) {
       const double b0 = EPI == EPI_RESIDUAL ? block_total(dot0r, red) : block_total(dot0, red);
@@ -1174,13 +1203,16 @@ cudaError_t launch_t(const BatchDev& b, int role, int post, int gate, cudaStream
   constexpr bool f64 = sizeof(T) == 8;  // FP64 and double-float share the 8-byte configuration
   constexpr bool kFF = std::is_same<T, ff>::value;
   static_assert(!NOHALO || (f64 && EPI == EPI_STORE_DOT && !AFFINE), "no-halo form: FP64 h -> Ah with h.Ah only");
-  // one block of up to 384 threads per SM for every arithmetic (FP32: 168 registers a thread; two
-  // blocks of 256 at 128 registers measured 6% slower)
-  auto kern = k_apply<Tin, T, Tvec, EPI, AFFINE, f64 ? kMaxThreadsF64 : kMaxThreadsF32, 1, NOHALO, ONE>;
+  // FP64 and double-float: one block of 384 threads per SM (168 registers a thread).  FP32: two blocks
+  // of 256 (128 registers), whose barriers do not wait for each other: 300^3 product 603 us against 659
+  // for one block of 384.  (With the coefficients read anew for every voxel one block of 384 was the
+  // faster form; keeping them took the loads out that the second block would have doubled.)
+  auto kern = k_apply<Tin, T, Tvec, EPI, AFFINE, f64 ? kMaxThreadsF64 : kMaxThreadsF32, f64 ? 1 : kBlocksF32, NOHALO, ONE>;
   // the native FP64 form does without the double-float form's carried-force slots
   const size_t smem = kFF ? b.smemff : f64 ? b.smem64 : b.smem32;
   const int blocks = f64 ? b.blocks64 : b.blocks32;
-  if (b.apply_threads > (f64 ? kMaxThreadsF64 : kMaxThreadsF32)) return cudaErrorInvalidConfiguration;
+  const int threads = f64 ? b.apply_threads : kMaxThreadsF32;
+  if (threads > (f64 ? kMaxThreadsF64 : kMaxThreadsF32)) return cudaErrorInvalidConfiguration;
   if (smem > kApplySmemMax) return cudaErrorInvalidValue;
   // The dynamic shared-memory limit is a property of the kernel, shared by every context of the
   // process: it is raised once to the largest tile any tiling may choose and never lowered, so a
@@ -1191,7 +1223,7 @@ cudaError_t launch_t(const BatchDev& b, int role, int post, int gate, cudaStream
     set_err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kApplySmemMax);
   });
   if (set_err != cudaSuccess) return set_err;
-  kern<<<blocks, b.apply_threads, smem, s>>>(b.probs, b.item_prob, b.counts, role, post, gate, b.one);
+  kern<<<blocks, threads, smem, s>>>(b.probs, f64 ? b.item_prob : b.fitem_prob, b.counts, role, post, gate, b.one);
   cudaError_t e = cudaGetLastError();
   if (NOHALO && e == cudaSuccess) {
     k_edge64<<<4 * blocks, kEdgeThreads, 0, s>>>(b.probs, b.item_prob, b.counts,
@@ -1249,7 +1281,8 @@ bool apply_nohalo_fits(const Prob& p) {
 }
 
 int apply_resident_blocks(int elem_bytes, int threads, size_t smem) {
-  int R = elem_bytes == 8 ? 1 : std::max(1, (int)(65536 / (threads * 168)));
+  (void)threads;
+  int R = elem_bytes == 8 ? 1 : kBlocksF32;
   R = std::min(R, (int)((227 * 1024) / (smem + 1024)));
   return std::max(R, 1);
 }
@@ -1267,19 +1300,60 @@ size_t apply_smem_bytes_ff(int tx, int ty) {
   return plane_ring_bytes((int)NP, 8) + 2 * 4 * NV * 24 + kFupSlotBytes;
 }
 
-Tiling make_tiling(const Geo& g, int elem_bytes, int sm_count, int tx_hint, int ty_hint, int kc_hint) {
-  // Model: the SM is throughput-bound, so the time of a launch is the busiest SM's work.  With R
-  // blocks resident per SM (registers ~128/thread, shared memory per block), tiles are handed out
-  // round-robin to sm_count*R blocks; the busiest SM runs ceil(n_tiles/(sm_count*R)) rounds of R
-  // tiles, each (kc + 1) voxel layers of `threads` voxel slots plus a fixed per-layer overhead
-  // (the barrier and the staging).  FP32 tiles also pay for latency not hidden by fewer
-  // than two resident blocks.
+Tiling tiling_of(const Geo& g, int tx, int ty, int kc) {
+  Tiling t{};
+  t.tx = tx; t.ty = ty; t.kc = kc;
+  t.tiles_x = (g.nx - 1) / tx + 1; t.tiles_y = (g.ny - 1) / ty + 1; t.tiles_z = (g.nz - 1) / kc + 1;
+  t.n_tiles = (long long)t.tiles_x * t.tiles_y * t.tiles_z;
+  return t;
+}
+
+// FP32 product: two blocks of up to 256 columns share an SM.  Microseconds of a launch, from the
+// product's times at 48^3 ... 300^3: a pair of tiles takes 1.42 us per voxel layer at 8 warps each,
+// 1.38 at 7 (latency, not work, sets it) and 3.0 us to fill and drain, a tile alone on its SM 0.96 and
+// 2.6, rows of 8 nodes cost 11% more than rows of 15, and the busiest SM sets the time.
+static Tiling make_tiling32(const Geo& g, int sm_count, int tx_hint, int ty_hint, int kc_hint) {
   Tiling best{};
   double best_cost = 1e300;
   const int tx_lo = tx_hint ? tx_hint : 4, tx_hi = tx_hint ? tx_hint : 40;
   const int ty_lo = ty_hint ? ty_hint : 2, ty_hi = ty_hint ? ty_hint : 24;
-  const int min_threads = elem_bytes == 8 ? 192 : 96;
-  const int max_threads = elem_bytes == 8 ? kMaxThreadsF64 : kMaxThreadsF32;
+  for (int tx = tx_lo; tx <= tx_hi; ++tx)
+    for (int ty = ty_lo; ty <= ty_hi; ++ty) {
+      const long long nv = (long long)(tx + 1) * (ty + 1);
+      if (nv > kMaxThreadsF32 || (nv < 64 && !(tx_hint && ty_hint))) continue;
+      if (apply_smem_bytes(tx, ty, 4) > kApplySmemMax / kBlocksF32) continue;
+      const double narrow = 1.0 + 0.0022 * std::max(0, 15 - tx) * std::max(0, 15 - tx);  // short rows
+      const double warps = (double)((nv + 31) / 32);
+      const double pair = narrow * (1.10 + 0.04 * warps), alone = narrow * (0.80 + 0.02 * warps);
+      for (int kc = (kc_hint ? kc_hint : 1); kc <= (kc_hint ? kc_hint : std::min(64, g.nz)); ++kc) {
+        const Tiling t = tiling_of(g, tx, ty, kc);
+        if (t.n_tiles > (1LL << 30)) continue;
+        const long long m = (t.n_tiles + sm_count - 1) / sm_count;  // tiles of the busiest SM
+        const double cost = (double)(m / 2) * (pair * (kc + 1) + 3.0) + (double)(m % 2) * (alone * (kc + 1) + 2.6);
+        if (cost < best_cost * 0.999) {
+          best_cost = cost;
+          best = t;
+          best.threads = kMaxThreadsF32;
+          best.blocks = (int)std::min<long long>(t.n_tiles, (long long)sm_count * kBlocksF32);
+          best.smem = apply_smem_bytes(tx, ty, 4);
+        }
+      }
+    }
+  return best;
+}
+
+Tiling make_tiling(const Geo& g, int elem_bytes, int sm_count, int tx_hint, int ty_hint, int kc_hint) {
+  if (elem_bytes == 4) return make_tiling32(g, sm_count, tx_hint, ty_hint, kc_hint);
+  // Model: the SM is throughput-bound, so the time of a launch is the busiest SM's work.  With R
+  // blocks resident per SM (registers ~128/thread, shared memory per block), tiles are handed out
+  // round-robin to sm_count*R blocks; the busiest SM runs ceil(n_tiles/(sm_count*R)) rounds of R
+  // tiles, each (kc + 1) voxel layers of `threads` voxel slots plus a fixed per-layer overhead
+  // (the barrier and the staging).
+  Tiling best{};
+  double best_cost = 1e300;
+  const int tx_lo = tx_hint ? tx_hint : 4, tx_hi = tx_hint ? tx_hint : 40;
+  const int ty_lo = ty_hint ? ty_hint : 2, ty_hi = ty_hint ? ty_hint : 24;
+  const int min_threads = 192, max_threads = kMaxThreadsF64;
   for (int tx = tx_lo; tx <= tx_hi; ++tx)
     for (int ty = ty_lo; ty <= ty_hi; ++ty) {
       // every item of a launch runs with the same block size; threads beyond the tile idle
@@ -1287,8 +1361,7 @@ Tiling make_tiling(const Geo& g, int elem_bytes, int sm_count, int tx_hint, int 
       const int threads = max_threads;
       if (nv > threads || tx * ty > threads) continue;
       if (nv < min_threads && !(tx_hint && ty_hint)) continue;
-      const size_t smem = elem_bytes == 8 ? std::max(apply_smem_bytes(tx, ty, 8), apply_smem_bytes_ff(tx, ty))
-                                          : apply_smem_bytes(tx, ty, elem_bytes);
+      const size_t smem = std::max(apply_smem_bytes(tx, ty, 8), apply_smem_bytes_ff(tx, ty));
       if (smem > kApplySmemMax) continue;
       const int R = apply_resident_blocks(elem_bytes, threads, smem);
       const int tiles_x = (g.nx + tx - 1) / tx, tiles_y = (g.ny + ty - 1) / ty;
@@ -1301,7 +1374,6 @@ Tiling make_tiling(const Geo& g, int elem_bytes, int sm_count, int tx_hint, int 
         const double per_sm_tiles = (double)rounds * std::min<long long>(R, (n_tiles + sm_count - 1) / sm_count);
         double cost = per_sm_tiles * (kc + 1 + 0.5) * (threads + 64);
         if (n_tiles > (1LL << 30)) continue;
-        if (elem_bytes == 4 && blocks < 2LL * sm_count) cost *= 1.0 + 0.5 * (2.0 - (double)blocks / sm_count) / 2.0;
         if (cost < best_cost * 0.999) {
           best_cost = cost;
           best.tx = tx; best.ty = ty; best.kc = kc;

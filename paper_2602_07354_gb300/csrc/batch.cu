@@ -29,7 +29,7 @@ thread_local std::string g_batch_err;
 struct RveDev {
   GridHost grid;
   Geo geo{};
-  Tiling tl{};
+  Tiling tl64{}, tl32{};  // tl32: mixed batches only
   int32_t* phase = nullptr;
   double* coef64 = nullptr;
   float* coef32 = nullptr;
@@ -86,11 +86,9 @@ int bfail(elas_batch* b, int code, const std::string& m) {
 
 // Workspace layout (sizing when base == nullptr).  Per RVE: ids, tables, Jacobi inverse; per
 // problem: load-case sigma, w (FP64 and the mixed pair), g, h, Ah, z and per-item partials.
-size_t batch_carve(elas_batch* b, char* base, int n_rve, const elas_rve* rv, int n_rhs, int precision,
-                   const std::vector<Tiling>& tls) {
+size_t batch_carve(elas_batch* b, char* base, int n_rve, const elas_rve* rv, int n_rhs, int precision) {
   const bool mixed = precision == ELAS_PREC_MIXED;
   const size_t vb = mixed ? sizeof(float) : sizeof(double);
-  (void)tls;
   long long cap_apply = 0, cap_vec = 0, max_bound = 0;
   for (int i = 0; i < n_rve; ++i) {
     const long long N = (long long)rv[i].nx * rv[i].ny * rv[i].nz;
@@ -143,20 +141,11 @@ size_t batch_carve(elas_batch* b, char* base, int n_rve, const elas_rve* rv, int
   return cv.off;
 }
 
-std::vector<Tiling> batch_tilings(int n_rve, const elas_rve* rv, int precision, int sm_count) {
-  std::vector<Tiling> tls;
-  for (int i = 0; i < n_rve; ++i)
-    tls.push_back(choose_tiling(Geo{rv[i].nx, rv[i].ny, rv[i].nz, (long long)rv[i].nx * rv[i].ny * rv[i].nz},
-                                precision == ELAS_PREC_MIXED ? 4 : 8, sm_count));
-  return tls;
-}
-
 Prob prob_of(elas_batch* b, const ProbDev& pd) {
   const RveDev& R = b->rves[pd.rve];
   Prob p{};
   p.nx = R.geo.nx; p.ny = R.geo.ny; p.nz = R.geo.nz; p.N = R.geo.N;
-  p.tx = R.tl.tx; p.ty = R.tl.ty; p.kc = R.tl.kc; p.tiles_x = R.tl.tiles_x; p.tiles_y = R.tl.tiles_y;
-  p.n_tiles = (int)R.tl.n_tiles;
+  set_tilings(p, R.tl64, b->precision == ELAS_PREC_MIXED ? &R.tl32 : nullptr);
   const bool mixed = b->precision == ELAS_PREC_MIXED;
   p.chunk = vec_chunk(R.geo.N, mixed);
   p.n_chunks = (int)chunks_of(R.geo.N, mixed);
@@ -192,7 +181,7 @@ int elas_batch_workspace_bytes(int n_rve, const elas_rve* rves, int n_rhs, int p
   for (int i = 0; i < n_rve; ++i)
     if (rves[i].nx < 2 || rves[i].ny < 2 || rves[i].nz < 2 || rves[i].n_phases < 0)
       return bfail(nullptr, ELAS_ERR_INVALID_ARG, "elas_batch_workspace_bytes: grid dimensions must be >= 2");
-  *bytes = batch_carve(nullptr, nullptr, n_rve, rves, n_rhs, precision, {});
+  *bytes = batch_carve(nullptr, nullptr, n_rve, rves, n_rhs, precision);
   return ELAS_OK;
 }
 
@@ -229,22 +218,24 @@ int elas_batch_create(elas_batch** out, int n_rve, const elas_rve* rves, int n_r
     }
     b->rves[i].geo = Geo{rves[i].nx, rves[i].ny, rves[i].nz, b->rves[i].grid.N};
   }
-  const std::vector<Tiling> tls = batch_tilings(n_rve, rves, precision, sms);
-  const size_t need = batch_carve(nullptr, nullptr, n_rve, rves, n_rhs, precision, tls);
+  const size_t need = batch_carve(nullptr, nullptr, n_rve, rves, n_rhs, precision);
   if (!workspace || ((uintptr_t)workspace % kAlign) != 0 || ws_bytes < need) {
     char buf[160];
     std::snprintf(buf, sizeof buf, "elas_batch_create: workspace needs %zu bytes, 256-byte aligned (got %zu)", need,
                   ws_bytes);
     return bail(bfail(b, ELAS_ERR_WORKSPACE, buf));
   }
-  batch_carve(b, (char*)workspace, n_rve, rves, n_rhs, precision, tls);
-  for (int i = 0; i < n_rve; ++i) b->rves[i].tl = tls[i];
+  batch_carve(b, (char*)workspace, n_rve, rves, n_rhs, precision);
   const bool mixed = precision == ELAS_PREC_MIXED;
+  for (RveDev& R : b->rves) {
+    R.tl64 = choose_tiling(R.geo, 8, sms);
+    if (mixed) R.tl32 = choose_tiling(R.geo, 4, sms);
+  }
   std::string m;
-  int r = engine_init(b->main, mixed, sms, apply_max_threads(mixed ? 4 : 8), n_rve * n_rhs, b->cap_apply, b->cap_vec,
+  int r = engine_init(b->main, mixed, sms, apply_max_threads(8), n_rve * n_rhs, b->cap_apply, b->cap_vec,
                       b->main_tables, b->stream, &m);
   if (r == ELAS_OK)
-    r = engine_init(b->aux, mixed, sms, apply_max_threads(mixed ? 4 : 8), 1, b->max_stride, b->max_stride,
+    r = engine_init(b->aux, mixed, sms, apply_max_threads(8), 1, b->max_stride, b->max_stride,
                     b->aux_tables, b->stream, &m);
   if (r != ELAS_OK) return bail(bfail(b, r, "elas_batch_create: " + m));
   b->stress_state = b->aux.d_states;
@@ -312,7 +303,7 @@ int elas_batch_autotune(elas_batch* b, int max_candidates) {
       if (r != ELAS_OK) return bfail(b, r, "elas_batch_autotune: " + m);
       it = done.emplace(key, best).first;
     }
-    R.tl = it->second;
+    (mixed ? R.tl32 : R.tl64) = it->second;
   }
   std::vector<Prob> ps;
   for (const ProbDev& pd : b->probs) ps.push_back(prob_of(b, pd));

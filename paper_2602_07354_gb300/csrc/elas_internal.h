@@ -40,7 +40,10 @@ constexpr int kSymStride = 21;
 // each pair the double value split exactly as hi = fl32(v), lo = fl32(v - hi).
 constexpr int kCoefFF = 128, kCoefFFBlock = 48;
 constexpr int kCoef32Stride = 288;
-constexpr int kMaxThreadsF64 = 384, kMaxThreadsF32 = 384;
+constexpr int kMaxThreadsF64 = 384, kMaxThreadsF32 = 256;
+// widest FP32 tile ((tx + 1)(ty + 1) columns) that a tuning record may name; one wider than a block
+// of the product is kept in the record but not used
+constexpr int kMaxColumnsF32 = 384;
 // largest dynamic shared memory of an operator tile (the 4-slot node ring and the face buffers)
 constexpr size_t kApplySmemMax = 200 * 1024;
 // per-thread slots of the double-float operator's carried face forces (6 float4 per thread)
@@ -345,10 +348,13 @@ constexpr int kPartsSlots = 3;
 struct Prob {
   int nx, ny, nz;
   long long N;
-  int tx, ty, kc, tiles_x, tiles_y, n_tiles;  // operator tiling of this grid
+  int tx, ty, kc, tiles_x, tiles_y, n_tiles;  // tiling of the FP64 and double-float products
+  // tiling of the FP32 product: an item is fmerge consecutive z-chunks of fkc layers, marched in one go
+  // with one partial sum per chunk, so that results do not depend on how many chunks an item takes
+  int fx, fy, fkc, ftiles_x, ftiles_y, fn_tiles, fmerge, fn_items;
   int chunk, n_chunks;                         // nodes per vector-kernel item, items
-  int parts_stride;                            // >= max(n_tiles, n_chunks)
-  long long item0_apply, item0_vec;            // first work item of this problem
+  int parts_stride;                            // >= max(n_tiles, fn_tiles, n_chunks)
+  long long item0_apply, item0_f32, item0_vec;  // first work items of this problem
   const int32_t* phase;
   const double* coef64;
   const float* coef32;
@@ -369,9 +375,10 @@ struct Prob {
 // Launch description shared by the iteration kernels of one batch (device pointers).
 struct BatchDev {
   const Prob* probs;
-  const int* item_prob;    // apply item -> problem
+  const int* item_prob;    // FP64 / double-float product item -> problem
+  const int* fitem_prob;   // FP32 product item -> problem
   const int* vitem_prob;   // vector item -> problem
-  const long long* counts; // [0] apply items, [1] vector items (read on the device)
+  const long long* counts; // [0] FP64 product items, [1] vector items, [2] FP32 product items
   int apply_threads;       // block size of every operator launch (>= every tile's voxel count)
   size_t smem32, smem64;   // dynamic shared memory of FP32 / native FP64 operator launches
   size_t smemff;           // ... of double-float FP64 operator launches
@@ -400,6 +407,8 @@ enum ApplyKind {
 
 size_t apply_smem_bytes(int tx, int ty, int elem_bytes);
 size_t apply_smem_bytes_ff(int tx, int ty);
+constexpr int kBlocksF32 = 2;  // resident blocks per SM of the FP32 product
+Tiling tiling_of(const Geo& g, int tx, int ty, int kc);
 Tiling make_tiling(const Geo& g, int elem_bytes, int sm_count, int tx_hint = 0, int ty_hint = 0, int kc_hint = 0);
 int apply_max_threads(int elem_bytes);
 int apply_resident_blocks(int elem_bytes, int threads, size_t smem);

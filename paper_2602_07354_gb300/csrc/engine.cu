@@ -55,7 +55,7 @@ int record_batch(Engine& e, int K, std::string* err) {
 }
 
 size_t engine_table_bytes(int cap_probs, long long cap_apply, long long cap_vec) {
-  return up(2 * sizeof(long long)) + up(sizeof(Prob) * std::max(cap_probs, 1)) + up(sizeof(int) * std::max(cap_apply, 1LL)) +
+  return up(3 * sizeof(long long)) + up(sizeof(Prob) * std::max(cap_probs, 1)) + 2 * up(sizeof(int) * std::max(cap_apply, 1LL)) +
          up(sizeof(int) * std::max(cap_vec, 1LL)) + up(sizeof(SolveSetup) * std::max(cap_probs, 1)) +
          up(sizeof(int) * std::max(cap_probs, 1)) + up(sizeof(DevState) * std::max(cap_probs, 1));
 }
@@ -70,10 +70,12 @@ int engine_init(Engine& e, bool mixed, int sm_count, int apply_threads, int cap_
   e.cap_vec = cap_vec;
   size_t off = 0;
   e.d_counts = reinterpret_cast<long long*>(mem + off);
-  off += up(2 * sizeof(long long));
+  off += up(3 * sizeof(long long));
   e.d_probs = reinterpret_cast<Prob*>(mem + off);
   off += up(sizeof(Prob) * std::max(cap_probs, 1));
   e.d_item = reinterpret_cast<int*>(mem + off);
+  off += up(sizeof(int) * std::max(cap_apply, 1LL));
+  e.d_fitem = reinterpret_cast<int*>(mem + off);
   off += up(sizeof(int) * std::max(cap_apply, 1LL));
   e.d_vitem = reinterpret_cast<int*>(mem + off);
   off += up(sizeof(int) * std::max(cap_vec, 1LL));
@@ -90,6 +92,7 @@ int engine_init(Engine& e, bool mixed, int sm_count, int apply_threads, int cap_
   if (c != cudaSuccess) return cfail(err, c, "engine pinned state mirror");
   e.bd.probs = e.d_probs;
   e.bd.item_prob = e.d_item;
+  e.bd.fitem_prob = e.d_fitem;
   e.bd.vitem_prob = e.d_vitem;
   e.bd.counts = e.d_counts;
   e.bd.apply_threads = apply_threads;
@@ -107,37 +110,61 @@ void engine_set_ff64(Engine& e, bool on) {
   }
 }
 
+// z-chunks per FP32 item.  A single problem keeps one, its tiling being made for a launch of its own
+// (a 48^3 grid's chunks are 3 layers so that its tiles fill the SMs).  Problems that share launches
+// have tiles to spare, and every item recomputes the voxel layer below it, a third more work at 3
+// layers: their items take about 32 layers, as long as four items per SM remain.
+static void merge_chunks(Engine& e) {
+  const bool shared = e.fixed_smem32 != 0 || e.probs.size() > 1;
+  for (int want = shared ? 32 : 1;; want /= 2) {
+    long long n = 0;
+    for (Prob& p : e.probs) {
+      if (p.fn_tiles == 0) continue;
+      const int xy = p.ftiles_x * p.ftiles_y, z = p.fn_tiles / xy;
+      p.fmerge = std::max(1, std::min(z, (want + p.fkc - 1) / p.fkc));
+      p.fn_items = xy * ((z + p.fmerge - 1) / p.fmerge);
+      n += p.fn_items;
+    }
+    if (want <= 1 || n >= 4LL * e.sm_count) return;
+  }
+}
+
 int engine_set_problems(Engine& e, const std::vector<Prob>& probs, std::string* err) {
   if ((int)probs.size() > e.cap_probs) {
     if (err) *err = "engine: more problems than its tables hold";
     return ELAS_ERR_INVALID_ARG;
   }
   e.probs = probs;
-  long long na = 0, nv = 0;
+  merge_chunks(e);
+  long long na = 0, nf = 0, nv = 0;
   size_t smem32 = 0, smem64 = 0, smemff = 0;
   for (size_t i = 0; i < e.probs.size(); ++i) {
     Prob& p = e.probs[i];
     p.st = e.d_states + i;
     p.item0_apply = na;
+    p.item0_f32 = nf;
     p.item0_vec = nv;
     na += p.n_tiles;
+    nf += p.fn_items;
     nv += p.n_chunks;
-    smem32 = std::max(smem32, apply_smem_bytes(p.tx, p.ty, 4));
+    smem32 = std::max(smem32, apply_smem_bytes(p.fx, p.fy, 4));
     smem64 = std::max(smem64, apply_smem_bytes(p.tx, p.ty, 8));
     smemff = std::max(smemff, apply_smem_bytes_ff(p.tx, p.ty));
   }
-  if (na > e.cap_apply || nv > e.cap_vec) {
+  if (na > e.cap_apply || nf > e.cap_apply || nv > e.cap_vec) {
     if (err) *err = "engine: more work items than its tables hold";
     return ELAS_ERR_INVALID_ARG;
   }
   e.n_apply = na;
+  e.n_f32 = nf;
   e.n_vec = nv;
-  std::vector<int> item(std::max(na, 1LL)), vitem(std::max(nv, 1LL));
+  std::vector<int> item(std::max(na, 1LL)), fitem(std::max(nf, 1LL)), vitem(std::max(nv, 1LL));
   for (int i = 0; i < (int)e.probs.size(); ++i) {
     for (long long t = 0; t < e.probs[i].n_tiles; ++t) item[e.probs[i].item0_apply + t] = i;
+    for (long long t = 0; t < e.probs[i].fn_items; ++t) fitem[e.probs[i].item0_f32 + t] = i;
     for (long long t = 0; t < e.probs[i].n_chunks; ++t) vitem[e.probs[i].item0_vec + t] = i;
   }
-  const long long counts[2] = {na, nv};
+  const long long counts[3] = {na, nv, nf};
   if (e.fixed_smem32) {
     // fixed launch shape: the recorded graph stays valid whatever the set of problems
     if (smem32 > e.fixed_smem32 || smem64 > e.fixed_smem64 || smemff > e.fixed_smemff) {
@@ -147,7 +174,7 @@ int engine_set_problems(Engine& e, const std::vector<Prob>& probs, std::string* 
     e.bd.smem32 = e.fixed_smem32;
     e.bd.smem64 = e.fixed_smem64;
     e.bd.smemff = e.fixed_smemff;
-    e.bd.blocks32 = e.sm_count * apply_resident_blocks(4, e.bd.apply_threads, e.bd.smem32);
+    e.bd.blocks32 = e.sm_count * apply_resident_blocks(4, kMaxThreadsF32, e.bd.smem32);
     e.bd.blocks64 = e.sm_count * apply_resident_blocks(8, e.bd.apply_threads, e.bd.smem64);
     e.bd.vec_blocks = e.sm_count * 8;
     e.bd.nohalo64 = 0;  // the kernel choice is part of the recorded graph, which must outlive any set
@@ -155,9 +182,9 @@ int engine_set_problems(Engine& e, const std::vector<Prob>& probs, std::string* 
     e.bd.smem32 = std::max<size_t>(smem32, 16);
     e.bd.smem64 = std::max<size_t>(smem64, 16);
     e.bd.smemff = std::max<size_t>(smemff, 16);
-    const int r32 = apply_resident_blocks(4, e.bd.apply_threads, e.bd.smem32);
+    const int r32 = apply_resident_blocks(4, kMaxThreadsF32, e.bd.smem32);
     const int r64 = apply_resident_blocks(8, e.bd.apply_threads, e.bd.smem64);
-    e.bd.blocks32 = (int)std::max(1LL, std::min<long long>(na, (long long)e.sm_count * r32));
+    e.bd.blocks32 = (int)std::max(1LL, std::min<long long>(nf, (long long)e.sm_count * r32));
     e.bd.blocks64 = (int)std::max(1LL, std::min<long long>(na, (long long)e.sm_count * r64));
     e.bd.vec_blocks = (int)std::max(1LL, std::min<long long>(nv, (long long)e.sm_count * 8));
     bool fits = !e.probs.empty();
@@ -167,6 +194,8 @@ int engine_set_problems(Engine& e, const std::vector<Prob>& probs, std::string* 
   cudaError_t c = cudaMemcpyAsync(e.d_counts, counts, sizeof counts, cudaMemcpyHostToDevice, e.stream);
   if (c == cudaSuccess)
     c = cudaMemcpyAsync(e.d_item, item.data(), sizeof(int) * item.size(), cudaMemcpyHostToDevice, e.stream);
+  if (c == cudaSuccess && nf > 0)
+    c = cudaMemcpyAsync(e.d_fitem, fitem.data(), sizeof(int) * fitem.size(), cudaMemcpyHostToDevice, e.stream);
   if (c == cudaSuccess)
     c = cudaMemcpyAsync(e.d_vitem, vitem.data(), sizeof(int) * vitem.size(), cudaMemcpyHostToDevice, e.stream);
   if (c != cudaSuccess) return cfail(err, c, "engine tables");

@@ -18,10 +18,11 @@ struct Engine {
   cudaStream_t stream = nullptr;      // owner's stream: all work is ordered on it
   cudaStream_t cap_stream = nullptr;  // private stream used only to record graphs
   std::vector<Prob> probs;            // host mirror of the device descriptors
-  long long n_apply = 0, n_vec = 0;   // work items of the operator and vector kernels
+  long long n_apply = 0, n_f32 = 0, n_vec = 0;  // work items of the operators and vector kernels
   long long* d_counts = nullptr;
   Prob* d_probs = nullptr;
   int* d_item = nullptr;
+  int* d_fitem = nullptr;
   int* d_vitem = nullptr;
   SolveSetup* d_setups = nullptr;
   int* d_idx = nullptr;               // problem indices of a partial set-up (server admissions)
@@ -45,6 +46,18 @@ size_t engine_table_bytes(int cap_probs, long long cap_apply, long long cap_vec)
 inline long long tiles_of(const Tiling& t) { return t.n_tiles; }
 inline long long chunks_of(long long N, bool mixed) { return (N + vec_chunk(N, mixed) - 1) / vec_chunk(N, mixed); }
 constexpr int kMoreChunks = 2048;  // chunks_of(N) <= N / 2048 + kMoreChunks
+
+// A problem's operator tilings: t64 for the FP64 and double-float products, t32 for the FP32 one (null
+// in FP64 engines).
+inline void set_tilings(Prob& p, const Tiling& t64, const Tiling* t32) {
+  p.tx = t64.tx; p.ty = t64.ty; p.kc = t64.kc; p.tiles_x = t64.tiles_x; p.tiles_y = t64.tiles_y;
+  p.n_tiles = (int)t64.n_tiles;
+  p.fx = p.fy = p.fkc = p.ftiles_x = p.ftiles_y = p.fmerge = 1;
+  p.fn_tiles = p.fn_items = 0;
+  if (!t32) return;
+  p.fx = t32->tx; p.fy = t32->ty; p.fkc = t32->kc; p.ftiles_x = t32->tiles_x; p.ftiles_y = t32->tiles_y;
+  p.fn_tiles = (int)t32->n_tiles;
+}
 
 // Prepare an engine: tables in `mem` (engine_table_bytes), streams and pinned state mirror.
 int engine_init(Engine& e, bool mixed, int sm_count, int apply_threads, int cap_probs, long long cap_apply,

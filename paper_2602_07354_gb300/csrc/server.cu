@@ -93,7 +93,7 @@ struct Request {
   // device block
   size_t off = 0, bytes = 0;
   Prob prob{};
-  Tiling tl{};
+  Tiling tl64{}, tl32{};  // tl32: mixed servers only
   int slot = -1;      // index in the engine's problem table while active
   DevState final_state{};
   bool finished = false;
@@ -104,12 +104,12 @@ struct Layout {
   long long stride;
 };
 
-Layout request_layout(const Geo& geo, int n_phases, bool mixed, const Tiling& tl) {
+Layout request_layout(const Geo& geo, int n_phases, bool mixed, const Tiling& tl64, const Tiling& tl32) {
   const long long N = geo.N;
   const size_t vb = mixed ? sizeof(float) : sizeof(double);
   const size_t P = (size_t)std::max(n_phases, 1);
   Layout L{};
-  L.stride = std::max<long long>(tl.n_tiles, chunks_of(N, mixed));
+  L.stride = std::max<long long>({tl64.n_tiles, mixed ? tl32.n_tiles : 0, chunks_of(N, mixed)});
   size_t o = 0;
   auto take = [&](size_t b) {
     const size_t at = o;
@@ -205,10 +205,8 @@ int rebuild(elas_server* s) {
       ps[i] = Prob{};
       ps[i].nx = ps[i].ny = ps[i].nz = 2;
       ps[i].N = 8;
-      ps[i].tx = ps[i].ty = 1;
-      ps[i].kc = 1;
-      ps[i].tiles_x = ps[i].tiles_y = 1;
-      ps[i].n_tiles = 0;
+      const Tiling none{1, 1, 1, 1, 1, 0, 0};
+      set_tilings(ps[i], none, nullptr);
       ps[i].chunk = 128;
       ps[i].n_chunks = 0;
     }
@@ -263,7 +261,7 @@ int elas_server_create(elas_server** out, size_t budget_bytes, int max_active, i
   s->eng.fixed_smem64 = max_tile_smem(8);
   s->eng.fixed_smemff = max_tile_smem(0);
   std::string m;
-  int r = engine_init(s->eng, mixed, s->sm_count, apply_max_threads(mixed ? 4 : 8), max_active,
+  int r = engine_init(s->eng, mixed, s->sm_count, apply_max_threads(8), max_active,
                       vox / 48 + 4096LL * max_active, vox / 2048 + (long long)kMoreChunks * max_active, s->arena_base + s->budget,
                       s->stream, &m);
   if (r != ELAS_OK) {
@@ -301,8 +299,9 @@ int elas_server_submit(elas_server* s, const elas_rve* rve, const double* strain
   }
   const bool mixed = s->precision == ELAS_PREC_MIXED;
   const Geo geo{rve->nx, rve->ny, rve->nz, r->grid.N};
-  r->tl = choose_tiling(geo, mixed ? 4 : 8, s->sm_count);
-  const Layout L = request_layout(geo, rve->n_phases, mixed, r->tl);
+  r->tl64 = choose_tiling(geo, 8, s->sm_count);
+  if (mixed) r->tl32 = choose_tiling(geo, 4, s->sm_count);
+  const Layout L = request_layout(geo, rve->n_phases, mixed, r->tl64, r->tl32);
   if (L.total > s->budget) {
     delete r;
     return sfail(s, ELAS_ERR_ADMISSION, "elas_server_submit: the request alone exceeds the memory budget");
@@ -338,13 +337,12 @@ int elas_server_step(elas_server* s, int* n_active_out, int* n_queued, int* n_fi
     r->off = off;
     r->t_admit = now_s();
     const Geo geo{r->grid.nx, r->grid.ny, r->grid.nz, r->grid.N};
-    const Layout L = request_layout(geo, r->grid.n_phases, mixed, r->tl);
+    const Layout L = request_layout(geo, r->grid.n_phases, mixed, r->tl64, r->tl32);
     char* base = s->arena_base + off;
     Prob& p = r->prob;
     p = Prob{};
     p.nx = geo.nx; p.ny = geo.ny; p.nz = geo.nz; p.N = geo.N;
-    p.tx = r->tl.tx; p.ty = r->tl.ty; p.kc = r->tl.kc; p.tiles_x = r->tl.tiles_x; p.tiles_y = r->tl.tiles_y;
-    p.n_tiles = (int)r->tl.n_tiles;
+    set_tilings(p, r->tl64, mixed ? &r->tl32 : nullptr);
     p.chunk = vec_chunk(geo.N, mixed);
     p.n_chunks = (int)chunks_of(geo.N, mixed);
     p.parts_stride = (int)L.stride;
