@@ -325,7 +325,8 @@ struct Geo {
 // A single solve is a batch of one problem.
 // ------------------------------------------------------------------------------------------
 constexpr int kVecThreads = 256;                    // block size of the vector kernels
-// Nodes per vector-kernel work item, by the grid's size and precision alone (so a problem's sums do
+// Nodes per partial sum of the vector kernels (an item is one such chunk, or several where problems
+// share launches), by the grid's size and precision alone (so a problem's sums do
 // not depend on its batch).  The grid's nodes are split evenly over whole waves of resident blocks
 // (four a SM in FP64, three mixed), because an uneven split leaves the last wave nearly empty (977
 // items of 1,024 nodes over 608 resident blocks took 246 us per FP64 iteration at 100^3, 607 of 1,648
@@ -352,7 +353,8 @@ struct Prob {
   // tiling of the FP32 product: an item is fmerge consecutive z-chunks of fkc layers, marched in one go
   // with one partial sum per chunk, so that results do not depend on how many chunks an item takes
   int fx, fy, fkc, ftiles_x, ftiles_y, fn_tiles, fmerge, fn_items;
-  int chunk, n_chunks;                         // nodes per vector-kernel item, items
+  int chunk, n_chunks;                         // nodes per partial sum of the vector kernels, their number
+  int vmerge, n_vitems;                        // chunks per vector-kernel item, items
   int parts_stride;                            // >= max(n_tiles, fn_tiles, n_chunks)
   long long item0_apply, item0_f32, item0_vec;  // first work items of this problem
   const int32_t* phase;

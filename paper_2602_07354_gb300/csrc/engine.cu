@@ -116,6 +116,17 @@ void engine_set_ff64(Engine& e, bool on) {
 // layers: their items take about 32 layers, as long as four items per SM remain.
 static void merge_chunks(Engine& e) {
   const bool shared = e.fixed_smem32 != 0 || e.probs.size() > 1;
+  // vector kernels: up to four chunks an item, so that the descriptor loads, the arrival and its fence
+  // come once in about 4,096 nodes (update of 30 problems of 32^3 ... 96^3: 170 -> 118 us)
+  for (int want = shared ? 4 : 1;; want /= 2) {
+    long long n = 0;
+    for (Prob& p : e.probs) {
+      p.vmerge = want;
+      p.n_vitems = (p.n_chunks + want - 1) / want;
+      n += p.n_vitems;
+    }
+    if (want == 1 || n >= 8LL * e.sm_count) break;
+  }
   for (int want = shared ? 32 : 1;; want /= 2) {
     long long n = 0;
     for (Prob& p : e.probs) {
@@ -146,7 +157,7 @@ int engine_set_problems(Engine& e, const std::vector<Prob>& probs, std::string* 
     p.item0_vec = nv;
     na += p.n_tiles;
     nf += p.fn_items;
-    nv += p.n_chunks;
+    nv += p.n_vitems;
     smem32 = std::max(smem32, apply_smem_bytes(p.fx, p.fy, 4));
     smem64 = std::max(smem64, apply_smem_bytes(p.tx, p.ty, 8));
     smemff = std::max(smemff, apply_smem_bytes_ff(p.tx, p.ty));
@@ -162,7 +173,7 @@ int engine_set_problems(Engine& e, const std::vector<Prob>& probs, std::string* 
   for (int i = 0; i < (int)e.probs.size(); ++i) {
     for (long long t = 0; t < e.probs[i].n_tiles; ++t) item[e.probs[i].item0_apply + t] = i;
     for (long long t = 0; t < e.probs[i].fn_items; ++t) fitem[e.probs[i].item0_f32 + t] = i;
-    for (long long t = 0; t < e.probs[i].n_chunks; ++t) vitem[e.probs[i].item0_vec + t] = i;
+    for (long long t = 0; t < e.probs[i].n_vitems; ++t) vitem[e.probs[i].item0_vec + t] = i;
   }
   const long long counts[3] = {na, nv, nf};
   if (e.fixed_smem32) {
@@ -186,7 +197,7 @@ int engine_set_problems(Engine& e, const std::vector<Prob>& probs, std::string* 
     const int r64 = apply_resident_blocks(8, e.bd.apply_threads, e.bd.smem64);
     e.bd.blocks32 = (int)std::max(1LL, std::min<long long>(nf, (long long)e.sm_count * r32));
     e.bd.blocks64 = (int)std::max(1LL, std::min<long long>(na, (long long)e.sm_count * r64));
-    e.bd.vec_blocks = (int)std::max(1LL, std::min<long long>(nv, (long long)e.sm_count * 8));
+    e.bd.vec_blocks = (int)std::max(1LL, std::min<long long>(nv, (long long)e.sm_count * 32));
     bool fits = !e.probs.empty();
     for (const Prob& p : e.probs) fits = fits && apply_nohalo_fits(p);
     e.bd.nohalo64 = fits ? 1 : 0;

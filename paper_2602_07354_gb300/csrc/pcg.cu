@@ -54,12 +54,12 @@ __device__ double total_of(const double* slot, int n, double* red) {
   return block_sum(v, red);
 }
 
-// Thread 0 publishes this item's partials; true in every thread of the problem's last item.
-__device__ bool publish_item(const Prob& P, int chunk, const double* vals, int nvals, unsigned int* ctr, int* s_last) {
+// Publishes the partials this block has written; true in every thread of the problem's last item.
+__device__ bool arrive_item(const Prob& P, unsigned int* ctr, int* s_last) {
+  __syncthreads();
   if (threadIdx.x == 0) {
-    for (int q = 0; q < nvals; ++q) P.parts[q * P.parts_stride + chunk] = vals[q];
     __threadfence();
-    *s_last = atomicAdd(ctr, 1u) == (unsigned)(P.n_chunks - 1);
+    *s_last = atomicAdd(ctr, 1u) == (unsigned)(P.n_vitems - 1);
   }
   __syncthreads();
   return *s_last != 0;
@@ -120,8 +120,7 @@ __global__ void k_pcg_init(const Prob* __restrict__ probs, const int* __restrict
   for (long long item = blockIdx.x; item < n_items; item += gridDim.x) {
     const Prob& P = probs[vitem_prob[item]];
     if (!P.st->needs_init) continue;  // only problems set up since their last start
-    const int chunk = (int)(item - P.item0_vec);
-    const long long N = P.N, n0 = (long long)chunk * P.chunk, n1 = min(n0 + P.chunk, N);
+    const long long N = P.N;
     const int nx = P.nx, ny = P.ny, nz = P.nz;
     Tv* __restrict__ g = reinterpret_cast<Tv*>(P.g);
     Tv* __restrict__ h = reinterpret_cast<Tv*>(P.h);
@@ -132,47 +131,53 @@ __global__ void k_pcg_init(const Prob* __restrict__ probs, const int* __restrict
     const int32_t* __restrict__ phase = P.phase;
     const double* __restrict__ sig = P.sig;
     const Tv* __restrict__ minv = reinterpret_cast<const Tv*>(P.minv);
-    DotAcc<Tv> zg, gg2;
-    DotAcc<double> bb;
-    for (long long n = n0 + threadIdx.x; n < n1; n += kVecThreads) {
-      const int i = (int)(n % nx), j = (int)((n / nx) % ny), k = (int)(n / ((long long)nx * ny));
-      double b[3] = {0, 0, 0};
+    const int c0 = (int)(item - P.item0_vec) * P.vmerge, c1 = min(c0 + P.vmerge, P.n_chunks);
+    for (int chunk = c0; chunk < c1; ++chunk) {
+      const long long n0 = (long long)chunk * P.chunk, n1 = min(n0 + P.chunk, N);
+      DotAcc<Tv> zg, gg2;
+      DotAcc<double> bb;
+      for (long long n = n0 + threadIdx.x; n < n1; n += kVecThreads) {
+        const int i = (int)(n % nx), j = (int)((n / nx) % ny), k = (int)(n / ((long long)nx * ny));
+        double b[3] = {0, 0, 0};
 #pragma unroll
-      for (int a = 0; a < 8; ++a) {
-        const int ax = a & 1, ay = (a >> 1) & 1, az = (a >> 2) & 1;
-        const long long e = (long long)wrapi(i - ax, nx) +
-                            (long long)nx * (wrapi(j - ay, ny) + (long long)ny * wrapi(k - az, nz));
-        const int ph = phase[e];
-        if (ph < 0) continue;
-        const double* S = sig + 6 * (long long)ph;
-        const double sx = 0.25 * (2 * ax - 1), sy = 0.25 * (2 * ay - 1), sz = 0.25 * (2 * az - 1);
-        b[0] += S[0] * sx + S[5] * sy + S[4] * sz;
-        b[1] += S[5] * sx + S[1] * sy + S[3] * sz;
-        b[2] += S[4] * sx + S[3] * sy + S[2] * sz;
-      }
-      Tv gv[3], zv[3];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        gv[c] = (Tv)b[c];
-        bb.add(b[c], b[c]);
-        gg2.add(gv[c], gv[c]);
-      }
-      jacobi_apply(minv, N, n, gv, zv);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        w[c * N + n] = 0.0;
-        if (w_hi) {
-          w_hi[c * N + n] = 0.f;
-          w_lo[c * N + n] = 0.f;
+        for (int a = 0; a < 8; ++a) {
+          const int ax = a & 1, ay = (a >> 1) & 1, az = (a >> 2) & 1;
+          const long long e = (long long)wrapi(i - ax, nx) +
+                              (long long)nx * (wrapi(j - ay, ny) + (long long)ny * wrapi(k - az, nz));
+          const int ph = phase[e];
+          if (ph < 0) continue;
+          const double* S = sig + 6 * (long long)ph;
+          const double sx = 0.25 * (2 * ax - 1), sy = 0.25 * (2 * ay - 1), sz = 0.25 * (2 * az - 1);
+          b[0] += S[0] * sx + S[5] * sy + S[4] * sz;
+          b[1] += S[5] * sx + S[1] * sy + S[3] * sz;
+          b[2] += S[4] * sx + S[3] * sy + S[2] * sz;
         }
-        g[c * N + n] = gv[c];
-        z[c * N + n] = zv[c];
-        h[c * N + n] = zv[c];
-        zg.add(zv[c], gv[c]);
+        Tv gv[3], zv[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          gv[c] = (Tv)b[c];
+          bb.add(b[c], b[c]);
+          gg2.add(gv[c], gv[c]);
+        }
+        jacobi_apply(minv, N, n, gv, zv);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          w[c * N + n] = 0.0;
+          if (w_hi) {
+            w_hi[c * N + n] = 0.f;
+            w_lo[c * N + n] = 0.f;
+          }
+          g[c * N + n] = gv[c];
+          z[c * N + n] = zv[c];
+          h[c * N + n] = zv[c];
+          zg.add(zv[c], gv[c]);
+        }
       }
+      const double vals[3] = {block_total(zg, red), block_total(bb, red), block_total(gg2, red)};
+      if (threadIdx.x == 0)
+        for (int q = 0; q < 3; ++q) P.parts[q * P.parts_stride + chunk] = vals[q];
     }
-    const double vals[3] = {block_total(zg, red), block_total(bb, red), block_total(gg2, red)};
-    if (publish_item(P, chunk, vals, 3, &P.st->ctr[1], &s_last)) {
+    if (arrive_item(P, &P.st->ctr[1], &s_last)) {
       const double s_zg = total_of(P.parts, P.n_chunks, red);
       const double s_bb = total_of(P.parts + P.parts_stride, P.n_chunks, red);
       const double s_gg = total_of(P.parts + 2 * P.parts_stride, P.n_chunks, red);
@@ -339,30 +344,27 @@ __device__ __forceinline__ void update_items(const Prob* __restrict__ probs, con
   __shared__ double buf[2 * kVecThreads];
   __shared__ int s_last;
   constexpr bool kMixed = sizeof(Tv) == 4;
-  const long long n_items = ONE ? one.n_chunks : counts[1];
+  const long long n_items = ONE ? one.n_vitems : counts[1];
   for (long long item = blockIdx.x; item < n_items; item += gridDim.x) {
     const Prob& P = ONE ? one : probs[vitem_prob[item]];
     const DevState* cst = P.st;
     if (cst->done || cst->want_check) continue;
-    const int chunk = (int)(item - P.item0_vec);
-    const long long N = P.N, n0 = (long long)chunk * P.chunk, n1 = min(n0 + P.chunk, N);
+    const long long N = P.N;
     const Tv lam = kMixed ? (Tv)cst->lam_hi : (Tv)cst->lambda;
-    DotAcc<Tv> zg, gg2;
     const int V = N % Row<Tv>::V == 0 ? Row<Tv>::V : 1;
-    if (V > 1)
-      update_chunk<Tv, Row<Tv>::V>(P, n0, n1, lam, zg, gg2);
-    else
-      update_chunk<Tv, 1>(P, n0, n1, lam, zg, gg2);
-    const double v = block_total2(zg, gg2, buf, min(kVecThreads, ((int)(n1 - n0) + V - 1) / V));
-    if (threadIdx.x == 0) P.parts[chunk] = v;
-    if (threadIdx.x == 32) P.parts[P.parts_stride + chunk] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      __threadfence();
-      s_last = atomicAdd(&P.st->ctr[2], 1u) == (unsigned)(P.n_chunks - 1);
+    const int c0 = (int)(item - P.item0_vec) * P.vmerge, c1 = ONE ? c0 + 1 : min(c0 + P.vmerge, P.n_chunks);
+    for (int chunk = c0; chunk < c1; ++chunk) {
+      const long long n0 = (long long)chunk * P.chunk, n1 = min(n0 + P.chunk, N);
+      DotAcc<Tv> zg, gg2;
+      if (V > 1)
+        update_chunk<Tv, Row<Tv>::V>(P, n0, n1, lam, zg, gg2);
+      else
+        update_chunk<Tv, 1>(P, n0, n1, lam, zg, gg2);
+      const double v = block_total2(zg, gg2, buf, min(kVecThreads, ((int)(n1 - n0) + V - 1) / V));
+      if (threadIdx.x == 0) P.parts[chunk] = v;
+      if (threadIdx.x == 32) P.parts[P.parts_stride + chunk] = v;
     }
-    __syncthreads();
-    if (s_last) {
+    if (arrive_item(P, &P.st->ctr[2], &s_last)) {
       DotAcc<double> a, b;
       for (int i = threadIdx.x; i < P.n_chunks; i += kVecThreads) {
         a.s += __ldcg(P.parts + i);
@@ -451,13 +453,12 @@ template <typename Tv, bool ONE>
 __global__ void __launch_bounds__(kVecThreads, sizeof(Tv) == 8 ? 4 : 3)
     k_pcg_direction(const Prob* __restrict__ probs, const int* __restrict__ vitem_prob,
                     const long long* __restrict__ counts, const __grid_constant__ Prob one) {
-  const long long n_items = ONE ? one.n_chunks : counts[1];
+  const long long n_items = ONE ? one.n_vitems : counts[1];
   for (long long item = blockIdx.x; item < n_items; item += gridDim.x) {
     const Prob& P = ONE ? one : probs[vitem_prob[item]];
     const DevState* cst = P.st;
     if (cst->done || cst->want_check) continue;
-    const int chunk = (int)(item - P.item0_vec);
-    const long long n0 = (long long)chunk * P.chunk, n1 = min(n0 + P.chunk, P.N);
+    const long long per = (long long)P.chunk * P.vmerge, n0 = (item - P.item0_vec) * per, n1 = min(n0 + per, P.N);
     const Tv gam = sizeof(Tv) == 4 ? (Tv)cst->gam_f : (Tv)cst->gamma;
     const bool w_due = !cst->w_applied;
     if (P.N % Row<Tv>::V == 0)
@@ -481,8 +482,8 @@ __global__ void __launch_bounds__(kVecThreads)
     const DevState* st = P.st;
     if (gate == GATE_REPLACE && (st->done || !replacement_due(st))) continue;
     if (gate == GATE_FINALIZE && (!st->done || st->finalized)) continue;
-    const int chunk = (int)(item - P.item0_vec);
-    const long long N = P.N, n0 = (long long)chunk * P.chunk, n1 = min(n0 + P.chunk, N);
+    const long long N = P.N, per = (long long)P.chunk * P.vmerge;
+    const long long n0 = (item - P.item0_vec) * per, n1 = min(n0 + per, N);
     if (!st->w_applied && (gate == GATE_REPLACE || st->done)) direction_chunk<Tv, 1, false>(P, n0, n1, true, Tv(0));
     if constexpr (sizeof(Tv) == 4) {  // a thread reads back its own nodes
       for (long long n = n0 + threadIdx.x; n < n1; n += kVecThreads)
