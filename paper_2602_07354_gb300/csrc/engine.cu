@@ -125,7 +125,7 @@ static void merge_chunks(Engine& e) {
       p.n_vitems = (p.n_chunks + want - 1) / want;
       n += p.n_vitems;
     }
-    if (want == 1 || n >= 8LL * e.sm_count) break;
+    if (want == 1 || n >= 4LL * e.sm_count) break;
   }
   for (int want = shared ? 32 : 1;; want /= 2) {
     long long n = 0;
