@@ -591,6 +591,7 @@ __global__ void __launch_bounds__(MAXT, MINB)
   for (long long item = blockIdx.x; item < n_items; item += gridDim.x) {
     const Prob& P = ONE ? one : probs[item_prob[item]];
     if (gate != GATE_NONE && gate_skips(gate, P.st)) continue;  // uniform over the block
+    if (kFF && EPI == EPI_STORE_DOT && thin_tiling(P.tx, P.ty, P.kc)) continue;  // k_apply_thin's
     const int nx = P.nx, ny = P.ny, nz = P.nz;
     const long long N = P.N;
     const int tx = kF32 ? P.fx : P.tx, ty = kF32 ? P.fy : P.ty, kc = kF32 ? P.fkc : P.kc;
@@ -1104,6 +1105,131 @@ __global__ void __launch_bounds__(MAXT, MINB)
   }
 }
 
+// The double-float product h -> Ah on tiles of one node layer (small grids, whose tiles are cut that
+// thin to fill the SMs): the two voxel layers that meet at the nodes are computed side by side by the
+// two halves of the block instead of one after the other, as a layer's latency (about 6 us, nearly the
+// same for 6 warps as for 12) sets the time.  Each half leaves its corner forces on the node layer in
+// its own buffer and a node gathers eight records.  20^3 product 18.6 -> 14.5 us.
+template <bool ONE>
+__global__ void __launch_bounds__(kMaxThreadsF64, 1)
+    k_apply_thin(const Prob* __restrict__ probs, const int* __restrict__ item_prob, const long long* __restrict__ counts,
+                 int post, int gate, const __grid_constant__ Prob one) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ double red[32];
+  __shared__ int s_last;
+  const int t = threadIdx.x;
+  const long long n_items = ONE ? one.n_tiles : counts[0];
+  for (long long item = blockIdx.x; item < n_items; item += gridDim.x) {
+    const Prob& P = ONE ? one : probs[item_prob[item]];
+    if (gate != GATE_NONE && gate_skips(gate, P.st)) continue;  // uniform over the block
+    if (!ONE && !thin_tiling(P.tx, P.ty, P.kc)) continue;       // k_apply's
+    const int nx = P.nx, ny = P.ny, nz = P.nz, tx = P.tx, ty = P.ty;
+    const long long N = P.N, plane = (long long)nx * ny;
+    const int NXv = tx + 1, NV = NXv * (ty + 1), NXp = tx + 2, NP = NXp * (ty + 2);
+    float4* const rxy = reinterpret_cast<float4*>(smem_raw);  // [3 layers][NP]
+    float2* const rz = reinterpret_cast<float2*>(rxy + 3 * NP);
+    ff* const Fc = reinterpret_cast<ff*>(smem_raw + plane_ring_bytes(NP, 8));
+    const int tile = (int)(item - P.item0_apply);
+    const int i0 = (tile % P.tiles_x) * tx, j0 = ((tile / P.tiles_x) % P.tiles_y) * ty;
+    const int k0 = tile / (P.tiles_x * P.tiles_y);
+    const double* __restrict__ u = reinterpret_cast<const double*>(P.h);
+    double* __restrict__ y = reinterpret_cast<double*>(P.Ah);
+    // column of this thread; the block's second half takes the upper voxel layer
+    const int half = t >= kMaxThreadsF64 / 2, col = t - half * (kMaxThreadsF64 / 2);
+    const int vi = col % NXv, vj = col / NXv, rec = vj * NXp + vi;
+    const bool has_vox = col < NV;
+    int ph = -1;
+    if (has_vox)
+      ph = P.phase[wrapi(k0 - 1 + half, nz) * plane + (long long)wrapi(j0 - 1 + vj, ny) * nx + wrapi(i0 - 1 + vi, nx)];
+    for (int s = t; s < 3 * NP; s += kMaxThreadsF64) {
+      const int l = s / NP, r = s - l * NP;
+      const long long e =
+          wrapi(k0 - 1 + l, nz) * plane + (long long)wrapi(j0 - 1 + r / NXp, ny) * nx + wrapi(i0 - 1 + r % NXp, nx);
+      const ff px = split_double(u[e]), py = split_double(u[N + e]), pz = split_double(u[2 * N + e]);
+      rxy[s] = make_float4(px.hi, py.hi, px.lo, py.lo);
+      rz[s] = make_float2(pz.hi, pz.lo);
+    }
+    __syncthreads();
+    if (has_vox) {
+      P2<ff> m_xy[4], cor_xy[4];
+      ff m_z[4], cor_z[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        m_xy[q] = pk2(ff(0), ff(0));
+        m_z[q] = ff(0);
+      }
+      const ff* coef = CoefOf<ff>::table(P) + CoefOf<ff>::base;
+      const ff* K = ph >= 0 ? coef + (long long)ph * CoefOf<ff>::stride : nullptr;
+      if (K != nullptr && __ldg(reinterpret_cast<const float*>(K + kCoefSolid0)) != 0.f) {
+        P2<ff> lo_xy[4], up_xy[4];
+        ff lo_z[4], up_z[4];
+        face_forward_ff(rxy + half * NP + rec, rz + half * NP + rec, NXp, lo_xy, lo_z);
+        face_forward_ff(rxy + (half + 1) * NP + rec, rz + (half + 1) * NP + rec, NXp, up_xy, up_z);
+        ff W[3][8], F[3][8];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const P2<ff> a = lo_xy[q] + up_xy[q], b = up_xy[q] - lo_xy[q];
+          W[0][q] = lane0(a); W[1][q] = lane1(a); W[2][q] = lo_z[q] + up_z[q];
+          W[0][q + 4] = lane0(b); W[1][q + 4] = lane1(b); W[2][q + 4] = up_z[q] - lo_z[q];
+        }
+        modal_forces(W, LazyK{K + kCoefMode0}, K, F);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {  // the lower layer's upper face, the upper layer's lower face
+          const P2<ff> a = pk2(F[0][q], F[1][q]), b = pk2(F[0][q + 4], F[1][q + 4]);
+          m_xy[q] = half ? a - b : a + b;
+          m_z[q] = half ? F[2][q] - F[2][q + 4] : F[2][q] + F[2][q + 4];
+        }
+      }
+      face_bf_t(m_xy, cor_xy);
+      face_bf_t(m_z, cor_z);
+#pragma unroll
+      for (int b = 0; b < 4; ++b) st_face_ff(Fc, NV, half * 4 * NV + b * NV + col, cor_xy[b], cor_z[b]);
+    }
+    __syncthreads();
+    DotAcc<ff> dot;
+    const int i = i0 + vi - 1, j = j0 + vj - 1;
+    if (!half && has_vox && vi >= 1 && vj >= 1 && i < nx && j < ny) {
+      P2<ff> oxy = pk2(ff(0), ff(0));
+      ff oz = ff(0);
+#pragma unroll
+      for (int b = 3; b >= 0; --b)
+#pragma unroll
+        for (int l = 0; l < 2; ++l) {
+          P2<ff> xy;
+          ff z;
+          ld_face_ff(Fc, NV, col + l * 4 * NV + b * NV - (b & 1) - NXv * (b >> 1), xy, z);
+          oxy = oxy + xy;
+          oz = oz + z;
+        }
+      P2<ff> hxy;
+      ff hz;
+      ld_node_ff(rxy + NP + rec, rz + NP + rec, hxy, hz);
+      const long long n = k0 * plane + (long long)j * nx + i;
+      const ff out[3] = {lane0(oxy), lane1(oxy), oz};
+#pragma unroll
+      for (int c = 0; c < 3; ++c) y[c * N + n] = (double)out[c];
+      dot.add(lane0(hxy), out[0]);
+      dot.add(lane1(hxy), out[1]);
+      dot.add(hz, out[2]);
+    }
+    const double b0 = block_total(dot, red);
+    if (t == 0) {
+      P.parts[tile] = b0;
+      __threadfence();
+      s_last = atomicAdd(&P.st->ctr[0], 1u) == (unsigned)(P.n_tiles - 1);
+    }
+    __syncthreads();
+    if (s_last) {
+      const double s0 = total_of(P.parts, P.n_tiles, red);
+      if (t == 0) {
+        P.st->ctr[0] = 0u;
+        post_scalars(P.st, post, s0, 0.0);
+      }
+    }
+    __syncthreads();
+  }
+}
+
 // Tile-edge pass of the FP64 operator without recomputed halo.  The operator leaves a tile's
 // first node column and row (ni = 0 or nj = 0) with its own voxels' forces only, and exports per
 // node layer the forces its last voxel column and row put on the nodes just beyond it, into z
@@ -1233,6 +1359,19 @@ cudaError_t launch_t(const BatchDev& b, int role, int post, int gate, cudaStream
   return e;
 }
 
+template <bool ONE>
+cudaError_t launch_thin(const BatchDev& b, int post, int gate, cudaStream_t s) {
+  static std::once_flag once;
+  static cudaError_t set_err = cudaSuccess;
+  std::call_once(once, [&] {
+    set_err = cudaFuncSetAttribute(k_apply_thin<ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kApplySmemMax);
+  });
+  if (set_err != cudaSuccess) return set_err;
+  if (b.smemff > kApplySmemMax) return cudaErrorInvalidValue;
+  k_apply_thin<ONE><<<b.blocks64, kMaxThreadsF64, b.smemff, s>>>(b.probs, b.item_prob, b.counts, post, gate, b.one);
+  return cudaGetLastError();
+}
+
 template <typename Tvec, int EPI, bool AFFINE>
 cudaError_t launch_ff(const BatchDev& b, int role, int post, int gate, cudaStream_t s) {
   return b.single ? launch_t<double, ff, Tvec, EPI, AFFINE, false, true>(b, role, post, gate, s)
@@ -1245,6 +1384,12 @@ cudaError_t launch_apply(const BatchDev& b, int kind, int post, int gate, cudaSt
   if (b.ff64) {  // FP64 products in double-float arithmetic
     switch (kind) {
       case AK_F64_DOT:
+        // tiles of one layer and at most half a block of columns go to the thin form, each kernel passing
+        // over the other's problems
+        if (b.thin) {
+          const cudaError_t e = b.single ? launch_thin<true>(b, post, gate, s) : launch_thin<false>(b, post, gate, s);
+          if (e != cudaSuccess || !b.thick) return e;
+        }
         // the recomputed-halo form: its halo columns cost the FP32 pipe less than the no-halo
         // form's edge pass and layout cost it (173 against 223 us per product at 100^3); the
         // no-halo form pays for native FP64, whose halo columns would occupy the FP64 pipe
@@ -1372,7 +1517,8 @@ Tiling make_tiling(const Geo& g, int elem_bytes, int sm_count, int tx_hint, int 
         const long long blocks = n_tiles < slots ? n_tiles : slots;
         const long long rounds = (n_tiles + slots - 1) / slots;
         const double per_sm_tiles = (double)rounds * std::min<long long>(R, (n_tiles + sm_count - 1) / sm_count);
-        double cost = per_sm_tiles * (kc + 1 + 0.5) * (threads + 64);
+        // (a thin tile's two layers run side by side)
+        double cost = per_sm_tiles * ((thin_tiling(tx, ty, kc) ? 1 : kc + 1) + 0.5) * (threads + 64);
         if (n_tiles > (1LL << 30)) continue;
         if (cost < best_cost * 0.999) {
           best_cost = cost;

@@ -389,6 +389,7 @@ struct BatchDev {
   int single;              // the batch is one problem: its descriptor also goes as a kernel argument
   Prob one;
   int nohalo64;            // native FP64 iteration operator without recomputed x/y halo (+ edge pass)
+  int thin, thick;         // the problems' FP64 tilings: some are thin (k_apply_thin), some are not
   int ff64;                // FP64 products in double-float arithmetic (ELAS_FP64_OP_PAIRED)
 };
 
@@ -409,6 +410,11 @@ enum ApplyKind {
 
 size_t apply_smem_bytes(int tx, int ty, int elem_bytes);
 size_t apply_smem_bytes_ff(int tx, int ty);
+// Tiles of one node layer whose columns fit half a block: the double-float product takes their two
+// voxel layers side by side.
+__host__ __device__ constexpr bool thin_tiling(int tx, int ty, int kc) {
+  return kc == 1 && (tx + 1) * (ty + 1) <= kMaxThreadsF64 / 2;
+}
 constexpr int kBlocksF32 = 2;  // resident blocks per SM of the FP32 product
 Tiling tiling_of(const Geo& g, int tx, int ty, int kc);
 Tiling make_tiling(const Geo& g, int elem_bytes, int sm_count, int tx_hint = 0, int ty_hint = 0, int kc_hint = 0);

@@ -149,6 +149,7 @@ int engine_set_problems(Engine& e, const std::vector<Prob>& probs, std::string* 
   merge_chunks(e);
   long long na = 0, nf = 0, nv = 0;
   size_t smem32 = 0, smem64 = 0, smemff = 0;
+  e.bd.thin = e.bd.thick = e.fixed_smem32 != 0;  // a fixed launch shape holds either
   for (size_t i = 0; i < e.probs.size(); ++i) {
     Prob& p = e.probs[i];
     p.st = e.d_states + i;
@@ -160,6 +161,10 @@ int engine_set_problems(Engine& e, const std::vector<Prob>& probs, std::string* 
     nv += p.n_vitems;
     smem32 = std::max(smem32, apply_smem_bytes(p.fx, p.fy, 4));
     smem64 = std::max(smem64, apply_smem_bytes(p.tx, p.ty, 8));
+    if (thin_tiling(p.tx, p.ty, p.kc))
+      e.bd.thin = 1;
+    else
+      e.bd.thick = 1;
     smemff = std::max(smemff, apply_smem_bytes_ff(p.tx, p.ty));
   }
   if (na > e.cap_apply || nf > e.cap_apply || nv > e.cap_vec) {
@@ -251,7 +256,7 @@ int engine_solve(Engine& e, const std::vector<SolveSetup>& setups, int K, int* l
     for (int i = 0; i < n; ++i) all_done &= e.h_states[i].done != 0;
     if (all_done || b >= max_batches) break;
     if ((c = cudaGraphLaunch(e.exec, s)) != cudaSuccess) return cfail(err, c, "cudaGraphLaunch");
-    L += 3 * K + 2;
+    L += (3 + (!e.mixed && e.bd.ff64 && e.bd.thin && e.bd.thick)) * K + 2;
   }
   if ((c = launch_w_finish(e.bd, e.mixed, GATE_NONE, s)) != cudaSuccess) return cfail(err, c, "w finish");
   L += 1;
