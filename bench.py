@@ -37,18 +37,19 @@ UNIT = "voxel-iter/s"
 E6 = np.array([0.0, 0.0, 1e-3, 0.0, 0.0, 0.0])
 TOL = 1e-8
 # Algorithmic HBM bytes per voxel per PCG iteration (each vector read/written once per kernel):
-#   FP64: apply 52 (h, ids, Ah) + update 216 (w,h,g,Ah,Minv in; w,g,z out) + direction 72 = 340
-#   mixed: apply 28 + update 132 (w as a float pair, FP32 vectors and Minv) + direction 36 = 196
-BYTES_PER_VOXEL_ITER = {"fp64": 340, "mixed": 196}
-# Algorithmic flops per voxel of the modal element product + node gather: 30 MUL + 108 FMA in the
-# 6x6/5x5/3x3 mode products, 186 adds (transform 72 + 72, strain/force assembly 21, gather 21)
-APPLY_FLOPS_PER_VOXEL = 432
+#   FP64: apply 52 (h, ids, Ah) + update 144 (g,Ah,Minv in; g,z out) + direction 120 (z,h,w in; h,w
+#   out) = 316
+#   mixed: apply 28 + update 72 + direction 84 (w as a float pair) = 184
+BYTES_PER_VOXEL_ITER = {"fp64": 316, "mixed": 184}
+# Algorithmic flops per voxel of the modal element product + node gather: 24 MUL + 96 FMA in the
+# 6x6/5x5/3x3 mode products, 180 adds (transform 72 + 72, strain/force assembly 15, gather 21)
+APPLY_FLOPS_PER_VOXEL = 396
 # The FP64 product in double-float arithmetic (ELAS_FP64_OP_PAIRED, the default) performs these
-# FP32 operations per voxel (each FADD, FMUL and FFMA counted once): 126 pair sums x 8 (TwoSum 6 + 2),
-# 138 terms of the 30 symmetric-product rows (first term of a row 4: product, its rounding error and
-# two cross terms; every other term 12: those 4, TwoSum 6, 2 error sums), 30 row renormalisations x 3,
+# FP32 operations per voxel (each FADD, FMUL and FFMA counted once): 120 pair sums x 8 (TwoSum 6 + 2),
+# 120 terms of the 24 symmetric-product rows (first term of a row 4: product, its rounding error and
+# two cross terms; every other term 12: those 4, TwoSum 6, 2 error sums), 24 row renormalisations x 3,
 # and the h.Ah terms of the node (3 x 12)
-PAIRED_OPS_PER_VOXEL = 126 * 8 + 30 * 4 + 108 * 12 + 30 * 3 + 3 * 12
+PAIRED_OPS_PER_VOXEL = 120 * 8 + 24 * 4 + 96 * 12 + 24 * 3 + 3 * 12
 APPLY_BYTES_PER_VOXEL = {"fp64": 52, "mixed": 28}
 # FP64 pipe: 2 DFMA per clock per SM on GB300 (1.25 TFLOP/s nominal at 2070 MHz, 152 SMs)
 FP64_FMA_PER_CLK_PER_SM = 2

@@ -562,13 +562,14 @@ __device__ void post_scalars(DevState* st, int post, double s0, double s1) {
 // node tile and a chunk of kc node layers of its problem.  Thread t < (tx+1)(ty+1) owns voxel
 // column (vi, vj) of the tile (global voxel i0-1+vi, j0-1+vj) and marches it along z, keeping
 // in registers the modes of its lower face and the forces its previous voxel left on the shared
-// face (the double-float form keeps those forces in a per-thread shared-memory slot); thread
-// t < tx*ty owns node (ni, nj).  Shared memory: a 4-slot ring of node layers ((tx+2)(ty+2)
-// records of x, y, z and the phase id of the voxel whose low corner is that node) filled by
-// cp.async three layers ahead, so neither the node values nor the phase ids of a layer are waited
-// for in the layer that uses them, and two buffers of per-column face corner forces
-// ([corner][column] records).  One barrier per layer.  Each item publishes its own partial sums;
-// the problem's last item sums them in tile order.
+// face (the double-float form keeps those forces in a per-thread shared-memory slot), and owns the
+// node at the column's low corner if the tile holds it.  Shared memory: a 4-slot ring of node layers
+// ((tx+2)(ty+2) records of x, y, z and the phase id of the voxel whose low corner is that node;
+// planes in FP32 and double-float) filled by cp.async three layers ahead, so neither the node values
+// nor the phase ids of a layer are waited for in the layer that uses them, and two buffers of
+// per-column face corner forces ([corner][column] records).  One barrier per layer.  Each item (in
+// FP32 each z-chunk of an item) publishes its own partial sums; the problem's last item sums them in
+// order.  ONE: a single problem, whose descriptor is the argument itself.
 template <typename Tin, typename T, typename Tvec, int EPI, bool AFFINE, int MAXT, int MINB, bool NOHALO = false,
           bool ONE = false>
 __global__ void __launch_bounds__(MAXT, MINB)
@@ -815,225 +816,225 @@ __global__ void __launch_bounds__(MAXT, MINB)
       // the layer's two independent halves: (gather) split layer kv+2 and gather layer kv-1 from the face
       // forces, (compute) the element products of voxel layer kv
       auto gather_half = [&]() {
-      cp_async_wait_ahead();  // this thread's copies of layer kv+2 have landed
-      if (kFF && kv + 2 <= k1) split_slot((L + 2) % kRing);
-      if (kv > k0 && has_node) {
-        // node (ni,nj) of layer kv-1 is corner 3 of column (ni,nj), 2 of (ni+1,nj), 1 of
-        // (ni,nj+1) and 0 of (ni+1,nj+1)
-        const T* fp = Fc + ((kv - 1) & 1) * fbuf;
-        P2<T> oxy = pk2(T(0), T(0));
-        T oz = T(0);
+        cp_async_wait_ahead();  // this thread's copies of layer kv+2 have landed
+        if (kFF && kv + 2 <= k1) split_slot((L + 2) % kRing);
+        if (kv > k0 && has_node) {
+          // node (ni,nj) of layer kv-1 is corner 3 of column (ni,nj), 2 of (ni+1,nj), 1 of
+          // (ni,nj+1) and 0 of (ni+1,nj+1)
+          const T* fp = Fc + ((kv - 1) & 1) * fbuf;
+          P2<T> oxy = pk2(T(0), T(0));
+          T oz = T(0);
 #pragma unroll
-        for (int b = 3; b >= 0; --b) {
-          P2<T> xy;
-          T z;
-          if constexpr (kPlanes) {
-            ld_face_ff(Fc, NV, t + (((kv - 1) & 1) * 4 * NV + b * NV - (b & 1) - NXv * (b >> 1)), xy, z);
-          } else {
-            ld_xyz(fp + goff[b], xy, z);
+          for (int b = 3; b >= 0; --b) {
+            P2<T> xy;
+            T z;
+            if constexpr (kPlanes) {
+              ld_face_ff(Fc, NV, t + (((kv - 1) & 1) * 4 * NV + b * NV - (b & 1) - NXv * (b >> 1)), xy, z);
+            } else {
+              ld_xyz(fp + goff[b], xy, z);
+            }
+            oxy = oxy + xy;
+            oz = oz + z;
           }
-          oxy = oxy + xy;
-          oz = oz + z;
-        }
-        const T out[3] = {lane0(oxy), lane1(oxy), oz};
-        const long long n = nrow;
-        if (EPI == EPI_STORE || EPI == EPI_STORE_DOT) {
+          const T out[3] = {lane0(oxy), lane1(oxy), oz};
+          const long long n = nrow;
+          if (EPI == EPI_STORE || EPI == EPI_STORE_DOT) {
 #pragma unroll
-          for (int c = 0; c < 3; ++c) y[c * N + n] = (Tst)out[c];
-          if (EPI == EPI_STORE_DOT && (!NOHALO || (ni >= 1 && nj >= 1))) {
-            dot0.add(hown[0], out[0]);
-            dot0.add(hown[1], out[1]);
-            dot0.add(hown[2], out[2]);
-          }
-        } else if (EPI == EPI_RESIDUAL) {
-          Tvec gv[3], zv[3];
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            gv[c] = (Tvec)out[c];
-            dot1.add((double)out[c], (double)out[c]);
-          }
-          block_jacobi_apply(minv_v, N, n, gv, zv);
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            g_v[c * N + n] = gv[c];
-            z_v[c * N + n] = zv[c];
-            dot0r.add((double)zv[c], (double)gv[c]);
-          }
-        } else {  // EPI_NORM, EPI_STORE_NORM
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            const double r = (double)out[c];
-            if (EPI == EPI_STORE_NORM) y[c * N + n] = (Tst)r;
-            dot1.add(r, r);
-          }
-        }
-      }
-      if (EPI == EPI_STORE_DOT && kv < k1 && has_node) {
-        P2<T> hxy;
-        if constexpr (kPlanes)
-          ld_node_ff(rxy + (L % kRing) * NP + face_rec, rz + (L % kRing) * NP + face_rec, hxy, hown[2]);
-        else
-          ld_xyz(hrec0 + (L % kRing) * slot_elems, hxy, hown[2]);
-        hown[0] = lane0(hxy);
-        hown[1] = lane1(hxy);
-      }
-      };
-      auto compute_half = [&]() {
-      if (kv < k1 && has_vox && own_col) {
-        const bool own = own_col;
-        P2<T> Vup_xy[4];
-        T Vup_z[4];
-        if constexpr (kPlanes) {
-          if (L == 0) face_forward_ff(rxy + face_rec, rz + face_rec, NXp, Vlo_xy, Vlo_z);
-          const int at = ((L + 1) % kRing) * NP + face_rec;
-          face_forward_ff(rxy + at, rz + at, NXp, Vup_xy, Vup_z);
-        } else {
-          if (L == 0) face_forward<RS>(face0, row, Vlo_xy, Vlo_z);
-          face_forward<RS>(face0 + ((L + 1) % kRing) * slot_elems, row, Vup_xy, Vup_z);
-        }
-        P2<T> FL_xy[4], FU_xy[4];
-        T FL_z[4], FU_z[4];
-        int ph = -1;
-        if constexpr (kPlanes)
-          ph = rid[(L % kRing) * NP + face_rec];
-        else if (own)
-          ph = *reinterpret_cast<const int*>(face0 + (L % kRing) * slot_elems + 3);
-        const T* K = ph >= 0 ? coef + (long long)ph * CoefOf<T>::stride : nullptr;
-        T k0[24];
-        bool solid = false;
-        if constexpr (kKeep) {
-          if (L == 0 && K != nullptr) load_k(K + kCoefMode0, kept);
-          solid = K != nullptr && kept[kCoefSolid0] != T(0);
-        } else if (K != nullptr) {
-          if constexpr (kFF) {
-            solid = __ldg(reinterpret_cast<const float*>(K + kCoefSolid0)) != 0.f;
-          } else {
-            load_k(K + kCoefMode0, k0);
-            solid = k0[kCoefSolid0] != T(0);
-          }
-        }
-        if (solid) {
-          // z stage of the forward transform (x and y components paired)
-          P2<T> Wxy[8];
-          T Wz[8];
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            Wxy[q] = Vlo_xy[q] + Vup_xy[q];
-            Wxy[q + 4] = Vup_xy[q] - Vlo_xy[q];
-            Wz[q] = Vlo_z[q] + Vup_z[q];
-            Wz[q + 4] = Vup_z[q] - Vlo_z[q];
-          }
-          T W[3][8], F[3][8];
-#pragma unroll
-          for (int m = 0; m < 8; ++m) {
-            W[0][m] = lane0(Wxy[m]);
-            W[1][m] = lane1(Wxy[m]);
-            W[2][m] = Wz[m];
-          }
-          if (AFFINE) {
+            for (int c = 0; c < 3; ++c) y[c * N + n] = (Tst)out[c];
+            if (EPI == EPI_STORE_DOT && (!NOHALO || (ni >= 1 && nj >= 1))) {
+              dot0.add(hown[0], out[0]);
+              dot0.add(hown[1], out[1]);
+              dot0.add(hown[2], out[2]);
+            }
+          } else if (EPI == EPI_RESIDUAL) {
+            Tvec gv[3], zv[3];
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-              W[c][1] += E4[c][0];
-              W[c][2] += E4[c][1];
-              W[c][4] += E4[c][2];
+              gv[c] = (Tvec)out[c];
+              dot1.add((double)out[c], (double)out[c]);
+            }
+            block_jacobi_apply(minv_v, N, n, gv, zv);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+              g_v[c * N + n] = gv[c];
+              z_v[c * N + n] = zv[c];
+              dot0r.add((double)zv[c], (double)gv[c]);
+            }
+          } else {  // EPI_NORM, EPI_STORE_NORM
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+              const double r = (double)out[c];
+              if (EPI == EPI_STORE_NORM) y[c * N + n] = (Tst)r;
+              dot1.add(r, r);
             }
           }
-          if constexpr (kFF)
-            modal_forces(W, LazyK{K + kCoefMode0}, K, F);
-          else if constexpr (kKeep)
-            modal_forces(W, kept, K, F);
-          else
-            modal_forces(W, k0, K, F);
-          // transposed z stage: forces on the lower (this node layer) and upper face
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const P2<T> a = pk2(F[0][q], F[1][q]), b = pk2(F[0][q + 4], F[1][q + 4]);
-            FL_xy[q] = a - b;
-            FU_xy[q] = a + b;
-            FL_z[q] = F[2][q] - F[2][q + 4];
-            FU_z[q] = F[2][q] + F[2][q + 4];
-          }
-        } else {
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            FL_xy[q] = FU_xy[q] = pk2(T(0), T(0));
-            FL_z[q] = FU_z[q] = T(0);
-          }
         }
-        if constexpr (kKeep) {
-          const int pn = rid[((L + 1) % kRing) * NP + face_rec];
-          if (pn != ph && pn >= 0) load_k(coef + (long long)pn * CoefOf<T>::stride + kCoefMode0, kept);
-        }
-        // face of node layer kv: lower-face forces of this voxel + upper-face forces of the one below,
-        // back-transformed to the 4 corners (transposed x and y stages)
-        P2<T> m_xy[4], cor_xy[4];
-        T m_z[4], cor_z[4];
-        if constexpr (kFF) {
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const float4 a = fup[q * fup_plane];
-            FUp_xy[q] = P2<T>{make_float2(a.x, a.y), make_float2(a.z, a.w)};
-          }
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const float4 a = fup[(4 + h) * fup_plane];
-            FUp_z[2 * h] = ff(a.x, a.y);
-            FUp_z[2 * h + 1] = ff(a.z, a.w);
-          }
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          m_xy[q] = FUp_xy[q] + FL_xy[q];
-          m_z[q] = FUp_z[q] + FL_z[q];
-        }
-        face_bf_t(m_xy, cor_xy);
-        face_bf_t(m_z, cor_z);
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
+        if (EPI == EPI_STORE_DOT && kv < k1 && has_node) {
+          P2<T> hxy;
           if constexpr (kPlanes)
-            st_face_ff(Fc, NV, (kv & 1) * 4 * NV + b * NV + vcol, cor_xy[b], cor_z[b]);
+            ld_node_ff(rxy + (L % kRing) * NP + face_rec, rz + (L % kRing) * NP + face_rec, hxy, hown[2]);
           else
-            st_xyz(fcol + (kv & 1) * fbuf + b * 4 * NV, cor_xy[b], cor_z[b]);
+            ld_xyz(hrec0 + (L % kRing) * slot_elems, hxy, hown[2]);
+          hown[0] = lane0(hxy);
+          hown[1] = lane1(hxy);
         }
-        if (NOHALO && own && kv >= kbase && (vi == rx || vj == ry)) {
-          // the tile's last voxel column and row also act on the nodes just beyond the tile: their
-          // corners with a_x = 1 (column) and a_y = 1 (row) go to the edge pass, per node layer
-          Tst* ex = reinterpret_cast<Tst*>(P.z) + 6 * ((long long)tile * P.kc + (kv - kbase)) * (tx + ty);
-          auto put = [&](Tst* d, int b) {
-            d[0] = (Tst)lane0(cor_xy[b]); d[1] = (Tst)lane1(cor_xy[b]); d[2] = (Tst)cor_z[b];
-          };
-          if (vi == rx) {
-            Tst* d = ex + 6 * (vj - 1);
-            put(d, 1);
-            put(d + 3, 3);
+      };
+      auto compute_half = [&]() {
+        if (kv < k1 && has_vox && own_col) {
+          const bool own = own_col;
+          P2<T> Vup_xy[4];
+          T Vup_z[4];
+          if constexpr (kPlanes) {
+            if (L == 0) face_forward_ff(rxy + face_rec, rz + face_rec, NXp, Vlo_xy, Vlo_z);
+            const int at = ((L + 1) % kRing) * NP + face_rec;
+            face_forward_ff(rxy + at, rz + at, NXp, Vup_xy, Vup_z);
+          } else {
+            if (L == 0) face_forward<RS>(face0, row, Vlo_xy, Vlo_z);
+            face_forward<RS>(face0 + ((L + 1) % kRing) * slot_elems, row, Vup_xy, Vup_z);
           }
-          if (vj == ry) {
-            Tst* d = ex + 6 * (ty + vi - 1);
-            put(d, 2);
-            put(d + 3, 3);
+          P2<T> FL_xy[4], FU_xy[4];
+          T FL_z[4], FU_z[4];
+          int ph = -1;
+          if constexpr (kPlanes)
+            ph = rid[(L % kRing) * NP + face_rec];
+          else if (own)
+            ph = *reinterpret_cast<const int*>(face0 + (L % kRing) * slot_elems + 3);
+          const T* K = ph >= 0 ? coef + (long long)ph * CoefOf<T>::stride : nullptr;
+          T k0[24];
+          bool solid = false;
+          if constexpr (kKeep) {
+            if (L == 0 && K != nullptr) load_k(K + kCoefMode0, kept);
+            solid = K != nullptr && kept[kCoefSolid0] != T(0);
+          } else if (K != nullptr) {
+            if constexpr (kFF) {
+              solid = __ldg(reinterpret_cast<const float*>(K + kCoefSolid0)) != 0.f;
+            } else {
+              load_k(K + kCoefMode0, k0);
+              solid = k0[kCoefSolid0] != T(0);
+            }
           }
-        }
+          if (solid) {
+            // z stage of the forward transform (x and y components paired)
+            P2<T> Wxy[8];
+            T Wz[8];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          Vlo_xy[q] = Vup_xy[q];
-          Vlo_z[q] = Vup_z[q];
-        }
-        if constexpr (kFF) {
+            for (int q = 0; q < 4; ++q) {
+              Wxy[q] = Vlo_xy[q] + Vup_xy[q];
+              Wxy[q + 4] = Vup_xy[q] - Vlo_xy[q];
+              Wz[q] = Vlo_z[q] + Vup_z[q];
+              Wz[q + 4] = Vup_z[q] - Vlo_z[q];
+            }
+            T W[3][8], F[3][8];
 #pragma unroll
-          for (int q = 0; q < 4; ++q)
-            fup[q * fup_plane] = make_float4(FU_xy[q].hi.x, FU_xy[q].hi.y, FU_xy[q].lo.x, FU_xy[q].lo.y);
+            for (int m = 0; m < 8; ++m) {
+              W[0][m] = lane0(Wxy[m]);
+              W[1][m] = lane1(Wxy[m]);
+              W[2][m] = Wz[m];
+            }
+            if (AFFINE) {
 #pragma unroll
-          for (int h = 0; h < 2; ++h)
-            fup[(4 + h) * fup_plane] =
-                make_float4(FU_z[2 * h].hi, FU_z[2 * h].lo, FU_z[2 * h + 1].hi, FU_z[2 * h + 1].lo);
-        } else {
+              for (int c = 0; c < 3; ++c) {
+                W[c][1] += E4[c][0];
+                W[c][2] += E4[c][1];
+                W[c][4] += E4[c][2];
+              }
+            }
+            if constexpr (kFF)
+              modal_forces(W, LazyK{K + kCoefMode0}, K, F);
+            else if constexpr (kKeep)
+              modal_forces(W, kept, K, F);
+            else
+              modal_forces(W, k0, K, F);
+            // transposed z stage: forces on the lower (this node layer) and upper face
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const P2<T> a = pk2(F[0][q], F[1][q]), b = pk2(F[0][q + 4], F[1][q + 4]);
+              FL_xy[q] = a - b;
+              FU_xy[q] = a + b;
+              FL_z[q] = F[2][q] - F[2][q + 4];
+              FU_z[q] = F[2][q] + F[2][q + 4];
+            }
+          } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              FL_xy[q] = FU_xy[q] = pk2(T(0), T(0));
+              FL_z[q] = FU_z[q] = T(0);
+            }
+          }
+          if constexpr (kKeep) {
+            const int pn = rid[((L + 1) % kRing) * NP + face_rec];
+            if (pn != ph && pn >= 0) load_k(coef + (long long)pn * CoefOf<T>::stride + kCoefMode0, kept);
+          }
+          // face of node layer kv: lower-face forces of this voxel + upper-face forces of the one below,
+          // back-transformed to the 4 corners (transposed x and y stages)
+          P2<T> m_xy[4], cor_xy[4];
+          T m_z[4], cor_z[4];
+          if constexpr (kFF) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const float4 a = fup[q * fup_plane];
+              FUp_xy[q] = P2<T>{make_float2(a.x, a.y), make_float2(a.z, a.w)};
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const float4 a = fup[(4 + h) * fup_plane];
+              FUp_z[2 * h] = ff(a.x, a.y);
+              FUp_z[2 * h + 1] = ff(a.z, a.w);
+            }
+          }
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
-            FUp_xy[q] = FU_xy[q];
-            FUp_z[q] = FU_z[q];
+            m_xy[q] = FUp_xy[q] + FL_xy[q];
+            m_z[q] = FUp_z[q] + FL_z[q];
+          }
+          face_bf_t(m_xy, cor_xy);
+          face_bf_t(m_z, cor_z);
+#pragma unroll
+          for (int b = 0; b < 4; ++b) {
+            if constexpr (kPlanes)
+              st_face_ff(Fc, NV, (kv & 1) * 4 * NV + b * NV + vcol, cor_xy[b], cor_z[b]);
+            else
+              st_xyz(fcol + (kv & 1) * fbuf + b * 4 * NV, cor_xy[b], cor_z[b]);
+          }
+          if (NOHALO && own && kv >= kbase && (vi == rx || vj == ry)) {
+            // the tile's last voxel column and row also act on the nodes just beyond the tile: their
+            // corners with a_x = 1 (column) and a_y = 1 (row) go to the edge pass, per node layer
+            Tst* ex = reinterpret_cast<Tst*>(P.z) + 6 * ((long long)tile * P.kc + (kv - kbase)) * (tx + ty);
+            auto put = [&](Tst* d, int b) {
+              d[0] = (Tst)lane0(cor_xy[b]); d[1] = (Tst)lane1(cor_xy[b]); d[2] = (Tst)cor_z[b];
+            };
+            if (vi == rx) {
+              Tst* d = ex + 6 * (vj - 1);
+              put(d, 1);
+              put(d + 3, 3);
+            }
+            if (vj == ry) {
+              Tst* d = ex + 6 * (ty + vi - 1);
+              put(d, 2);
+              put(d + 3, 3);
+            }
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            Vlo_xy[q] = Vup_xy[q];
+            Vlo_z[q] = Vup_z[q];
+          }
+          if constexpr (kFF) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              fup[q * fup_plane] = make_float4(FU_xy[q].hi.x, FU_xy[q].hi.y, FU_xy[q].lo.x, FU_xy[q].lo.y);
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+              fup[(4 + h) * fup_plane] =
+                  make_float4(FU_z[2 * h].hi, FU_z[2 * h].lo, FU_z[2 * h + 1].hi, FU_z[2 * h + 1].lo);
+          } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              FUp_xy[q] = FU_xy[q];
+              FUp_z[q] = FU_z[q];
+            }
           }
         }
-      }
       };
       if constexpr (kFF) {
 #pragma unroll 1
@@ -1391,8 +1392,9 @@ cudaError_t launch_apply(const BatchDev& b, int kind, int post, int gate, cudaSt
           if (e != cudaSuccess || !b.thick) return e;
         }
         // the recomputed-halo form: its halo columns cost the FP32 pipe less than the no-halo
-        // form's edge pass and layout cost it (173 against 223 us per product at 100^3); the
-        // no-halo form pays for native FP64, whose halo columns would occupy the FP64 pipe
+        // form's edge pass and layout cost it (173 against 223 us per product at 100^3, before the node
+        // planes and staggered halves); the no-halo form pays for native FP64, whose halo columns would
+        // occupy the FP64 pipe
         return launch_ff<double, EPI_STORE_DOT, false>(b, ROLE_H, post, gate, s);
       case AK_F64_RESID: return launch_ff<double, EPI_RESIDUAL, true>(b, ROLE_W, post, gate, s);
       case AK_MIX_RESID: return launch_ff<float, EPI_RESIDUAL, true>(b, ROLE_W, post, gate, s);
