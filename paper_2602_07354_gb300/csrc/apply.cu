@@ -464,15 +464,27 @@ __device__ __forceinline__ void ld_face_ff(const float* Fc, int NV, int r, P2<fl
   xy.v = *reinterpret_cast<const float2*>(Fc + 2 * r);
   z = Fc[16 * NV + r];
 }
-__device__ __forceinline__ void st_face_ff(ff* Fc, int NV, int r, const P2<ff>& xy, ff z) {
+__device__ __forceinline__ void st_face_xy(ff* Fc, int r, const P2<ff>& xy) {
   *reinterpret_cast<float4*>(Fc + 2 * r) = make_float4(xy.hi.x, xy.hi.y, xy.lo.x, xy.lo.y);
+}
+__device__ __forceinline__ void st_face_z(ff* Fc, int NV, int r, ff z) {
   *reinterpret_cast<float2*>(Fc + 16 * NV + r) = make_float2(z.hi, z.lo);
 }
-__device__ __forceinline__ void ld_face_ff(const ff* Fc, int NV, int r, P2<ff>& xy, ff& z) {
+__device__ __forceinline__ P2<ff> ld_face_xy(const ff* Fc, int r) {
   const float4 a = *reinterpret_cast<const float4*>(Fc + 2 * r);
+  return {make_float2(a.x, a.y), make_float2(a.z, a.w)};
+}
+__device__ __forceinline__ ff ld_face_z(const ff* Fc, int NV, int r) {
   const float2 b = *reinterpret_cast<const float2*>(Fc + 16 * NV + r);
-  xy = {make_float2(a.x, a.y), make_float2(a.z, a.w)};
-  z = ff(b.x, b.y);
+  return ff(b.x, b.y);
+}
+__device__ __forceinline__ void st_face_ff(ff* Fc, int NV, int r, const P2<ff>& xy, ff z) {
+  st_face_xy(Fc, r, xy);
+  st_face_z(Fc, NV, r, z);
+}
+__device__ __forceinline__ void ld_face_ff(const ff* Fc, int NV, int r, P2<ff>& xy, ff& z) {
+  xy = ld_face_xy(Fc, r);
+  z = ld_face_z(Fc, NV, r);
 }
 // Exact split of a double into its leading float and the float nearest the remainder, as ff(double),
 // but with the leading part rounded in integer arithmetic (the bits below a float's 24 are rounded to
@@ -1109,8 +1121,9 @@ __global__ void __launch_bounds__(MAXT, MINB)
 // The double-float product h -> Ah on tiles of one node layer (small grids, whose tiles are cut that
 // thin to fill the SMs): the two voxel layers that meet at the nodes are computed side by side by the
 // two halves of the block instead of one after the other, as a layer's latency (about 6 us, nearly the
-// same for 6 warps as for 12) sets the time.  Each half leaves its corner forces on the node layer in
-// its own buffer and a node gathers eight records.  20^3 product 18.6 -> 14.5 us.
+// same for 6 warps as for 12) sets the time.  The halves swap face modes (one takes x and y, the other
+// z), so that a column's two voxels are summed in mode space and a node gathers four records as in
+// k_apply: the product is the same bit for bit.  20^3 product 18.6 -> 14.5 us.
 template <bool ONE>
 __global__ void __launch_bounds__(kMaxThreadsF64, 1)
     k_apply_thin(const Prob* __restrict__ probs, const int* __restrict__ item_prob, const long long* __restrict__ counts,
@@ -1151,14 +1164,14 @@ __global__ void __launch_bounds__(kMaxThreadsF64, 1)
       rz[s] = make_float2(pz.hi, pz.lo);
     }
     __syncthreads();
-    if (has_vox) {
-      P2<ff> m_xy[4], cor_xy[4];
-      ff m_z[4], cor_z[4];
+    P2<ff> m_xy[4];
+    ff m_z[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        m_xy[q] = pk2(ff(0), ff(0));
-        m_z[q] = ff(0);
-      }
+    for (int q = 0; q < 4; ++q) {
+      m_xy[q] = pk2(ff(0), ff(0));
+      m_z[q] = ff(0);
+    }
+    if (has_vox) {
       const ff* coef = CoefOf<ff>::table(P) + CoefOf<ff>::base;
       const ff* K = ph >= 0 ? coef + (long long)ph * CoefOf<ff>::stride : nullptr;
       if (K != nullptr && __ldg(reinterpret_cast<const float*>(K + kCoefSolid0)) != 0.f) {
@@ -1181,37 +1194,55 @@ __global__ void __launch_bounds__(kMaxThreadsF64, 1)
           m_z[q] = half ? F[2][q] - F[2][q + 4] : F[2][q] + F[2][q + 4];
         }
       }
-      face_bf_t(m_xy, cor_xy);
-      face_bf_t(m_z, cor_z);
 #pragma unroll
-      for (int b = 0; b < 4; ++b) st_face_ff(Fc, NV, half * 4 * NV + b * NV + col, cor_xy[b], cor_z[b]);
+      for (int q = 0; q < 4; ++q) {  // to the other half: the upper voxel's x and y modes, the lower one's z
+        if (half)
+          st_face_xy(Fc, 4 * NV + q * NV + col, m_xy[q]);
+        else
+          st_face_z(Fc, NV, 4 * NV + q * NV + col, m_z[q]);
+      }
+    }
+    __syncthreads();
+    if (has_vox) {
+      if (!half) {
+        P2<ff> cor[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) m_xy[q] = m_xy[q] + ld_face_xy(Fc, 4 * NV + q * NV + col);
+        face_bf_t(m_xy, cor);
+#pragma unroll
+        for (int b = 0; b < 4; ++b) st_face_xy(Fc, b * NV + col, cor[b]);
+      } else {
+        ff cor[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) m_z[q] = ld_face_z(Fc, NV, 4 * NV + q * NV + col) + m_z[q];
+        face_bf_t(m_z, cor);
+#pragma unroll
+        for (int b = 0; b < 4; ++b) st_face_z(Fc, NV, b * NV + col, cor[b]);
+      }
     }
     __syncthreads();
     DotAcc<ff> dot;
     const int i = i0 + vi - 1, j = j0 + vj - 1;
-    if (!half && has_vox && vi >= 1 && vj >= 1 && i < nx && j < ny) {
-      P2<ff> oxy = pk2(ff(0), ff(0));
-      ff oz = ff(0);
-#pragma unroll
-      for (int b = 3; b >= 0; --b)
-#pragma unroll
-        for (int l = 0; l < 2; ++l) {
-          P2<ff> xy;
-          ff z;
-          ld_face_ff(Fc, NV, col + l * 4 * NV + b * NV - (b & 1) - NXv * (b >> 1), xy, z);
-          oxy = oxy + xy;
-          oz = oz + z;
-        }
+    if (has_vox && vi >= 1 && vj >= 1 && i < nx && j < ny) {
+      const long long n = k0 * plane + (long long)j * nx + i;
       P2<ff> hxy;
       ff hz;
       ld_node_ff(rxy + NP + rec, rz + NP + rec, hxy, hz);
-      const long long n = k0 * plane + (long long)j * nx + i;
-      const ff out[3] = {lane0(oxy), lane1(oxy), oz};
+      if (!half) {
+        P2<ff> out = pk2(ff(0), ff(0));
 #pragma unroll
-      for (int c = 0; c < 3; ++c) y[c * N + n] = (double)out[c];
-      dot.add(lane0(hxy), out[0]);
-      dot.add(lane1(hxy), out[1]);
-      dot.add(hz, out[2]);
+        for (int b = 3; b >= 0; --b) out = out + ld_face_xy(Fc, col + b * NV - (b & 1) - NXv * (b >> 1));
+        y[n] = (double)lane0(out);
+        y[N + n] = (double)lane1(out);
+        dot.add(lane0(hxy), lane0(out));
+        dot.add(lane1(hxy), lane1(out));
+      } else {
+        ff out = ff(0);
+#pragma unroll
+        for (int b = 3; b >= 0; --b) out = out + ld_face_z(Fc, NV, col + b * NV - (b & 1) - NXv * (b >> 1));
+        y[2 * N + n] = (double)out;
+        dot.add(hz, out);
+      }
     }
     const double b0 = block_total(dot, red);
     if (t == 0) {

@@ -42,6 +42,21 @@ def test_thin_tiles_match_the_oracle(oracle, tx, ty):
     assert np.linalg.norm(w.cpu().numpy() - ref["w"]) <= 1e-7 * np.linalg.norm(ref["w"])
 
 
+def test_thin_tiles_give_the_bits_of_thick_ones():
+    # the same sums in the same order: a column's two voxels in mode space, then four corners a node
+    dims = (12, 14, 9)
+    sm = torch.cuda.get_device_properties(0).multi_processor_count
+    ms = synth.random_problem(dims, 5, np.random.default_rng(21), pore_prob=0.15)
+    u = torch.from_numpy(np.random.default_rng(22).normal(size=3 * ms.N)).cuda()
+    out = []
+    for tile in ("6 7 1", "12 14 3", "12 14 1", "5 3 1"):
+        B.elas_tuning_import(f"{dims[0]} {dims[1]} {dims[2]} 8 {sm} {tile}\n")
+        y = torch.empty_like(u)
+        B.elas_apply(B.create_from_micro(ms), u, y)
+        out.append(y)
+    assert all(torch.equal(y, out[1]) for y in out)
+
+
 def test_thin_and_thick_problems_in_one_batch():
     rng = np.random.default_rng(8)
     micros = [synth.random_problem(d, 3, rng, pore_prob=0.1) for d in [(18, 17, 19), (40, 41, 42), (20, 20, 20)]]
