@@ -1486,6 +1486,13 @@ Tiling tiling_of(const Geo& g, int tx, int ty, int kc) {
   return t;
 }
 
+// The next chunk height worth a look: a height that leaves the number of chunks as it is only marches
+// further (both searches of a 100^3 grid: 368 us with every height tried, 129 us).
+static int next_chunk(int nz, int kc) {
+  const int tiles = (nz - 1) / kc + 1;
+  return tiles > 1 ? (nz - 1) / (tiles - 1) + 1 : nz + 1;
+}
+
 // FP32 product: two blocks of up to 256 columns share an SM.  Microseconds of a launch, from the
 // product's times at 48^3 ... 300^3: a pair of tiles takes 1.42 us per voxel layer at 8 warps each,
 // 1.38 at 7 (latency, not work, sets it) and 3.0 us to fill and drain, a tile alone on its SM 0.96 and
@@ -1503,7 +1510,8 @@ static Tiling make_tiling32(const Geo& g, int sm_count, int tx_hint, int ty_hint
       const double narrow = 1.0 + 0.0022 * std::max(0, 15 - tx) * std::max(0, 15 - tx);  // short rows
       const double warps = (double)((nv + 31) / 32);
       const double pair = narrow * (1.10 + 0.04 * warps), alone = narrow * (0.80 + 0.02 * warps);
-      for (int kc = (kc_hint ? kc_hint : 1); kc <= (kc_hint ? kc_hint : std::min(64, g.nz)); ++kc) {
+      for (int kc = (kc_hint ? kc_hint : 1); kc <= (kc_hint ? kc_hint : std::min(64, g.nz));
+           kc = kc_hint ? kc + 1 : next_chunk(g.nz, kc)) {
         const Tiling t = tiling_of(g, tx, ty, kc);
         if (t.n_tiles > (1LL << 30)) continue;
         const long long m = (t.n_tiles + sm_count - 1) / sm_count;  // tiles of the busiest SM
@@ -1543,7 +1551,8 @@ Tiling make_tiling(const Geo& g, int elem_bytes, int sm_count, int tx_hint, int 
       if (smem > kApplySmemMax) continue;
       const int R = apply_resident_blocks(elem_bytes, threads, smem);
       const int tiles_x = (g.nx + tx - 1) / tx, tiles_y = (g.ny + ty - 1) / ty;
-      for (int kc = (kc_hint ? kc_hint : 1); kc <= (kc_hint ? kc_hint : std::min(64, g.nz)); ++kc) {
+      for (int kc = (kc_hint ? kc_hint : 1); kc <= (kc_hint ? kc_hint : std::min(64, g.nz));
+           kc = kc_hint ? kc + 1 : next_chunk(g.nz, kc)) {
         const int tiles_z = (g.nz + kc - 1) / kc;
         const long long n_tiles = (long long)tiles_x * tiles_y * tiles_z;
         const long long slots = (long long)sm_count * R;
