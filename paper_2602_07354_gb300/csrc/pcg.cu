@@ -102,6 +102,7 @@ __global__ void k_state_init(const Prob* __restrict__ probs, const SolveSetup* _
   st->last_repl_iter = 0;
   st->done = 0;
   st->needs_init = 1;
+  st->finalized = 0;  // a server slot keeps its state: the request before this one has been finalised
   st->w_applied = 1;
   st->status = ST_RUNNING;
   st->gg = st->gg0 = st->gg_last = st->hAh = st->hAh_first = st->lambda = st->gamma = 0.0;
