@@ -282,7 +282,10 @@ __global__ void __launch_bounds__(kGenThreads)
         __syncthreads();
       }
     }
-    const float reach = ub + 1e-4f * (ub + h2);
+    // the largest lower bound that a seed of these weights may have and still win a voxel.  A lower bound
+    // is off by 2^-21 (D^2 + 3 h^2 w) at most: the rounding of an offset is 2^-23 (a + h) and enters 2 a w
+    // times (without w in it, a seed of weight 1e8 just outside a tile lost voxels that were its own)
+    auto reach = [&](const float2& w) { return ub + 1e-4f * (ub + h2 * fmaxf(w.x, w.y)); };
     const int raw = s_raw;
     auto wraps = [&](float ox, float oy, float oz) {
       return fabsf(ox) + h[0] > 0.499f * Lf[0] || fabsf(oy) + h[1] > 0.499f * Lf[1] || fabsf(oz) + h[2] > 0.499f * Lf[2];
@@ -309,7 +312,7 @@ __global__ void __launch_bounds__(kGenThreads)
           w[q] = WEIGHTED ? candw[at] : make_float2(1.f, 1.f);
           const float a = fmaxf(0.f, fabsf(v[q].x) - h[0]), b = fmaxf(0.f, fabsf(v[q].y) - h[1]);
           const float e = fmaxf(0.f, fabsf(v[q].z) - h[2]);
-          in[q] = (a * a + b * b) * w[q].x + e * e * w[q].y <= reach;
+          in[q] = (a * a + b * b) * w[q].x + e * e * w[q].y <= reach(w[q]);
         }
       }
       __syncthreads();
@@ -322,7 +325,7 @@ __global__ void __launch_bounds__(kGenThreads)
         float o[3], dlo, dhi;
         float2 w;
         bounds(t, o, w, dlo, dhi);
-        if (dlo <= reach) keep(make_float4(o[0], o[1], o[2], __int_as_float(t)), w);
+        if (dlo <= reach(w)) keep(make_float4(o[0], o[1], o[2], __int_as_float(t)), w);
       });
     }
     __syncthreads();
