@@ -408,8 +408,8 @@ __global__ void __launch_bounds__(kGenThreads)
 // first.  With |R_ij| <= 1 (to rounding), semi-axes within a factor 20 of each other and
 // amax >= 1/2, a difference is at most amax + 3 long inside the box, so u = R^T d / a is off by less
 // than 1e-4 and the sum by less than 4e-4 of max(1, sum): only voxels within 1e-3 of the surface
-// evaluate the FP64 sum.  A component near half the cell, where the minimum image may go either
-// way, is longer than amax, so its sum is in that band or above it for both images.
+// evaluate the FP64 sum, and voxels with a component within 1e-6 of half the cell, where rounding may pick
+// the other minimum image (a frame that is not a rotation may have either image inside).
 // Bound: FP64 arithmetic before (183 pores of r <= 6: 71 us with R / a still divided in FP64 by every
 // thread); 12.7 us now, issue-bound.
 __global__ void k_stamp(int nx, int ny, int nz, const double* __restrict__ pores, int32_t* __restrict__ phase) {
@@ -446,6 +446,7 @@ __global__ void k_stamp(int nx, int ny, int nz, const double* __restrict__ pores
     const int at[3] = {(int)(t % cnt[0]), (int)((t / cnt[0]) % cnt[1]), (int)(t / ((unsigned)cnt[0] * cnt[1]))};
     int idx[3];
     float f[3];
+    bool half = false;  // half a cell away but for rounding (1.5e-7 of the cell)
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       const int a = lo[d] + at[d];  // -n < a < 2 n
@@ -453,6 +454,7 @@ __global__ void k_stamp(int nx, int ny, int nz, const double* __restrict__ pores
       f[d] = first[d] + (float)at[d];
       const float Lf = (float)n[d];
       f[d] -= f[d] > 0.5f * Lf ? Lf : (f[d] < -0.5f * Lf ? -Lf : 0.f);
+      half = half || fabsf(fabsf(f[d]) - 0.5f * Lf) <= 1e-6f * Lf;
     }
     float sf = 0.f;
 #pragma unroll
@@ -461,7 +463,7 @@ __global__ void k_stamp(int nx, int ny, int nz, const double* __restrict__ pores
       sf = fmaf(u, u, sf);
     }
     bool inside = sf < 1.f;
-    if (!screen || !(fabsf(sf - 1.f) > 1e-3f * fmaxf(1.f, sf))) {
+    if (!screen || half || !(fabsf(sf - 1.f) > 1e-3f * fmaxf(1.f, sf))) {
       double dd[3], s = 0.0;
 #pragma unroll
       for (int d = 0; d < 3; ++d) dd[d] = min_image(idx[d] + 0.5 - P[d], (double)n[d]);
