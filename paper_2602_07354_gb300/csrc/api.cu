@@ -816,9 +816,10 @@ int elas_tuning_import(const char* text) {
     }
     const Geo geo{v[0], v[1], v[2], (long long)v[0] * v[1] * v[2]};
     Tiling t = make_tiling(geo, v[3], v[4], v[5], v[6], v[7]);
-    if (v[3] == 4 && t.n_tiles <= 0 && (v[5] + 1LL) * (v[6] + 1LL) <= kMaxColumnsF32)
+    const long long columns = (v[5] + 1LL) * (v[6] + 1LL);
+    if (v[3] == 4 && columns > kMaxThreadsF32 && columns <= kMaxColumnsF32)
       t = tiling_of(geo, v[5], v[6], v[7]);  // from a build with wider FP32 blocks: kept, not used
-    if (t.n_tiles <= 0 || t.tx != v[5] || t.ty != v[6] || t.kc != v[7]) {
+    if (t.n_tiles <= 0 || t.n_tiles > (1LL << 30) || t.tx != v[5] || t.ty != v[6] || t.kc != v[7]) {
       char m[96];
       std::snprintf(m, sizeof m, "elas_tuning_import: line %d is not a valid tiling for its grid", line_no);
       return fail(nullptr, ELAS_ERR_INVALID_ARG, m);
