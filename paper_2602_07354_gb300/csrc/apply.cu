@@ -1486,13 +1486,6 @@ Tiling tiling_of(const Geo& g, int tx, int ty, int kc) {
   return t;
 }
 
-// The next chunk height worth a look: a height that leaves the number of chunks as it is only marches
-// further (both searches of a 100^3 grid: 368 us with every height tried, 129 us).
-static int next_chunk(int nz, int kc) {
-  const int tiles = (nz - 1) / kc + 1;
-  return tiles > 1 ? (nz - 1) / (tiles - 1) + 1 : nz + 1;
-}
-
 // FP32 product: two blocks of up to 256 columns share an SM.  Microseconds of a launch, from the
 // product's times at 48^3 ... 300^3: a pair of tiles takes 1.42 us per voxel layer at 8 warps each,
 // 1.38 at 7 (latency, not work, sets it) and 3.0 us to fill and drain, a tile alone on its SM 0.96 and

@@ -8,6 +8,7 @@ namespace elas {
 struct ColumnTile {
   int tx = 0, ty = 0, zc = 0;  // columns of a tile, layers of an item
   int items = 0;               // one block per item
+  int threads = 0;             // of a block, where the kernel has a choice
 };
 
 // Tile of at most `threads` columns with the fewest idle threads over the grid (an idle lane costs
@@ -33,7 +34,7 @@ inline ColumnTile column_tile(const Geo& g, int threads, int hx, int hy, double 
   }
   const long long tiles = (long long)((g.nx - 1) / best.tx + 1) * ((g.ny - 1) / best.ty + 1);
   double c0 = 1e300;
-  for (int zc = 1; zc <= g.nz && (zc <= 256 || best.zc == 0); ++zc) {
+  for (int zc = 1; zc <= g.nz && (zc <= 256 || best.zc == 0); zc = next_chunk(g.nz, zc)) {
     const long long items = tiles * ((g.nz - 1) / zc + 1);
     if (items > (1 << 30) || (max_items && items > max_items && zc < g.nz)) continue;
     const double c = (double)((items + sm_count - 1) / sm_count) * (zc + extra);

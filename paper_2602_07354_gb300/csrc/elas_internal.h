@@ -415,6 +415,12 @@ size_t apply_smem_bytes_ff(int tx, int ty);
 __host__ __device__ constexpr bool thin_tiling(int tx, int ty, int kc) {
   return kc == 1 && (tx + 1) * (ty + 1) <= kMaxThreadsF64 / 2;
 }
+// The next chunk height worth a look: a height that leaves the number of chunks as it is only marches
+// further (both operator searches of a 100^3 grid: 368 us with every height tried, 129 us).
+inline int next_chunk(int nz, int kc) {
+  const int tiles = (nz - 1) / kc + 1;
+  return tiles > 1 ? (nz - 1) / (tiles - 1) + 1 : nz + 1;
+}
 constexpr int kBlocksF32 = 2;  // resident blocks per SM of the FP32 product
 Tiling tiling_of(const Geo& g, int tx, int ty, int kc);
 Tiling make_tiling(const Geo& g, int elem_bytes, int sm_count, int tx_hint = 0, int ty_hint = 0, int kc_hint = 0);

@@ -42,10 +42,13 @@ __device__ __forceinline__ int wrapn(int i, int n) {
 // (9.6 a voxel with the tile's halo, instead of 27), the weight sum is the constant full sum unless
 // the window holds a pore, and the division by that constant is a multiplication by its correctly
 // rounded reciprocal and one residual correction (Markstein 1990: correctly rounded).  200^3, s = 0.4:
-// 2.05 -> 0.84 ms,
-// FP64 pipe 82% busy.  For R >= 2 the classes outgrow shared memory: one product per tap and |dz|.
-template <int R>
-__global__ void __launch_bounds__(kHotThreads, R == 1 ? 2 : 1)
+// 2.05 -> 0.84 ms, FP64 pipe 82% busy.
+// For R >= 2 the classes outgrow shared memory: one product per tap and |dz|, shared by the outputs on
+// either side.  The planes beside an item reach only some of its outputs; computing all of them made
+// items of few layers (small grids) up to six times slower than a plain loop (the call on 24^3, s = 1.9:
+// 281 us with the loop, 1,660, 201 now; 48^3, s = 0.8: 176, 250, 151; 140^3, s = 0.8: 3.12 ms, 2.26, 2.19).
+template <int R, int NT>
+__global__ void __launch_bounds__(NT, (R == 1 ? 2 : 1) * kHotThreads / NT)
     k_smooth(int nx, int ny, int nz, int tx, int ty, int zc, const int32_t* __restrict__ phase,
              const double* __restrict__ vm, const __grid_constant__ Weights W, double* __restrict__ smooth) {
   constexpr int D = 2 * R + 1, C = R + 1, NQ = R == 1 ? 8 : 1;
@@ -64,7 +67,7 @@ __global__ void __launch_bounds__(kHotThreads, R == 1 ? 2 : 1)
     int off[kPos];
 #pragma unroll
     for (int q = 0; q < kPos; ++q) {
-      const int s = t + q * kHotThreads;
+      const int s = t + q * NT;
       off[q] = s < np ? wrapn(j0 - R + s / wx, ny) * nx + wrapn(i0 - R + s % wx, nx) : -1;
     }
     double pv[kPos];
@@ -95,7 +98,7 @@ __global__ void __launch_bounds__(kHotThreads, R == 1 ? 2 : 1)
 #pragma unroll
       for (int q = 0; q < kPos; ++q)
         if (off[q] >= 0) {
-          const int s = t + q * kHotThreads;
+          const int s = t + q * NT;
           const bool solid = pp[q] >= 0;
           so[s] = solid;
           if constexpr (R == 1) {
@@ -138,20 +141,28 @@ __global__ void __launch_bounds__(kHotThreads, R == 1 ? 2 : 1)
           }
           all = m == 0x1ff;
         } else {
+          // outputs p + cz and p - cz, as far as the item owns them (one cz after the other: an output meets
+          // the plane's taps in one of the loops, in the order dy, dx)
+#pragma unroll
+          for (int cz = 0; cz <= R; ++cz) {
+            const bool up = p + cz >= z0 && p + cz < z1, down = cz && p - cz >= z0 && p - cz < z1;
+            if (!up && !down) continue;
+            double a = acc[R - cz], b = acc[R + cz];
+#pragma unroll
+            for (int dy = 0; dy < D; ++dy)
+#pragma unroll
+              for (int dx = 0; dx < D; ++dx) {
+                const int cy = dy < R ? R - dy : dy - R, cx = dx < R ? R - dx : dx - R;
+                const double q = __dmul_rn(W.w[(cz * C + cy) * C + cx], v[(j + dy) * wx + i + dx]);
+                if (up) a = __dadd_rn(a, q);
+                if (down) b = __dadd_rn(b, q);
+              }
+            acc[R - cz] = a;
+            if (cz) acc[R + cz] = b;
+          }
           for (int dy = 0; dy < D; ++dy)
 #pragma unroll
-            for (int dx = 0; dx < D; ++dx) {
-              const int s = (j + dy) * wx + i + dx;
-              const int cy = dy < R ? R - dy : dy - R, cx = dx < R ? R - dx : dx - R;
-              const double x = v[s];
-              all = all && so[s];
-#pragma unroll
-              for (int cz = 0; cz <= R; ++cz) {
-                const double q = __dmul_rn(W.w[(cz * C + cy) * C + cx], x);
-                acc[R - cz] = __dadd_rn(acc[R - cz], q);
-                if (cz) acc[R + cz] = __dadd_rn(acc[R + cz], q);
-              }
-            }
+            for (int dx = 0; dx < D; ++dx) all = all && so[(j + dy) * wx + i + dx];
         }
 #pragma unroll
         for (int d = 0; d < D - 1; ++d) {
@@ -332,17 +343,57 @@ __global__ void __launch_bounds__(kHotThreads)
   }
 }
 
+// Block size, tile and layers of the smoothing: the busiest SM's FP64 operations (an output layer's, a
+// staged position's and, for R >= 2, those that an item's ends add), with a plane's barrier and load
+// counted as 3,300 (2,000 clocks).  Fewer threads than `few` on an SM wait for their own sums instead of
+// for the pipe.
+template <int R>
+ColumnTile smooth_tile(const Geo& g, int sm_count) {
+  constexpr int D = 2 * R + 1;
+  constexpr double layer = R == 1 ? 30 : D * D * (3 * R + 2), pos = R == 1 ? 8 : 0, ends = R == 1 ? 0 : D * D * R;
+  ColumnTile best{};
+  double cost0 = 1e300;
+  for (int threads = kHotThreads; threads >= 128; threads /= 2) {
+    ColumnTile h = column_tile(g, threads, 2 * R, 2 * R, 1.0, sm_count, R == 1 ? std::min(704, 3 * threads) : 3 * threads);
+    const int tiles = h.items / ((g.nz - 1) / h.zc + 1), last = h.zc;
+    for (int zc = R == 1 ? last : 1; zc <= last; zc = next_chunk(g.nz, zc)) {
+      const long long items = (long long)tiles * ((g.nz - 1) / zc + 1), m = (items + sm_count - 1) / sm_count;
+      if (items > (1 << 30)) continue;
+      const double few = R == 1 ? 0 : 224;
+      const double cost = std::max((double)m * threads, few) * (layer * zc + ends) +
+                          m * (zc + 2 * R) * (pos * (h.tx + 2 * R) * (h.ty + 2 * R) + 3300.0);
+      if (cost < cost0) {
+        cost0 = cost;
+        best = h;
+        best.threads = threads;
+        best.zc = zc;
+        best.items = (int)items;
+      }
+    }
+    // R = 1 from 64^3 on: smaller blocks give nothing and looking at them 3 us of a call of 94
+    if (R == 1 && last >= 4) break;
+  }
+  return best;
+}
+
+template <int R, int NT>
+cudaError_t launch_smooth_t(const Geo& g, const ColumnTile& h, const int32_t* phase, const double* vm, const Weights& W,
+                            double* smooth, cudaStream_t s) {
+  constexpr int NQ = R == 1 ? 8 : 1, most = 2 * (R == 1 ? std::min(704, 3 * NT) : 3 * NT) * (8 * NQ + 1);
+  const size_t smem = (size_t)(h.tx + 2 * R) * (h.ty + 2 * R) * 2 * (NQ * sizeof(double) + 1);
+  cudaError_t e = cudaFuncSetAttribute(k_smooth<R, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (e != cudaSuccess) return e;
+  k_smooth<R, NT><<<h.items, NT, smem, s>>>(g.nx, g.ny, g.nz, h.tx, h.ty, h.zc, phase, vm, W, smooth);
+  return cudaGetLastError();
+}
+
 template <int R>
 cudaError_t launch_smooth(const Geo& g, const int32_t* phase, const double* vm, const Weights& W, double* smooth,
                           int sm_count, cudaStream_t s) {
-  constexpr int NQ = R == 1 ? 8 : 1;
-  const ColumnTile h = column_tile(g, kHotThreads, 2 * R, 2 * R, R, sm_count, R == 1 ? 704 : 3 * kHotThreads);
-  const size_t smem = (size_t)(h.tx + 2 * R) * (h.ty + 2 * R) * 2 * (NQ * sizeof(double) + 1);
-  constexpr int most = R == 1 ? 2 * 704 * (8 * NQ + 1) : 2 * 3 * kHotThreads * (8 * NQ + 1);
-  cudaError_t e = cudaFuncSetAttribute(k_smooth<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-  if (e != cudaSuccess) return e;
-  k_smooth<R><<<h.items, kHotThreads, smem, s>>>(g.nx, g.ny, g.nz, h.tx, h.ty, h.zc, phase, vm, W, smooth);
-  return cudaGetLastError();
+  const ColumnTile h = smooth_tile<R>(g, sm_count);
+  return h.threads == 128   ? launch_smooth_t<R, 128>(g, h, phase, vm, W, smooth, s)
+         : h.threads == 256 ? launch_smooth_t<R, 256>(g, h, phase, vm, W, smooth, s)
+                            : launch_smooth_t<R, kHotThreads>(g, h, phase, vm, W, smooth, s);
 }
 
 }  // namespace
