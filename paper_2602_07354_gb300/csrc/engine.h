@@ -31,13 +31,15 @@ struct Engine {
   int cap_probs = 0;                  // capacity of the tables (problems)
   long long cap_apply = 0, cap_vec = 0;
   BatchDev bd{};
-  cudaGraphExec_t exec = nullptr;
+  cudaGraphExec_t exec[3] = {};       // the recorded batch by the FP64 product's forms (form_of)
   int exec_k = 0;
   size_t fixed_smem32 = 0, fixed_smem64 = 0, fixed_smemff = 0;  // non-zero: fixed launch shape (server)
 };
 
 // Record (or reuse) the CUDA graph of K PCG iterations over the engine's problems.
 int record_batch(Engine& e, int K, std::string* err);
+// Launch the recorded batch on the owner's stream.
+cudaError_t launch_batch(Engine& e);
 
 // Bytes of device tables for an engine with these capacities (carved from the owner's workspace).
 size_t engine_table_bytes(int cap_probs, long long cap_apply, long long cap_vec);

@@ -406,7 +406,7 @@ int elas_server_step(elas_server* s, int* n_active_out, int* n_queued, int* n_fi
   if (n_active(s) > 0) {
     int rc = record_batch(s->eng, s->K, &m);
     if (rc != ELAS_OK) return sfail(s, rc, "server: " + m);
-    cudaError_t e = cudaGraphLaunch(s->eng.exec, st);
+    cudaError_t e = launch_batch(s->eng);
     // 3. final FP64 w and true residual of the requests that stopped
     if (e == cudaSuccess) e = launch_w_finish(s->eng.bd, mixed, GATE_FINALIZE, st);
     if (e == cudaSuccess) e = launch_apply(s->eng.bd, AK_F64_NORM, POST_TRUE_NORM, GATE_FINALIZE, st);
