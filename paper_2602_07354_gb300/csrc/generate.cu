@@ -111,7 +111,7 @@ __device__ __forceinline__ void consider(double D2, int l, double& best, int& ar
 // The grain of one voxel by FP64 distances alone: the 5 x 5 x 5 cells around its own, and every seed
 // when those cannot be shown to hold the nearest one (seeds outside that block lie at least the
 // distance from the voxel to the block's faces away).  Tiles whose candidates do not fit the block's
-// list and weights outside the FP32 range take it.
+// list and grids outside the FP32 screen's range (k_assign_exact) take it.
 template <bool WEIGHTED>
 __device__ int nearest_exact(const double (&x)[3], const double* __restrict__ seeds, const double* __restrict__ semi,
                              int n, const int* __restrict__ start, const int* __restrict__ items, const GenGrid& G,
@@ -152,6 +152,20 @@ __device__ int nearest_exact(const double (&x)[3], const double* __restrict__ se
   return arg;
 }
 
+// Every voxel by FP64 distances, one a thread (by tiles of k_assign, two a thread one after the other, 55
+// seeds on 48^3 took 704 us, this form 545).
+template <bool WEIGHTED>
+__global__ void k_assign_exact(int nx, int ny, int nz, const double* __restrict__ seeds, const double* __restrict__ semi,
+                               int n, const int* __restrict__ start, const int* __restrict__ items, GenGrid G,
+                               int32_t* __restrict__ phase) {
+  const long long N = (long long)nx * ny * nz;
+  const double L[3] = {(double)nx, (double)ny, (double)nz};
+  for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < N; v += (long long)gridDim.x * blockDim.x) {
+    const double x[3] = {(int)(v % nx) + 0.5, (int)((v / nx) % ny) + 0.5, (int)(v / ((long long)nx * ny)) + 0.5};
+    phase[v] = nearest_exact<WEIGHTED>(x, seeds, semi, n, start, items, G, L);
+  }
+}
+
 // One tile of 8 x 8 x 8 voxels per block and turn, two voxels (z and z + 4) per thread.
 //
 // FP32 error.  A seed comes as a float pair hi + lo; its minimum-image offset from the tile's centre
@@ -170,7 +184,7 @@ template <bool WEIGHTED>
 __global__ void __launch_bounds__(kGenThreads)
     k_assign(int nx, int ny, int nz, const double* __restrict__ seeds, const double* __restrict__ semi,
              const float4* __restrict__ fast, int n, const int* __restrict__ start, const int* __restrict__ items,
-             GenGrid G, bool screen, int32_t* __restrict__ phase) {
+             GenGrid G, int32_t* __restrict__ phase) {
   __shared__ float4 cand[kTileCap];                // offset from the tile's centre, seed position
   __shared__ float2 candw[WEIGHTED ? kTileCap : 1];  // transverse and longitudinal weights
   __shared__ int s_raw, s_cnt, s_ub, s_wmax, s_wrap, s_lo[3], s_n[3];
@@ -253,34 +267,32 @@ __global__ void __launch_bounds__(kGenThreads)
         }
       }
     };
-    float ub = INFINITY;
-    if (screen) {
-      // the smallest upper bound over the tile; the candidates wait in the list as they come
-      for (int pass = 0; pass < 2; ++pass) {
-        float mine = INFINITY;
-        each_seed([&](int t) {
-          float o[3], dlo, dhi;
-          float2 w;
-          bounds(t, o, w, dlo, dhi);
-          mine = fminf(mine, dhi);
-          const int at = atomicAdd(&s_raw, 1);
-          if (at < kTileCap) {
-            cand[at] = make_float4(o[0], o[1], o[2], __int_as_float(t));
-            if (WEIGHTED) candw[at] = w;
-          }
-        });
+    float ub;
+    // the smallest upper bound over the tile; the candidates wait in the list as they come
+    for (int pass = 0; pass < 2; ++pass) {
+      float mine = INFINITY;
+      each_seed([&](int t) {
+        float o[3], dlo, dhi;
+        float2 w;
+        bounds(t, o, w, dlo, dhi);
+        mine = fminf(mine, dhi);
+        const int at = atomicAdd(&s_raw, 1);
+        if (at < kTileCap) {
+          cand[at] = make_float4(o[0], o[1], o[2], __int_as_float(t));
+          if (WEIGHTED) candw[at] = w;
+        }
+      });
 #pragma unroll
-        for (int s = 16; s > 0; s >>= 1) mine = fminf(mine, __shfl_xor_sync(0xffffffffu, mine, s));
-        if ((tid & 31) == 0) atomicMin(&s_ub, __float_as_int(mine));  // non-negative floats order as ints
-        __syncthreads();
-        ub = __int_as_float(s_ub);
-        // a seed outside the collected cells is at least the margin away, at weight >= 1
-        if (pass == 1 || ub < 0.999f * margin * margin) break;
-        all = true;
-        __syncthreads();
-        if (tid == 0) s_raw = 0;
-        __syncthreads();
-      }
+      for (int s = 16; s > 0; s >>= 1) mine = fminf(mine, __shfl_xor_sync(0xffffffffu, mine, s));
+      if ((tid & 31) == 0) atomicMin(&s_ub, __float_as_int(mine));  // non-negative floats order as ints
+      __syncthreads();
+      ub = __int_as_float(s_ub);
+      // a seed outside the collected cells is at least the margin away, at weight >= 1
+      if (pass == 1 || ub < 0.999f * margin * margin) break;
+      all = true;
+      __syncthreads();
+      if (tid == 0) s_raw = 0;
+      __syncthreads();
     }
     // the largest lower bound that a seed of these weights may have and still win a voxel.  A lower bound
     // is off by 2^-21 (D^2 + 3 h^2 w) at most: the rounding of an offset is 2^-23 (a + h) and enters 2 a w
@@ -299,7 +311,7 @@ __global__ void __launch_bounds__(kGenThreads)
       if (wraps(v.x, v.y, v.z)) s_wrap = 1;
       if (WEIGHTED) atomicMax(&s_wmax, __float_as_int(fmaxf(w.x, w.y)));
     };
-    if (screen && raw <= kTileCap) {  // compact the list in place
+    if (raw <= kTileCap) {  // compact the list in place
       float4 v[4];
       float2 w[4];
       bool in[4];
@@ -319,7 +331,7 @@ __global__ void __launch_bounds__(kGenThreads)
 #pragma unroll
       for (int q = 0; q < 4; ++q)
         if (in[q]) keep(v[q], w[q]);
-    } else if (screen) {  // more candidates than the list holds: collect again, pruned
+    } else {  // more candidates than the list holds: collect again, pruned
       __syncthreads();
       each_seed([&](int t) {
         float o[3], dlo, dhi;
@@ -332,7 +344,7 @@ __global__ void __launch_bounds__(kGenThreads)
     const int m = s_cnt;
     const int vi = org[0] + i, vj = org[1] + j;
     const bool in_xy = vi < nx && vj < ny;
-    if (screen && m <= kTileCap) {
+    if (m <= kTileCap) {
       const float rx = (float)i - h[0], ry = (float)j - h[1], rz[2] = {(float)k - h[2], (float)(k + 4) - h[2]};
       const bool wrap = s_wrap != 0;
       float m1[2] = {INFINITY, INFINITY}, m2[2] = {INFINITY, INFINITY};
@@ -592,14 +604,22 @@ int elas_assign_grains(int nx, int ny, int nz, const double* seeds, const double
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(base + Ly.items, items.data(), sizeof(int) * items.size(), cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return gen_fail(ELAS_ERR_CUDA, std::string("elas_assign_grains: ") + cudaGetErrorString(e));
-  const long long tiles = (long long)((nx - 1) / kTile + 1) * ((ny - 1) / kTile + 1) * ((nz - 1) / kTile + 1);
   const int sms = std::max(sm_count(), 1);
-  const long long blocks = std::min<long long>(tiles, (long long)sms * 32);
-  auto kern = semi_axes ? k_assign<true> : k_assign<false>;
-  kern<<<(int)blocks, kGenThreads, 0, s>>>(nx, ny, nz, (const double*)(base + Ly.seeds),
-                                           semi_axes ? (const double*)(base + Ly.semi) : nullptr,
-                                           (const float4*)(base + Ly.fast), n_grains, (const int*)(base + Ly.start),
-                                           (const int*)(base + Ly.items), G, screen, phase);
+  const double* d_seeds = (const double*)(base + Ly.seeds);
+  const double* d_semi = semi_axes ? (const double*)(base + Ly.semi) : nullptr;
+  const int *d_start = (const int*)(base + Ly.start), *d_items = (const int*)(base + Ly.items);
+  if (screen) {
+    const long long tiles = (long long)((nx - 1) / kTile + 1) * ((ny - 1) / kTile + 1) * ((nz - 1) / kTile + 1);
+    const int blocks = (int)std::min<long long>(tiles, (long long)sms * 32);
+    auto kern = semi_axes ? k_assign<true> : k_assign<false>;
+    kern<<<blocks, kGenThreads, 0, s>>>(nx, ny, nz, d_seeds, d_semi, (const float4*)(base + Ly.fast), n_grains, d_start,
+                                        d_items, G, phase);
+  } else {
+    const long long N = (long long)nx * ny * nz;
+    const int blocks = (int)std::min<long long>((N + kGenThreads - 1) / kGenThreads, (long long)sms * 32);
+    auto kern = semi_axes ? k_assign_exact<true> : k_assign_exact<false>;
+    kern<<<blocks, kGenThreads, 0, s>>>(nx, ny, nz, d_seeds, d_semi, n_grains, d_start, d_items, G, phase);
+  }
   e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // the host tables above go out of scope
   if (e != cudaSuccess) return gen_fail(ELAS_ERR_CUDA, std::string("elas_assign_grains: ") + cudaGetErrorString(e));
