@@ -23,11 +23,6 @@ namespace elas {
 
 namespace {
 
-// one warp per block: a grain costs about 100 FP64 operations (trigonometric functions), so the grains
-// of one microstructure (thousands) are spread over all SMs' FP64 pipes (2,048 grains: 8 blocks of 256
-// 10.9 us, 64 of 32: 7.6 us)
-constexpr int kTexThreads = 32;
-
 // lognormal parameters (log-space mean m, spread s) of a variate with mean mu and deviation sd
 void lognormal_params(double mu, double sd, double* m, double* s) {
   const double r = sd / mu;
@@ -131,7 +126,12 @@ __global__ void k_orientations(int n, OrientArgs a, const double* __restrict__ d
   }
 }
 
-int blocks_for(int n) { return std::max(1, std::min((n + kTexThreads - 1) / kTexThreads, 4096)); }
+// One warp per block: a grain costs about 100 FP64 operations (trigonometric functions), so the grains of
+// one microstructure (thousands) are spread over all SMs' FP64 pipes (2,048 grains: 8 blocks of 256
+// 10.9 us, 64 of 32 7.6 us).  More than the 4,096 blocks of a launch take eight warps a block (seeding
+// 2,000,000 grains: one warp 163 us, eight 156; 300,000 orientations: 61.6 and 59.7).
+int threads_for(int n) { return n <= 4096 * 32 ? 32 : 256; }
+int blocks_for(int n) { return std::max(1, std::min((n - 1) / threads_for(n) + 1, 4096)); }
 
 bool finite3(const double* v) { return std::isfinite(v[0]) && std::isfinite(v[1]) && std::isfinite(v[2]); }
 
@@ -173,8 +173,8 @@ int elas_seed_grains(int n_grains, const double* lo, const double* hi, double me
   }
   lognormal_params(mean_d, sd_d, &a.m_d, &a.s_d);
   lognormal_params(mean_alpha, sd_alpha, &a.m_a, &a.s_a);
-  k_seed_grains<<<blocks_for(n_grains), kTexThreads, 0, (cudaStream_t)cuda_stream>>>(n_grains, a, z, u, seeds,
-                                                                                      semi_axes);
+  k_seed_grains<<<blocks_for(n_grains), threads_for(n_grains), 0, (cudaStream_t)cuda_stream>>>(n_grains, a, z, u,
+                                                                                               seeds, semi_axes);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return gen_error(ELAS_ERR_CUDA, std::string("elas_seed_grains: ") + cudaGetErrorString(e));
   return ELAS_OK;
@@ -215,7 +215,7 @@ int elas_orientations(int n_grains, int texture, const double* crystal_axis, con
     }
   }
   if (n_grains == 0) return ELAS_OK;
-  k_orientations<<<blocks_for(n_grains), kTexThreads, 0, (cudaStream_t)cuda_stream>>>(n_grains, a, draws, rho);
+  k_orientations<<<blocks_for(n_grains), threads_for(n_grains), 0, (cudaStream_t)cuda_stream>>>(n_grains, a, draws, rho);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return gen_error(ELAS_ERR_CUDA, std::string("elas_orientations: ") + cudaGetErrorString(e));
   return ELAS_OK;
