@@ -63,21 +63,8 @@ __device__ double total_of(const double* slot, int n, double* red) {
   return block_sum(v, red);
 }
 
-// Ampere-style asynchronous global->shared element copies (cp.async), used to prefetch the
-// periodically wrapped halo of the next node layer while the current one is computed.
-template <typename T>
-__device__ __forceinline__ void cp_async_elem(T* smem, const T* gmem) {
-  const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-  if (sizeof(T) == 8)
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(gmem));
-  else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem));
-}
-__device__ __forceinline__ void cp_async_i32(void* smem, const int32_t* gmem) {
-  const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem));
-}
-// element copy to a shared-memory address (4 or 8 bytes)
+// Asynchronous global->shared element copies (cp.async), used to prefetch the periodically wrapped halo
+// of the node layers ahead while the current one is computed: to a shared-memory address, 4 or 8 bytes.
 template <typename E>
 __device__ __forceinline__ void cp_async_to(unsigned s, const E* gmem) {
   static_assert(sizeof(E) == 4 || sizeof(E) == 8, "4- or 8-byte elements");
@@ -87,7 +74,6 @@ __device__ __forceinline__ void cp_async_to(unsigned s, const E* gmem) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem));
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
-__device__ __forceinline__ void cp_async_wait_1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 // Node-layer ring of the operator: kRing slots, layers staged kAhead = kRing - 1 ahead; a thread
 // waits for a layer's copies kAhead - 2 iterations after issuing them.
 constexpr int kRing = 4, kAhead = kRing - 1;
@@ -300,11 +286,6 @@ __device__ __forceinline__ ff lane1(P2<ff> a) { return ff(a.hi.y, a.lo.y); }
 
 // (x, y, z, 4th) shared-memory records: float [x y z id], double [x y | z id]; the 4th element holds a
 // phase id in the node ring.  Double-float nodes: planes of [x.hi y.hi x.lo y.lo] and [z.hi z.lo].
-__device__ __forceinline__ void ld_xyz(const float* p, P2<float>& xy, float& z) {
-  const float4 v = *reinterpret_cast<const float4*>(p);
-  xy.v = make_float2(v.x, v.y);
-  z = v.z;
-}
 __device__ __forceinline__ void ld_xyz(const double* p, P2<double>& xy, double& z) {
   const double2 a = *reinterpret_cast<const double2*>(p);
   xy = {a.x, a.y};
@@ -322,9 +303,6 @@ __device__ __forceinline__ void ld_node_ff(const float2* pxy, const float* pz, P
 }
 // (never called for native FP64)
 __device__ __forceinline__ void ld_node_ff(const float2*, const float*, P2<double>&, double&) {}
-__device__ __forceinline__ void st_xyz(float* p, P2<float> xy, float z) {
-  *reinterpret_cast<float4*>(p) = make_float4(xy.v.x, xy.v.y, z, 0.f);
-}
 __device__ __forceinline__ void st_xyz(double* p, P2<double> xy, double z) {
   *reinterpret_cast<double2*>(p) = make_double2(xy.x, xy.y);
   p[2] = z;

@@ -45,7 +45,6 @@ cudaError_t launch_batch(Engine& e);
 size_t engine_table_bytes(int cap_probs, long long cap_apply, long long cap_vec);
 
 // Item counts of one grid under its tiling.
-inline long long tiles_of(const Tiling& t) { return t.n_tiles; }
 inline long long chunks_of(long long N, bool mixed) { return (N + vec_chunk(N, mixed) - 1) / vec_chunk(N, mixed); }
 constexpr int kMoreChunks = 2048;  // chunks_of(N) <= N / 2048 + kMoreChunks
 
