@@ -284,8 +284,8 @@ __device__ __forceinline__ double lane1(P2<double> a) { return a.y; }
 __device__ __forceinline__ ff lane0(P2<ff> a) { return ff(a.hi.x, a.lo.x); }
 __device__ __forceinline__ ff lane1(P2<ff> a) { return ff(a.hi.y, a.lo.y); }
 
-// (x, y, z, 4th) shared-memory records: float [x y z id], double [x y | z id]; the 4th element holds a
-// phase id in the node ring.  Double-float nodes: planes of [x.hi y.hi x.lo y.lo] and [z.hi z.lo].
+// Shared-memory records.  Native FP64: [x y | z id], the id being a phase id in the node ring.  FP32 and
+// double-float nodes: planes of [x y] and [z], [x.hi y.hi x.lo y.lo] and [z.hi z.lo], and of ids.
 __device__ __forceinline__ void ld_xyz(const double* p, P2<double>& xy, double& z) {
   const double2 a = *reinterpret_cast<const double2*>(p);
   xy = {a.x, a.y};
@@ -353,9 +353,10 @@ __device__ __forceinline__ void face_forward_ff(const Rxy* pxy, const Rz* pz, in
 
 // Modal element forces F[c][m] (m = 1..7; F[c][0] = 0) from the mode coefficients W[c][m]:
 // seven orthogonal gradient monomials, each a symmetric-stiffness product (see file header).
-// k0 holds the C/16 block (already loaded).  FP64 reads the C/48 block as well; FP32 instead scales
-// the linear-mode coefficients by 1/3 and uses C/16 for them too (C/48 e = C/16 (e/3)), which trades
-// 9 multiplies for 6 vector loads of the coefficient blocks.  The bilinear block is read by all.
+// k0 holds the C/16 block (already loaded).  FP64 reads the C/48 block and the bilinear block as well;
+// FP32 uses C/16 for all: it scales the linear-mode coefficients by 1/3 (C/48 e = C/16 (e/3)) and the
+// trilinear one by 1/9, and forms the bilinear block from C/16 entries: 12 multiplies and 12 additions
+// instead of 8 vector loads.
 template <typename T, typename K0>
 __device__ __forceinline__ void modal_forces(T (&W)[3][8], const K0& k0, const T* __restrict__ K,
                                              T (&F)[3][8]) {
@@ -464,10 +465,12 @@ __device__ __forceinline__ void ld_face_ff(const ff* Fc, int NV, int r, P2<ff>& 
   xy = ld_face_xy(Fc, r);
   z = ld_face_z(Fc, NV, r);
 }
-// Exact split of a double into its leading float and the float nearest the remainder, as ff(double),
-// but with the leading part rounded in integer arithmetic (the bits below a float's 24 are rounded to
-// nearest and cleared): 3 instead of 4 operations on the FP64 pipe, which all warps' splits share
-// (100^3 product 140 -> 137 us).  Leading parts beyond the float range become infinite, as there.
+// Split of a double into its leading float and the float nearest the remainder, as ff(double), but with
+// the leading part rounded in integer arithmetic (the bits below a float's 24 are rounded to nearest,
+// halves away from zero, and cleared): 3 instead of 4 operations on the FP64 pipe, which all warps'
+// splits share (100^3 product 140 -> 137 us).  There is no other branch: above the float range the leading
+// part is infinite, and below 2^-126 it is rounded once more, to a subnormal, so that the pair is off by
+// up to 3/4 of a subnormal unit (2^-149; ff(double): 1/2).
 __device__ __forceinline__ ff split_double(double v) {
   const double h = __longlong_as_double((__double_as_longlong(v) + (1LL << 28)) & ~((1LL << 29) - 1));
   return ff(__double2float_rn(h), __double2float_rn(v - h));
@@ -792,7 +795,7 @@ __global__ void __launch_bounds__(MAXT, MINB)
     // that one half's splits, gathers and stores (20 FP64-pipe operations a node) run beside the other's
     // element products on the FP32 pipe.  With all warps in one order they queued for the FP64 pipe
     // right after every barrier (short-scoreboard stalls 0.83 of 5.9 cycles per instruction, 0.21 now):
-    // 100^3 product 160 -> 139 us.  The native FP64 and FP32 forms have no such pair of pipes to overlap.
+    // 100^3 product 150 us in one order, 130 in two.  The native FP64 and FP32 forms have no such pair of pipes to overlap.
     const bool late = t >= (NV + 63) / 64 * 32;
     int chunk_end = min(k0 + kc, k1), part = bx + tiles_x * (by + tiles_y * bz * (kF32 ? P.fmerge : 1));  // (FP32)
     T hown[3] = {T(0), T(0), T(0)};  // the owned node's operand on the previous layer (h.Ah)
@@ -1501,11 +1504,10 @@ static Tiling make_tiling32(const Geo& g, int sm_count, int tx_hint, int ty_hint
 
 Tiling make_tiling(const Geo& g, int elem_bytes, int sm_count, int tx_hint, int ty_hint, int kc_hint) {
   if (elem_bytes == 4) return make_tiling32(g, sm_count, tx_hint, ty_hint, kc_hint);
-  // Model: the SM is throughput-bound, so the time of a launch is the busiest SM's work.  With R
-  // blocks resident per SM (registers ~128/thread, shared memory per block), tiles are handed out
-  // round-robin to sm_count*R blocks; the busiest SM runs ceil(n_tiles/(sm_count*R)) rounds of R
-  // tiles, each (kc + 1) voxel layers of `threads` voxel slots plus a fixed per-layer overhead
-  // (the barrier and the staging).
+  // Model of the FP64 and double-float products: the SM is throughput-bound, so the time of a launch is the
+  // busiest SM's work.  One block of 384 threads is resident per SM (168 registers a thread; R = 1), tiles
+  // are handed out round-robin, and the busiest SM runs ceil(n_tiles / sm_count) rounds, each (kc + 1)
+  // voxel layers of `threads` voxel slots and half a layer to fill and drain.
   Tiling best{};
   double best_cost = 1e300;
   const int tx_lo = tx_hint ? tx_hint : 4, tx_hi = tx_hint ? tx_hint : 40;

@@ -334,6 +334,9 @@ constexpr int kVecThreads = 256;                    // block size of the vector 
 // whose per-item cost a batch of small problems pays in full (mixed items of 256 nodes made a batch
 // of 32^3 and 48^3 cells 10% slower); the smallest FP64 grids are spread over the SMs' FP64 pipes all
 // the same.  At most 4,096 nodes an item, in whole rows of 4.
+// The waves are those of GB300's 152 SMs whatever the device has: chunks are what a problem's sums are
+// made of, so a fixed number keeps results the same on every device, and the workspace's sizing, which
+// knows no device, in step with them.  (A part with fewer SMs gets a short second wave.)
 constexpr long long kVecSms = 152;
 constexpr int vec_chunk(long long N, bool mixed) {
   const long long full = mixed ? 768 : 512;  // (nearly) every thread holds a row

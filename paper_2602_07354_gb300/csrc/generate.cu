@@ -12,8 +12,8 @@
 // (dx*dx + dy*dy) / (rt*rt) + (dz*dz) / (rl*rl), with the periodic minimum-image differences, and
 // ties go to the lowest grain index: every voxel gets exactly the grain of a brute-force scan.
 //
-// Pore overwrite: one block per pore scans the pore's bounding box (periodically wrapped) and
-// writes -1 into every voxel whose centre satisfies (q0/a0)^2 + (q1/a1)^2 + (q2/a2)^2 <= 1 with
+// Pore overwrite: several blocks per pore scan the pore's bounding box (periodically wrapped) and
+// write -1 into every voxel whose centre satisfies (q0/a0)^2 + (q1/a1)^2 + (q2/a2)^2 <= 1 with
 // q = R^T d; the writes are idempotent, so the order of pores and threads does not matter.
 #include <cuda_runtime.h>
 

@@ -46,7 +46,8 @@ __device__ __forceinline__ int wrapn(int i, int n) {
 // For R >= 2 the classes outgrow shared memory: one product per tap and |dz|, shared by the outputs on
 // either side.  The planes beside an item reach only some of its outputs; computing all of them made
 // items of few layers (small grids) up to six times slower than a plain loop (the call on 24^3, s = 1.9:
-// 281 us with the loop, 1,660, 201 now; 48^3, s = 0.8: 176, 250, 151; 140^3, s = 0.8: 3.12 ms, 2.26, 2.19).
+// 281 us with the loop, 1,660, 201 now; 48^3, s = 0.8: 176, 250, 151).  200^3, s = 0.8, 1.2 and 1.9:
+// 8.86, 22.3 and 46.2 ms with the loop, 4.47, 12.6 and 28.5 now.
 template <int R, int NT>
 __global__ void __launch_bounds__(NT, (R == 1 ? 2 : 1) * kHotThreads / NT)
     k_smooth(int nx, int ny, int nz, int tx, int ty, int zc, const int32_t* __restrict__ phase,

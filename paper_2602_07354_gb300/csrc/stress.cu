@@ -60,7 +60,7 @@ struct Strain {
 //
 // Bound: the FP64 pipe (1.66 operations per SM and clock): 24 multiply-adds a component in the
 // gradient made 150 operations a voxel with the 36 of C eps, von Mises and the mean; with shared
-// faces they are 96 (200^3: 2.03 -> 1.49 ms, pipe 86% busy before and after).
+// faces they are 96 (200^3, the call: 2.03 -> 1.52 ms, pipe 86% busy before and after).
 __global__ void __launch_bounds__(kStressThreads, 2)
     k_stress(int nx, int ny, int nz, int tx, int ty, int zc, long long N, const int32_t* __restrict__ phase,
              const double* __restrict__ cfull, const __grid_constant__ Strain E, const double* __restrict__ w,
