@@ -421,7 +421,9 @@ int elas_tuning_export(char* buf, size_t cap, size_t* len);
 
 /* Records tilings given as text in the export format (e.g. saved by an earlier process).  A line
  * that does not describe a valid tiling of its grid fails the call with ELAS_ERR_INVALID_ARG and
- * nothing is recorded; message in elas_last_error(NULL). */
+ * nothing is recorded; message in elas_last_error(NULL).  FP32 lines with more than 256 columns,
+ * (tx + 1)(ty + 1), up to the 384 that earlier versions used, are recorded and exported but not used:
+ * such a grid takes the model's tiling until it is tuned again. */
 int elas_tuning_import(const char* text);
 
 /* ---- stress without allocation ----------------------------------------------------------- */
