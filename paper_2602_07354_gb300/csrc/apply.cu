@@ -1534,7 +1534,7 @@ Tiling make_tiling(const Geo& g, int elem_bytes, int sm_count, int tx_hint, int 
         const double per_sm_tiles = (double)rounds * std::min<long long>(R, (n_tiles + sm_count - 1) / sm_count);
         // (a thin tile's two layers run side by side; in more rounds than one it gives the product nothing
         // and costs the forms without it, the residuals and native FP64: 2 x 3 x 200 in two rounds of thin
-        // tiles took 24.6, 51 and 71.7 us, in one of two-layer tiles 20.5, 39 and 52)
+        // tiles took 24.6, 51 and 71.7 us, in one of two-layer tiles 22.7, 42 and 52.3)
         const bool side = thin_tiling(tx, ty, kc) && rounds == 1;
         double cost = per_sm_tiles * ((side ? 1 : kc + 1) + 0.5) * (threads + 64);
         if (n_tiles > (1LL << 30)) continue;
